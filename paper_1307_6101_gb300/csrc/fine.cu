@@ -1327,9 +1327,8 @@ __global__ void k_fine_export(cd* __restrict__ dst, const cplx<T>* __restrict__ 
 // allocate device memory.  The reduction partials live in a file-scope device
 // array instead of a cudaMalloc'ed scratch buffer; b and x are read in the ABI
 // layout directly, so no conversion buffer is needed either.  The residual at a
-// site is computed with the same device functions and the same order of
-// operations as k_fine_dslash, so it is bit-identical to the library's own
-// residual; only the order of the final sums differs.
+// site is computed by one thread with k_fine_dslash's device functions; it differs
+// from the library's own residual by the order of the sums only.
 constexpr int NOALLOC_MAX_RHS = 64;
 constexpr int NOALLOC_CHUNKS = 1024;
 __device__ __align__(256) double g_noalloc_partials[NOALLOC_MAX_RHS * NOALLOC_CHUNKS * 2];
@@ -1419,6 +1418,12 @@ void set_gamma_products(const double* gg /* [6][4][4][2] */) {
 template <typename T>
 void fine_dslash(cplx<T>* out, const cplx<T>* in, const cplx<T>* b, const FineOp<T>& op, int nrhs,
                  size_t rstride, int sel, int sel_mu, int in_chir, cudaStream_t st) {
+  if constexpr (sizeof(T) == 8) {
+    if (sel == SEL_FULL && in_chir < 0) {   // the Galerkin terms stay with the kernel below
+      fine_dslash_split(out, in, b, op, nrhs, rstride, st);
+      return;
+    }
+  }
   dim3 grid(div_up(op.g.V, 128), nrhs);
   count_launch();
   if constexpr (sizeof(T) == 4) {
@@ -1433,12 +1438,15 @@ void fine_dslash(cplx<T>* out, const cplx<T>* in, const cplx<T>* b, const FineOp
       return;
     }
   }
-  if (b)
-    k_fine_dslash<T, true, cplx<T>, T><<<grid, 128, 0, st>>>(out, in, b, op.U, op.clov, op.g, op.bc_t, rstride, sel,
-                                                             sel_mu, in_chir, T(0));
-  else
-    k_fine_dslash<T, false, cplx<T>, T><<<grid, 128, 0, st>>>(out, in, b, op.U, op.clov, op.g, op.bc_t, rstride,
-                                                              sel, sel_mu, in_chir, T(0));
+  if constexpr (sizeof(T) == 4) {
+    if (b) {
+      k_fine_dslash<T, true, cplx<T>, T><<<grid, 128, 0, st>>>(out, in, b, op.U, op.clov, op.g, op.bc_t, rstride, sel,
+                                                               sel_mu, in_chir, T(0));
+      return;
+    }
+  }
+  k_fine_dslash<T, false, cplx<T>, T><<<grid, 128, 0, st>>>(out, in, b, op.U, op.clov, op.g, op.bc_t, rstride,
+                                                            sel, sel_mu, in_chir, T(0));
 }
 
 // the staged kernel needs: FP32 compute, the SAP block tiling the aggregate
@@ -1555,41 +1563,42 @@ template <typename T>
 void fine_sap_sweep(cplx<T>* z, const cplx<T>* b, const FineOp<T>& op, const int* blocks, int nblocks, int nrhs,
                     size_t rstride, int k_mr, cudaStream_t st) {
   if (nrhs < 1 || nblocks < 1) return;   // the staged kernels issue their copies before the rhs loop
-  const bool tma = sap_tma_ok(op) && op.err;
-  if constexpr (sizeof(T) == 4) {
-    if (op.schur && op.err && sap_b4_ok(op, z, rstride)) {
+  if constexpr (sizeof(T) == 8) {
+    // Six threads per site, except where blocks of more than 64 sites (a cluster per block) are enough of
+    // them to fill the chip with one thread per site: 4^4 blocks, 128 per colour: 670 us per sweep with
+    // six threads and 540 with one, 16 per colour: 195 and 530.
+    if (op.g.vB <= 64 || nblocks < 96)
+      fine_sap_split(z, b, op, blocks, nblocks, nrhs, rstride, k_mr, st);   // a refused launch: the last error
+    else
+      launch_sap_plain<T, cplx<T>, T>(z, b, op.U, op.clov, op, blocks, nblocks, nrhs, rstride, k_mr, T(0), st);
+  } else {
+    const bool tma = sap_tma_ok(op) && op.err;
+    const bool b4 = op.err && sap_b4_ok(op, z, rstride);
+    if (op.schur && b4) {
       // block solves on the even-odd Schur complement (per-site clover / inverse tables)
       if (op.Uh)
         launch_sap_b4_eo<__half2, __half2>(z, b, op.Uh, op.mixh, op, blocks, nblocks, nrhs, rstride, k_mr, op.shift,
                                            st);
       else
         launch_sap_b4_eo<cplx<float>, float>(z, b, op.U, op.mix32, op, blocks, nblocks, nrhs, rstride, k_mr, 0.f, st);
-      return;
-    }
-    if (op.err && sap_b4_ok(op, z, rstride)) {
+    } else if (b4) {
       if (op.Uh)
         launch_sap_b4<__half2, __half2>(z, b, op.Uh, op.clovh, op, blocks, nblocks, nrhs, rstride, k_mr, op.shift, st);
       else
         launch_sap_b4<cplx<float>, float>(z, b, op.U, op.clov, op, blocks, nblocks, nrhs, rstride, k_mr, 0.f, st);
-      return;
-    }
-    if (op.Uh) {
+    } else if (op.Uh) {
       if (tma)
         launch_sap_tma<float, __half2, __half2>(z, b, op.Uh, op.clovh, op, blocks, nblocks, nrhs, rstride, k_mr,
                                                op.shift, st);
       else
         launch_sap_plain<float, __half2, __half2>(z, b, op.Uh, op.clovh, op, blocks, nblocks, nrhs, rstride, k_mr,
                                                  op.shift, st);
-      return;
-    }
-  }
-  if constexpr (sizeof(T) == 4) {   // the staged kernel is an FP32 kernel (sap_tma_ok)
-    if (tma) {
+    } else if (tma) {
       launch_sap_tma<T, cplx<T>, T>(z, b, op.U, op.clov, op, blocks, nblocks, nrhs, rstride, k_mr, T(0), st);
-      return;
+    } else {
+      launch_sap_plain<T, cplx<T>, T>(z, b, op.U, op.clov, op, blocks, nblocks, nrhs, rstride, k_mr, T(0), st);
     }
   }
-  launch_sap_plain<T, cplx<T>, T>(z, b, op.U, op.clov, op, blocks, nblocks, nrhs, rstride, k_mr, T(0), st);
 }
 
 __global__ void k_links_to_half(__half2* __restrict__ dst, const cplx<double>* __restrict__ U, size_t n) {

@@ -57,6 +57,12 @@ void fine_dslash(cplx<T>* out, const cplx<T>* in, const cplx<T>* b, const FineOp
 template <typename T>
 void fine_sap_sweep(cplx<T>* z, const cplx<T>* b, const FineOp<T>& op, const int* blocks, int nblocks, int nrhs,
                     size_t rstride, int k_mr, cudaStream_t st);
+// FP64 with six threads per site (fine_split.cu): the full operator (b set: b - D in), and one SAP
+// colour sweep
+void fine_dslash_split(cplx<double>* out, const cplx<double>* in, const cplx<double>* b, const FineOp<double>& op,
+                       int nrhs, size_t rstride, cudaStream_t st);
+cudaError_t fine_sap_split(cplx<double>* z, const cplx<double>* b, const FineOp<double>& op, const int* blocks,
+                           int nblocks, int nrhs, size_t rstride, int k_mr, cudaStream_t st);
 // ||b_i - D x_i|| / ||b_i|| with FP64 b, x in the ABI layout (device memory), no
 // allocation (static scratch); returns 0 or a negative code with *msg set
 int fine_residual_norm_noalloc(double* out, bool out_on_device, const cplx<double>* b, const cplx<double>* x,
