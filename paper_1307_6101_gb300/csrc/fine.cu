@@ -460,6 +460,204 @@ __global__ void k_fine_sap(cplx<T>* __restrict__ z, const cplx<T>* __restrict__ 
 }
 
 // ---------------------------------------------------------------------------
+// SAP colour sweep for 2^4 blocks (the default SAP block): half a warp per block, one thread per site,
+// no shared memory and no barrier.
+//
+// Every site of a 2^4 block has one hop per direction inside the block, to lane ^ (8 >> mu): forward
+// where its coordinate is even (l = 0), backward where it is odd.  Both directions run as one: the sender
+// projects for the receiver's direction (a sign), the half spinor goes through a shuffle (12 words
+// instead of a spinor's 24), and the receiver multiplies by the link of the pair (of its l = 0 site), which
+// every thread holds in registers for the whole sweep, already transposed and conjugated where its hop is
+// the backward one.  The hops leaving the block are the opposite ones (forward for l = 1) and are only
+// needed for rho = b - D z; z and those links come from global memory.  The clover term is read through L1
+// in every step (72 words against about 850 FMA-class instructions; the pointer is made opaque there, since
+// the compiler otherwise keeps it in registers and spills).
+// Bound: latency at 8 (FP32 storage, 255 registers) to 12 warps per SM, at a quarter to a third of the FP32
+// issue rate.  Small CTAs and a right-hand side each balance the SMs; looping over right-hand sides with
+// the links kept was slower (12 of them on 16^3x32: 375 us per sweep against 260).  ddamg_smooth, 10 sweeps of
+// 3 MR steps on 24x12x20x16 with 2 right-hand sides, FP32 storage: 500 us, where the staged kernel below took
+// 2268 (16 blocks and 172 KB of shared memory per CTA: 8 warps per SM, and 28 SMs with a second CTA to run).
+template <typename LS> struct PairLink;   // link of a pair in registers
+template <> struct PairLink<cplx<float>> {
+  cplx<float> e[9];
+  __device__ __forceinline__ void load(const cplx<float>* __restrict__ U, int V, int mu, int site, bool dag) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const cplx<float> v = U[(size_t)(mu * 9 + (dag ? b * 3 + a : a * 3 + b)) * V + site];
+        e[a * 3 + b] = cmk<float>(v.re, sign_flip(v.im, dag));
+      }
+  }
+  __device__ __forceinline__ cplx<float> at(int k) const { return e[k]; }
+};
+template <> struct PairLink<__half2> {
+  unsigned e[9];
+  __device__ __forceinline__ void load(const __half2* __restrict__ U, int V, int mu, int site, bool dag) {
+    const unsigned* u = reinterpret_cast<const unsigned*>(U);
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+      for (int b = 0; b < 3; ++b)   // conjugation: the sign bit of the high half (the imaginary part)
+        e[a * 3 + b] = u[(size_t)(mu * 9 + (dag ? b * 3 + a : a * 3 + b)) * V + site] ^ (dag ? 0x80000000u : 0u);
+  }
+  __device__ __forceinline__ cplx<float> at(int k) const {
+    unsigned w = e[k];
+    asm volatile("" : "+r"(w));   // widened where it is used: held widened, the links take 72 registers
+    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w));
+    return cmk<float>(f.x, f.y);
+  }
+};
+
+// h = projection (1 - sg gamma_mu) psi, upper two spins
+__device__ __forceinline__ void project_signed(int mu, float sg, const cplx<float> psi[12], cplx<float> h[6]) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const cplx<float> u0 = psi[a], u1 = psi[3 + a], d0 = psi[6 + a], d1 = psi[9 + a];
+    if (mu == 0) {
+      h[a] = cmk<float>(fmaf(-sg, d0.re, u0.re), fmaf(-sg, d0.im, u0.im));
+      h[3 + a] = cmk<float>(fmaf(-sg, d1.re, u1.re), fmaf(-sg, d1.im, u1.im));
+    } else if (mu == 1) {
+      h[a] = cmk<float>(fmaf(-sg, d0.im, u0.re), fmaf(sg, d0.re, u0.im));
+      h[3 + a] = cmk<float>(fmaf(sg, d1.im, u1.re), fmaf(-sg, d1.re, u1.im));
+    } else if (mu == 2) {
+      h[a] = cmk<float>(fmaf(sg, d1.re, u0.re), fmaf(sg, d1.im, u0.im));
+      h[3 + a] = cmk<float>(fmaf(-sg, d0.re, u1.re), fmaf(-sg, d0.im, u1.im));
+    } else {
+      h[a] = cmk<float>(fmaf(-sg, d1.im, u0.re), fmaf(sg, d1.re, u0.im));
+      h[3 + a] = cmk<float>(fmaf(-sg, d0.im, u1.re), fmaf(sg, d0.re, u1.im));
+    }
+  }
+}
+
+// acc += reconstruction of (1 - sg gamma_mu) from e h, e the link matrix of the hop
+template <typename LS>
+__device__ __forceinline__ void link_reconstruct(int mu, float sg, const PairLink<LS>& e, const cplx<float> h[6],
+                                                 cplx<float> acc[12]) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const cplx<float> e0 = e.at(3 * a), e1 = e.at(3 * a + 1), e2 = e.at(3 * a + 2);
+    cplx<float> g0 = e0 * h[0], g1 = e0 * h[3];
+    cfma(g0, e1, h[1]);
+    cfma(g1, e1, h[4]);
+    cfma(g0, e2, h[2]);
+    cfma(g1, e2, h[5]);
+    acc[a] = acc[a] + g0;
+    acc[3 + a] = acc[3 + a] + g1;
+    if (mu == 0) {
+      acc[6 + a] = cmk<float>(fmaf(-sg, g0.re, acc[6 + a].re), fmaf(-sg, g0.im, acc[6 + a].im));
+      acc[9 + a] = cmk<float>(fmaf(-sg, g1.re, acc[9 + a].re), fmaf(-sg, g1.im, acc[9 + a].im));
+    } else if (mu == 1) {
+      acc[6 + a] = cmk<float>(fmaf(sg, g0.im, acc[6 + a].re), fmaf(-sg, g0.re, acc[6 + a].im));
+      acc[9 + a] = cmk<float>(fmaf(-sg, g1.im, acc[9 + a].re), fmaf(sg, g1.re, acc[9 + a].im));
+    } else if (mu == 2) {
+      acc[6 + a] = cmk<float>(fmaf(-sg, g1.re, acc[6 + a].re), fmaf(-sg, g1.im, acc[6 + a].im));
+      acc[9 + a] = cmk<float>(fmaf(sg, g0.re, acc[9 + a].re), fmaf(sg, g0.im, acc[9 + a].im));
+    } else {
+      acc[6 + a] = cmk<float>(fmaf(sg, g1.im, acc[6 + a].re), fmaf(-sg, g1.re, acc[6 + a].im));
+      acc[9 + a] = cmk<float>(fmaf(sg, g0.im, acc[9 + a].re), fmaf(-sg, g0.re, acc[9 + a].im));
+    }
+  }
+}
+
+constexpr int B2T = 64;   // threads: 4 blocks
+
+template <typename LS, typename CS>
+__global__ void __launch_bounds__(B2T, sizeof(LS) == 4 ? 6 : 4) k_fine_sap_b2(cplx<float>* __restrict__ z,
+                                                        const cplx<float>* __restrict__ bsrc,
+                                                        const LS* __restrict__ U, const CS* __restrict__ clov, Geom g,
+                                                        int bc_t, size_t rstride, const int* __restrict__ blocks,
+                                                        int nblocks, int k_mr, float shift) {
+  using C = cplx<float>;
+  pdl_launch_dependents();
+  const int hw = (blockIdx.x * B2T + threadIdx.x) >> 4;
+  const bool active = hw < nblocks;   // the last CTA's spare half-warps repeat a block and write nothing
+  const int loc = threadIdx.x & 15;
+  const int V = g.V;
+  const int x = blocks[active ? hw : nblocks - 1] * 16 + loc;
+  PairLink<LS> in[4];
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) {
+    const bool odd = (loc >> (3 - mu)) & 1;
+    in[mu].load(U, V, mu, odd ? x - (8 >> mu) : x, odd);
+  }
+  int c[4];
+  geom_coords(g, x, c);
+  pdl_wait();   // links and clover term are never written by the kernels this launch may overlap; z is
+  C* pz = z + (size_t)blockIdx.y * rstride;
+  C r[12], xs[12], acc[12], h[6];
+  // sum of the four hops inside the block on the field v, one shuffle of a half spinor each
+  auto inside = [&](const C v[12]) {
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+      const float sg = ((loc >> (3 - mu)) & 1) ? 1.f : -1.f;   // the partner's direction; the own one is -sg
+      project_signed(mu, sg, v, h);
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        h[k].re = __shfl_xor_sync(0xffffffffu, h[k].re, 8 >> mu);
+        h[k].im = __shfl_xor_sync(0xffffffffu, h[k].im, 8 >> mu);
+      }
+      link_reconstruct(mu, -sg, in[mu], h, acc);
+    }
+  };
+  // rho = b - D z
+#pragma unroll
+  for (int k = 0; k < 12; ++k) acc[k] = czero<float>();
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) {
+    const bool odd = (loc >> (3 - mu)) & 1;   // the hop leaving the block: forward where odd
+    const int n = geom_neighbor(g, c, mu, odd ? +1 : -1);
+    const bool neg = mu == 0 && bc_t < 0 && c[0] == (odd ? g.L[0] - 1 : 0);
+    PairLink<LS> e;
+    e.load(U, V, mu, odd ? x : n, !odd);
+    load_spinor(pz, V, n, r, neg ? -1.f : 1.f, -1);
+    project_signed(mu, odd ? 1.f : -1.f, r, h);
+    link_reconstruct(mu, odd ? 1.f : -1.f, e, h, acc);
+  }
+  load_spinor(pz, V, x, r, 1.f, -1);
+  inside(r);
+  clover_apply(clov, V, x, r, xs, shift);
+  const C* pb = bsrc + (size_t)blockIdx.y * rstride;
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    r[k] = pb[(size_t)k * V + x] - (xs[k] - 0.5f * acc[k]);
+    xs[k] = czero<float>();
+  }
+#pragma unroll 1
+  for (int it = 0; it < k_mr; ++it) {
+#pragma unroll
+    for (int k = 0; k < 12; ++k) acc[k] = czero<float>();
+    inside(r);
+    C p[12];
+    asm volatile("" : "+l"(clov));   // not hoisted: see above
+    clover_apply(clov, V, x, r, p, shift);
+    float nre = 0.f, nim = 0.f, den = 0.f;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      p[k] = p[k] - 0.5f * acc[k];
+      cdotc_acc(nre, nim, p[k], r[k]);
+      cnorm2_acc(den, p[k]);
+    }
+#pragma unroll
+    for (int off = 8; off >= 1; off >>= 1) {
+      nre += __shfl_xor_sync(0xffffffffu, nre, off);
+      nim += __shfl_xor_sync(0xffffffffu, nim, off);
+      den += __shfl_xor_sync(0xffffffffu, den, off);
+    }
+    const C alpha = den > 0.f ? cmk<float>(nre / den, nim / den) : czero<float>();
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      cfma(xs[k], alpha, r[k]);
+      r[k] = r[k] - alpha * p[k];
+    }
+  }
+  if (active) {
+#pragma unroll
+    for (int k = 0; k < 12; ++k) pz[(size_t)k * V + x] = pz[(size_t)k * V + x] + xs[k];
+  }
+}
+
+// ---------------------------------------------------------------------------
 // SAP colour sweep with the SAP block staged in shared memory by TMA.
 //
 // One CTA per SAP block (or several small blocks).  A single thread arms an
@@ -1482,6 +1680,36 @@ void launch_sap_tma(cplx<T>* z, const cplx<T>* b, const LS* U, const CS* clov, c
                                                                        blocks, nblocks, seg, k_mr, op.err, shift);
 }
 
+// the 2^4 kernel: 2^4 SAP blocks that are the inner tile (16 consecutive sites), none spanning a lattice
+// direction (there both hops of a site would stay inside)
+template <typename T>
+bool sap_b2_ok(const FineOp<T>& op) {
+  for (int d = 0; d < 4; ++d)
+    if (op.g.B[d] != 2 || op.g.I[d] != 2 || op.g.L[d] == 2) return false;
+  return true;
+}
+
+template <typename LS, typename CS>
+void launch_sap_b2(cplx<float>* z, const cplx<float>* b, const LS* U, const CS* clov, const FineOp<float>& op,
+                   const int* blocks, int nblocks, int nrhs, size_t rstride, int k_mr, float shift, cudaStream_t st) {
+  count_launch();
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute pdl[1];
+  pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  pdl[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3(div_up(nblocks, B2T / 16), nrhs, 1);
+  cfg.blockDim = dim3(B2T, 1, 1);
+  cfg.stream = st;
+  cfg.attrs = pdl;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, k_fine_sap_b2<LS, CS>, z, b, U, clov, op.g, op.bc_t, rstride, blocks, nblocks, k_mr,
+                         shift) != cudaSuccess) {
+    cudaGetLastError();   // the attribute refused here: the same sweep as a plain launch
+    k_fine_sap_b2<LS, CS><<<cfg.gridDim, B2T, 0, st>>>(z, b, U, clov, op.g, op.bc_t, rstride, blocks, nblocks, k_mr,
+                                                        shift);
+  }
+}
+
 // the 4^4 kernel: FP32 compute, 4^4 SAP blocks that are the inner tile (contiguous
 // sites), and 16-byte aligned rows of z (bulk copies)
 template <typename T>
@@ -1586,6 +1814,11 @@ void fine_sap_sweep(cplx<T>* z, const cplx<T>* b, const FineOp<T>& op, const int
         launch_sap_b4<__half2, __half2>(z, b, op.Uh, op.clovh, op, blocks, nblocks, nrhs, rstride, k_mr, op.shift, st);
       else
         launch_sap_b4<cplx<float>, float>(z, b, op.U, op.clov, op, blocks, nblocks, nrhs, rstride, k_mr, 0.f, st);
+    } else if (sap_b2_ok(op)) {
+      if (op.Uh)
+        launch_sap_b2<__half2, __half2>(z, b, op.Uh, op.clovh, op, blocks, nblocks, nrhs, rstride, k_mr, op.shift, st);
+      else
+        launch_sap_b2<cplx<float>, float>(z, b, op.U, op.clov, op, blocks, nblocks, nrhs, rstride, k_mr, 0.f, st);
     } else if (op.Uh) {
       if (tma)
         launch_sap_tma<float, __half2, __half2>(z, b, op.Uh, op.clovh, op, blocks, nblocks, nrhs, rstride, k_mr,
