@@ -68,6 +68,8 @@ __global__ void k_coarse_apply(cplx<T>* __restrict__ out, const cplx<T>* __restr
     take[k] = tk;
   }
   __syncthreads();
+  // the term of a hop that leaves the aggregate: sites without it are not written (nor read by the product with P^+)
+  if ((sel == SEL_AGG_FWD && !take[1 + sel_mu]) || (sel == SEL_AGG_BWD && !take[5 + sel_mu])) return;
   const int h = n / 2;
   for (int e = threadIdx.x; e < 9 * n; e += blockDim.x) {
     const int k = e / n, j = e % n;
@@ -965,29 +967,31 @@ __global__ void k_blocks_export(cplx<double>* __restrict__ dst, const cplx<doubl
   dst[lex * per + (size_t)k * n * n + (size_t)i * n + j] = blk[bidx(site, k, n, i, j)];
 }
 
-// FP16 copy of one site's 9 blocks: s = float(max |re|, |im|), q = RNE_half(x / s)
+// FP16 copy of one site's 9 blocks: s = float(max |re|, |im|), q = RNE_half(x / s) with x / s as the product
+// with the reciprocal (as in the copy of P: FP64 divisions and comparisons would bound the kernel)
 __global__ void k_blocks_to_half(__half2* __restrict__ dst, float* __restrict__ scale,
                                  const cplx<double>* __restrict__ blk, int n) {
-  __shared__ double sh[32];
-  const size_t per = (size_t)9 * n * n;
+  __shared__ unsigned long long sh[32];
+  __shared__ double rs;
+  const int per = 9 * n * n;
   const cplx<double>* src = blk + (size_t)blockIdx.x * per;
-  double mx = 0.0;
-  for (size_t e = threadIdx.x; e < per; e += blockDim.x) mx = fmax(mx, fmax(fabs(src[e].re), fabs(src[e].im)));
-  for (int off = 16; off >= 1; off >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+  unsigned long long mx = 0ull;
+  for (int e = threadIdx.x; e < per; e += blockDim.x) mx = max(mx, max(abs_bits(src[e].re), abs_bits(src[e].im)));
+  for (int off = 16; off >= 1; off >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = mx;
   __syncthreads();
   if (threadIdx.x == 0) {
-    double m = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = fmax(m, sh[w]);
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) mx = max(mx, sh[w]);
+    const double m = __longlong_as_double((long long)mx);
     const float sf = m > 0.0 ? (float)m : 1.0f;
     scale[blockIdx.x] = sf;
-    sh[0] = (double)sf;
+    rs = 1.0 / (double)sf;
   }
   __syncthreads();
-  const double sc = sh[0];
+  const double r = rs;
   __half2* d = dst + (size_t)blockIdx.x * per;
-  for (size_t e = threadIdx.x; e < per; e += blockDim.x)
-    d[e] = __halves2half2(__double2half(src[e].re / sc), __double2half(src[e].im / sc));
+  for (int e = threadIdx.x; e < per; e += blockDim.x)
+    d[e] = __halves2half2(__double2half(src[e].re * r), __double2half(src[e].im * r));
 }
 
 }  // namespace

@@ -88,6 +88,11 @@ __device__ __forceinline__ cplx<float> ld_cplx(const __half2* p, size_t i) {
   return cmk<float>(f.x, f.y);
 }
 
+// |x| as bits: ordered like |x| (NaN above all)
+__device__ __forceinline__ unsigned long long abs_bits(double x) {
+  return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffULL;
+}
+
 // ---------------------------------------------------------------------------
 // Geometry of one level: lattice extents L, aggregate extents A and SAP block
 // extents B, one of which tiles the other.  The larger is the outer tile O, the

@@ -175,9 +175,11 @@ __device__ __forceinline__ void load_spinor(const cplx<T>* __restrict__ p, int V
   const bool neg = sign < T(0);
 #pragma unroll
   for (int k = 0; k < 12; ++k) {
-    const bool keep = chir < 0 || (k / 6) == chir;
-    const cplx<T> v = p[(size_t)k * V + x];
-    s[k] = keep ? cmk<T>(sign_flip(v.re, neg), sign_flip(v.im, neg)) : czero<T>();
+    s[k] = czero<T>();
+    if (chir < 0 || (k / 6) == chir) {
+      const cplx<T> v = p[(size_t)k * V + x];
+      s[k] = cmk<T>(sign_flip(v.re, neg), sign_flip(v.im, neg));
+    }
   }
 }
 
@@ -194,6 +196,9 @@ __global__ void k_fine_dslash(cplx<T>* __restrict__ out, const cplx<T>* __restri
   const int V = g.V;
   int c[4];
   geom_coords(g, x, c);
+  // the term of a hop that leaves the aggregate: sites without it are not written (nor read by the product with P^+)
+  if (sel == SEL_AGG_FWD && hop_internal(g, c, sel_mu, +1, g.A)) return;
+  if (sel == SEL_AGG_BWD && hop_internal(g, c, sel_mu, -1, g.A)) return;
   cplx<T> acc[12];
 #pragma unroll
   for (int k = 0; k < 12; ++k) acc[k] = czero<T>();

@@ -178,6 +178,15 @@ template <typename T>
 void restrict_op(cplx<T>* out, const cplx<T>* in, const cplx<T>* P, const Geom& gf, const Geom& gc, bool fine,
                  int n, int N, int nrhs, size_t in_rstride, size_t out_rstride, size_t out_site_stride,
                  cudaStream_t st, const __half2* Ph = nullptr, const float* pscale = nullptr, int tc_ks = 0);
+// the same for C <= galerkin_cols() columns of a Galerkin term (TermSel sel, direction sel_mu): only the
+// sites that the term reaches are read
+int galerkin_cols();
+template <typename T>
+bool galerkin_fits(int N, int C, int vA);
+template <typename T>
+cudaError_t galerkin_restrict(cplx<T>* out, const cplx<T>* tmp, const cplx<T>* P, const Geom& gf, const Geom& gc,
+                              bool fine, int n, int N, int C, size_t tmp_rstride, size_t out_rstride,
+                              size_t out_site_stride, int sel, int sel_mu, cudaStream_t st);
 // out(x, f) = [out +] sum_j P_j(x, f) in(A(x))[s(f)*N + j]
 // batch != 0 (FP32 compute on FP16 P only): one CTA per aggregate for the whole batch (P read once)
 template <typename T>

@@ -1226,6 +1226,36 @@ struct SetupTimer {
   }
 };
 
+// blk = the blocks of P_l^+ D_l P_l; term(t, p, jb, sel, mu, sp) = term (sel, mu) of D_l on the chirality-sp part
+// of jb fields p
+template <typename T, class Term>
+void galerkin(ddamg_handle* h, int l, const cplx<T>* P, cplx<T>* blk, Term term) {
+  Level& F = h->lv[l];
+  Level& C = h->lv[l + 1];
+  const int nc = C.n;
+  const int jb_max = std::min(F.N, sizeof(T) == 4 ? galerkin_cols() : SETUP_CHUNK);
+  cplx<T>* tmp = static_cast<cplx<T>*>(scratch(h, 4, sizeof(cplx<T>) * F.vlen * jb_max));
+  for (int sp = 0; sp < 2; ++sp)
+    for (int k = 0; k < 9; ++k) {
+      const int sel = k == 0 ? SEL_AGG_SELF : (k <= 4 ? SEL_AGG_FWD : SEL_AGG_BWD);
+      const int mu = k == 0 ? 0 : (k - 1) % 4;
+      for (int j0 = 0; j0 < F.N; j0 += jb_max) {
+        const int jb = std::min(jb_max, F.N - j0);
+        cplx<T>* out = blk + (size_t)k * nc * nc + (size_t)(sp * F.N + j0) * nc;
+        if (!galerkin_fits<T>(F.N, jb, F.g.vA)) {   // an aggregate of tens of thousands of sites
+          blas_zero<T>(tmp, F.vlen, jb, F.vlen, h->st);
+          term(tmp, P + (size_t)j0 * F.vlen, jb, sel, mu, sp);
+          restrict_op<T>(out, tmp, P, F.g, C.g, F.fine, F.n, F.N, jb, F.vlen, (size_t)nc, (size_t)9 * nc * nc, h->st);
+          continue;
+        }
+        term(tmp, P + (size_t)j0 * F.vlen, jb, sel, mu, sp);
+        if (galerkin_restrict<T>(out, tmp, P, F.g, C.g, F.fine, F.n, F.N, jb, F.vlen, (size_t)nc, (size_t)9 * nc * nc,
+                                 sel, mu, h->st) != cudaSuccess)
+          fail(DDAMG_ERR_CUDA, "launch of the Galerkin product failed");
+      }
+    }
+}
+
 void rebuild(ddamg_handle* h, int l) {
   SetupTimer tm{h, l, DDAMG_SETUP_REBUILD};
   Level& F = h->lv[l];
@@ -1237,53 +1267,32 @@ void rebuild(ddamg_handle* h, int l) {
   check_err_flag(h, "test vectors are linearly dependent on an aggregate");
   blas_convert<float, double>(F.P32, F.P64, tot, 1, 0, 0, st);
   // Galerkin: column (s', j) of every block = P^+ (term of D applied to P_j restricted to chirality s'),
-  // in chunks of SETUP_CHUNK columns (bounded scratch).  A handle with the FP32 preconditioner forms
-  // the product in FP32 from the FP32 copies of the operator and P (the preconditioner's setup runs
-  // in single precision, Sec. 3); an FP64 handle in FP64.
-  const int jb_max = F.N < SETUP_CHUNK ? F.N : SETUP_CHUNK;
-  const int nc = C.n;
-  const size_t nb = (size_t)C.g.V * 9 * nc * nc;
+  // in chunks of columns (bounded scratch: eight FP32 or four FP64 fields).  A handle with the FP32
+  // preconditioner forms the product in FP32 from the FP32 copies of the operator and P (the preconditioner's
+  // setup runs in single precision, Sec. 3); an FP64 handle in FP64.
+  const size_t nb = (size_t)C.g.V * 9 * C.n * C.n;
   if (h->p.precision != 0) {
-    cplx<float>* tmp = static_cast<cplx<float>*>(scratch(h, 4, sizeof(cplx<float>) * F.vlen * jb_max));
     FineOp<float> fo = F.f32;   // FP32 storage, not the FP16 copies
     fo.Uh = nullptr;
     fo.clovh = nullptr;
     CoarseOp<float> co = F.c32;
     co.blkh = nullptr;
     co.bscale = nullptr;
-    for (int sp = 0; sp < 2; ++sp)
-      for (int k = 0; k < 9; ++k) {
-        const int sel = k == 0 ? SEL_AGG_SELF : (k <= 4 ? SEL_AGG_FWD : SEL_AGG_BWD);
-        const int mu = k == 0 ? 0 : (k - 1) % 4;
-        for (int j0 = 0; j0 < F.N; j0 += jb_max) {
-          const int jb = F.N - j0 < jb_max ? F.N - j0 : jb_max;
-          const cplx<float>* pj = F.P32 + (size_t)j0 * F.vlen;
-          if (F.fine) fine_dslash<float>(tmp, pj, nullptr, fo, jb, F.vlen, sel, mu, sp, st);
-          else coarse_apply<float>(tmp, pj, nullptr, co, jb, F.vlen, sel, mu, sp, st);
-          restrict_op<float>(C.c32.blk + (size_t)k * nc * nc + (size_t)(sp * F.N + j0) * nc, tmp, F.P32, F.g, C.g,
-                             F.fine, F.n, F.N, jb, F.vlen, (size_t)nc, (size_t)9 * nc * nc, st);
-        }
-      }
+    galerkin<float>(h, l, F.P32, C.c32.blk, [&](cplx<float>* t, const cplx<float>* p, int jb, int sel, int mu, int sp) {
+      if (F.fine) fine_dslash<float>(t, p, nullptr, fo, jb, F.vlen, sel, mu, sp, st);
+      else coarse_apply<float>(t, p, nullptr, co, jb, F.vlen, sel, mu, sp, st);
+    });
     blas_convert<double, float>(C.c64.blk, C.c32.blk, nb, 1, 0, 0, st);
   } else {
-    cplx<double>* tmp = static_cast<cplx<double>*>(scratch(h, 4, sizeof(cplx<double>) * F.vlen * jb_max));
-    for (int sp = 0; sp < 2; ++sp)
-      for (int k = 0; k < 9; ++k) {
-        const int sel = k == 0 ? SEL_AGG_SELF : (k <= 4 ? SEL_AGG_FWD : SEL_AGG_BWD);
-        const int mu = k == 0 ? 0 : (k - 1) % 4;
-        for (int j0 = 0; j0 < F.N; j0 += jb_max) {
-          const int jb = F.N - j0 < jb_max ? F.N - j0 : jb_max;
-          apply_D<double>(h, F, tmp, F.P64 + (size_t)j0 * F.vlen, nullptr, jb, sel, mu, sp);
-          restrict_op<double>(C.c64.blk + (size_t)k * nc * nc + (size_t)(sp * F.N + j0) * nc, tmp, F.P64, F.g, C.g,
-                              F.fine, F.n, F.N, jb, F.vlen, (size_t)nc, (size_t)9 * nc * nc, st);
-        }
-      }
+    galerkin<double>(h, l, F.P64, C.c64.blk, [&](cplx<double>* t, const cplx<double>* p, int jb, int sel, int mu, int sp) {
+      apply_D<double>(h, F, t, p, nullptr, jb, sel, mu, sp);
+    });
     blas_convert<float, double>(C.c32.blk, C.c64.blk, nb, 1, 0, 0, st);
   }
   if (C.coarsest && C.eo) {
-    coarse_selfinv_build(C.c64.selfinv, C.c64.blk, C.g.V, nc, h->d_err, st);
+    coarse_selfinv_build(C.c64.selfinv, C.c64.blk, C.g.V, C.n, h->d_err, st);
     check_err_flag(h, "singular self block on the coarsest level");
-    blas_convert<float, double>(C.c32.selfinv, C.c64.selfinv, (size_t)C.g.V * nc * nc, 1, 0, 0, st);
+    blas_convert<float, double>(C.c32.selfinv, C.c64.selfinv, (size_t)C.g.V * C.n * C.n, 1, 0, 0, st);
   }
   if (F.Ph) half_refresh(h, l);
   sync(h);

@@ -8,6 +8,8 @@
 #include "common.cuh"
 #include "kernels.h"
 
+#include <mutex>
+
 namespace {
 
 // address of (site x, component f) in a level field: fine [12][V], coarse [V][n]
@@ -141,98 +143,302 @@ __global__ void k_prolong(cplx<T>* __restrict__ out, const cplx<T>* __restrict__
   *po = accumulate ? *po + acc : acc;
 }
 
-// CGS2 of the N test vectors restricted to (aggregate, chirality), in column order.
-__global__ void k_orthonormalise(cplx<double>* __restrict__ P, Geom g, bool fine, int n, int N, size_t pstride,
-                                 int* err) {
-  __shared__ double sh[32 * 2 * 8];
+// Galerkin products: columns of P^+ (term of D P), for C <= 8 columns of one launch.
+//   out[c][site of A][s*N + i] = sum over x in A, f in s of conj(P_i(x, f)) tmp_c(x, f)
+// A term of a hop that leaves the aggregate is nonzero on one face of it only, and only those sites are read
+// (tmp is not even written elsewhere): of 4^4 aggregates a quarter, for eight of the nine terms.
+// One CTA per (aggregate, chirality): the N x K by K x C product with K staged in chunks, each lane a 4 x 4
+// tile of the result (64 FMAs for 8 shared-memory loads), the lanes that N x C does not need and the warps
+// splitting K (summed at the end in a fixed order).
+// Replaces k_restrict with one right-hand side per CTA, which read all of P again for each: the nine terms and
+// 40 columns of 16^3x32 with 20 test vectors took 24.3 ms there and take 4.9 ms here, and the second level's
+// (4^3x8 sites, 28 test vectors) 4.2 and 0.85 ms.
+constexpr int GT = 256;    // threads
+constexpr int GKC = 64;    // K rows per staged chunk
+constexpr int GCMAX = 8;   // columns per launch
+
+constexpr int GFLUSH = 4;  // chunks whose products run into one accumulator
+
+struct GalerkinSmem {
+  size_t red, list, total;
+};
+DD_HD GalerkinSmem galerkin_smem(int N, int C, int vA, size_t cs) {
+  GalerkinSmem L;
+  const int tiles = ((N + 3) / 4) * ((C + 3) / 4);
+  L.red = (((size_t)GKC * ((N | 1) + (C | 1)) * cs) + 15) & ~size_t(15);
+  L.list = L.red + (size_t)(GT / 32) * (32 / tiles) * tiles * 16 * cs;
+  L.total = L.list + (size_t)vA * sizeof(int);
+  return L;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(GT) k_galerkin(cplx<T>* __restrict__ out, const cplx<T>* __restrict__ tmp,
+                                                 const cplx<T>* __restrict__ P, Geom gf, Geom gc, bool fine, int n,
+                                                 int N, int C, size_t tmp_rstride, size_t pstride, size_t out_rstride,
+                                                 size_t out_site_stride, int sel, int sel_mu) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int wcount[GT / 32];
+  __shared__ int nsites;
+  const int agg = blockIdx.x, s = blockIdx.y;
+  const int V = gf.V, vA = gf.vA, h = n / 2;
+  const int NP = N | 1, CP = C | 1;
+  cplx<T>* sA = reinterpret_cast<cplx<T>*>(smem_raw);   // [GKC][NP]
+  cplx<T>* sB = sA + (size_t)GKC * NP;                  // [GKC][CP]
+  const GalerkinSmem L = galerkin_smem(N, C, vA, sizeof(cplx<T>));
+  cplx<T>* red = reinterpret_cast<cplx<T>*>(smem_raw + L.red);   // [warp][sub][tile][16] partial tiles
+  int* list = reinterpret_cast<int*>(smem_raw + L.list);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // the sites of the aggregate that the term reaches, in site order
+  if (tid == 0) nsites = 0;
+  for (int x0 = 0; x0 < vA; x0 += GT) {
+    bool take = x0 + tid < vA;
+    if (take && sel != SEL_AGG_SELF) {
+      int c[4];
+      geom_coords(gf, agg * vA + x0 + tid, c);
+      take = !hop_internal(gf, c, sel_mu, sel == SEL_AGG_FWD ? +1 : -1, gf.A);
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, take);
+    if (lane == 0) wcount[warp] = __popc(m);
+    __syncthreads();
+    int at = nsites;
+    for (int w = 0; w < warp; ++w) at += wcount[w];
+    if (take) list[at + __popc(m & ((1u << lane) - 1))] = x0 + tid;
+    __syncthreads();
+    if (tid == 0)
+      for (int w = 0; w < GT / 32; ++w) nsites += wcount[w];
+    __syncthreads();
+  }
+  const int nS = nsites, K = nS * h;
+  const int TI = (N + 3) / 4, TC = (C + 3) / 4, tiles = TI * TC, nsub = 32 / tiles;
+  const int sub = lane / tiles, tile = lane - sub * tiles;
+  const int i0 = 4 * (tile % TI), c0 = 4 * (tile / TI);
+  cplx<T> acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[i][c] = czero<T>();
+  // row tid % GKC of a chunk, columns tid / GKC + 4 q of [P | tmp], the next chunk on its way during the product
+  constexpr int NL = (32 + GCMAX + GT / GKC - 1) / (GT / GKC);
+  const int kr = tid % GKC, j0 = tid / GKC;
+  cplx<T> v[NL];
+  auto fetch = [&](int k0) {
+    const int kk = k0 + kr;
+    if (kk < K) {
+      // component-major on the fine level (neighbouring rows: neighbouring sites), dof-contiguous on a coarse one
+      const int q = fine ? kk / nS : kk / h, r = kk - q * (fine ? nS : h);
+      const size_t a = faddr(fine, V, n, agg * vA + list[fine ? r : q], s * h + (fine ? q : r));
+#pragma unroll
+      for (int e = 0; e < NL; ++e) {
+        const int j = j0 + e * (GT / GKC);
+        if (j < N) v[e] = P[(size_t)j * pstride + a];
+        else if (j < N + C) v[e] = tmp[(size_t)(j - N) * tmp_rstride + a];
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < NL; ++e) v[e] = czero<T>();
+    }
+  };
+  cplx<T>* mine = red + (((size_t)warp * nsub + sub) * tiles + tile) * 16;
+  fetch(0);
+  int chunk = 0;
+  for (int k0 = 0; k0 < K; k0 += GKC, ++chunk) {
+#pragma unroll
+    for (int e = 0; e < NL; ++e) {
+      const int j = j0 + e * (GT / GKC);
+      if (j < N) sA[kr * NP + j] = v[e];
+      else if (j < N + C) sB[kr * CP + j - N] = v[e];
+    }
+    __syncthreads();
+    if (k0 + GKC < K) fetch(k0 + GKC);
+    const int kc = min(GKC, K - k0);
+    if (sub < nsub) {
+      for (int k = warp * nsub + sub; k < kc; k += (GT / 32) * nsub) {
+        cplx<T> a[4], b[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) a[i] = i0 + i < N ? sA[k * NP + i0 + i] : czero<T>();
+#pragma unroll
+        for (int c = 0; c < 4; ++c) b[c] = c0 + c < C ? sB[k * CP + c0 + c] : czero<T>();
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) cfmac(acc[i][c], a[i], b[c]);
+      }
+      // long sums in parts: their rounding errors do not add up along the whole of K
+      if (chunk % GFLUSH == GFLUSH - 1 || k0 + GKC >= K) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            mine[4 * i + c] = chunk < GFLUSH ? acc[i][c] : mine[4 * i + c] + acc[i][c];
+            acc[i][c] = czero<T>();
+          }
+      }
+    }
+    __syncthreads();
+  }
+  int ca[4];
+  geom_coords(gf, agg * vA, ca);
+  cplx<T>* po = out + (size_t)coarse_site_of(gf, gc, ca) * out_site_stride + (size_t)s * N;
+  for (int e = tid; e < N * C; e += GT) {
+    const int c = e / N, i = e - c * N;
+    const cplx<T>* r = red + ((size_t)(c / 4) * TI + i / 4) * 16 + 4 * (i % 4) + c % 4;
+    cplx<T> t[4] = {czero<T>(), czero<T>(), czero<T>(), czero<T>()};   // the parts in four chains
+    for (int q = 0; K > 0 && q < (GT / 32) * nsub; q += 4)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) t[u] = t[u] + r[(size_t)(q + u) * tiles * 16];
+    po[(size_t)c * out_rstride + i] = (t[0] + t[1]) + (t[2] + t[3]);
+  }
+}
+
+// CGS2 of the N test vectors restricted to (aggregate, chirality), in column order.  One CTA per
+// (aggregate, chirality); the column in work stays in shared memory (SW) while it is orthogonalised, the earlier
+// ones are read from L2 or HBM, and both run through the elements as memory holds them.
+// Bound by the FP64 rate: 16 FMAs per element and pair of columns, 4.8 G of them for 20 columns on 16^3x32,
+// 9.1 ms, measured 11.4 (21.8 before).  Eight dot products are reduced together by lanes that share the values out as they fold (16 additions
+// per lane instead of 80, and the warps' sums are added by one warp instead of all).
+constexpr int OT = 128;   // threads
+
+// sum 16 values per thread over the warp: lane l returns value l / 2
+__device__ __forceinline__ double warp_fold16(double* v, int lane) {
+#pragma unroll
+  for (int w = 8, off = 16; w >= 1; w >>= 1, off >>= 1) {
+    const bool up = (lane & off) != 0;
+#pragma unroll
+    for (int k = 0; k < w; ++k) {
+      const double keep = up ? v[k + w] : v[k], send = up ? v[k] : v[k + w];
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+    }
+  }
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+template <bool SW>
+__global__ void __launch_bounds__(OT) k_orthonormalise(cplx<double>* __restrict__ P, Geom g, bool fine, int n, int N,
+                                                       size_t pstride, int* err) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ double sh[OT / 32][16];
   __shared__ cplx<double> hs[64];
+  __shared__ double tot;
+  cplx<double>* sw = reinterpret_cast<cplx<double>*>(smem_raw);   // [ne] the column in work
   const int agg = blockIdx.x;
   const int s = blockIdx.y;
   const int h = n / 2;
   const int ne = g.vA * h;
-  const int V = g.V;
-  auto addr = [&](int e) {
-    const int x = agg * g.vA + e / h;
-    const int f = s * h + e % h;
-    return faddr(fine, V, n, x, f);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // element e of the block: fine fields by component, then site; coarse fields by site, then dof
+  auto addr = [&](int e) -> size_t {
+    if (fine) {
+      const int f = e / g.vA;
+      return (size_t)(s * h + f) * g.V + (size_t)agg * g.vA + (e - f * g.vA);
+    }
+    const int x = e / h;
+    return (size_t)(agg * g.vA + x) * n + s * h + (e - x * h);
+  };
+  auto cta_norm2 = [&](const cplx<double>* w) {
+    double a = 0.0;
+    for (int e = threadIdx.x; e < ne; e += OT) cnorm2_acc(a, SW ? sw[e] : w[addr(e)]);
+    for (int off = 16; off >= 1; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
+    __syncthreads();
+    if (lane == 0) sh[warp][0] = a;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double t = 0.0;
+      for (int w2 = 0; w2 < OT / 32; ++w2) t += sh[w2][0];
+      tot = t;
+    }
+    __syncthreads();
+    return tot;
   };
   for (int j = 0; j < N; ++j) {
     cplx<double>* w = P + (size_t)j * pstride;
-    double n0 = 0.0;
-    for (int e = threadIdx.x; e < ne; e += blockDim.x) n0 += cnorm2(w[addr(e)]);
-    block_sum(&n0, 1, sh);
-    for (int pass = 0; pass < 2; ++pass) {
+    if (SW)
+      for (int e = threadIdx.x; e < ne; e += OT) sw[e] = w[addr(e)];   // read back by the same thread
+    const double n0 = cta_norm2(w);
+    for (int pass = 0; pass < 2 && j > 0; ++pass) {
       for (int i0 = 0; i0 < j; i0 += 8) {
         double acc[16];
+#pragma unroll
         for (int k = 0; k < 16; ++k) acc[k] = 0.0;
-        for (int e = threadIdx.x; e < ne; e += blockDim.x) {
+        for (int e = threadIdx.x; e < ne; e += OT) {
           const size_t a = addr(e);
-          const cplx<double> we = w[a];
-          for (int ii = 0; ii < 8 && i0 + ii < j; ++ii) {
-            const cplx<double> t = cdotc(P[(size_t)(i0 + ii) * pstride + a], we);
-            acc[2 * ii] += t.re;
-            acc[2 * ii + 1] += t.im;
-          }
+          const cplx<double> we = SW ? sw[e] : w[a];
+#pragma unroll
+          for (int ii = 0; ii < 8; ++ii)
+            if (i0 + ii < j) cdotc_acc(acc[2 * ii], acc[2 * ii + 1], P[(size_t)(i0 + ii) * pstride + a], we);
         }
-        block_sum(acc, 16, sh);
-        if (threadIdx.x < 8 && i0 + threadIdx.x < j) hs[i0 + threadIdx.x] = cmk(acc[2 * threadIdx.x], acc[2 * threadIdx.x + 1]);
+        const double v = warp_fold16(acc, lane);
+        if ((lane & 1) == 0) sh[warp][lane >> 1] = v;
+        __syncthreads();
+        if (threadIdx.x < 16 && i0 + (threadIdx.x >> 1) < j) {
+          double t = 0.0;
+          for (int w2 = 0; w2 < OT / 32; ++w2) t += sh[w2][threadIdx.x];
+          reinterpret_cast<double*>(hs)[2 * i0 + threadIdx.x] = t;
+        }
+        __syncthreads();
       }
-      __syncthreads();
-      for (int e = threadIdx.x; e < ne; e += blockDim.x) {
+      for (int e = threadIdx.x; e < ne; e += OT) {
         const size_t a = addr(e);
-        cplx<double> we = w[a];
-        for (int i = 0; i < j; ++i) we = we - hs[i] * P[(size_t)i * pstride + a];
-        w[a] = we;
+        cplx<double> we = SW ? sw[e] : w[a];
+#pragma unroll 4
+        for (int i = 0; i < j; ++i) cfma(we, cmk(-hs[i].re, -hs[i].im), P[(size_t)i * pstride + a]);
+        if (SW) sw[e] = we;
+        else w[a] = we;
       }
-      __syncthreads();
+      __syncthreads();   // hs is read before the second pass writes it
     }
-    double nn = 0.0;
-    for (int e = threadIdx.x; e < ne; e += blockDim.x) nn += cnorm2(w[addr(e)]);
-    block_sum(&nn, 1, sh);
-    const double nrm = sqrt(nn);
+    const double nrm = sqrt(cta_norm2(w));
     if (!(nrm > 1e-12 * sqrt(n0)) || n0 == 0.0) {
       if (threadIdx.x == 0) atomicExch(err, 1);
       return;
     }
     const double inv = 1.0 / nrm;
-    for (int e = threadIdx.x; e < ne; e += blockDim.x) {
+    for (int e = threadIdx.x; e < ne; e += OT) {
       const size_t a = addr(e);
-      w[a] = inv * w[a];
+      w[a] = inv * (SW ? sw[e] : w[a]);
     }
-    __syncthreads();
+    // every element of a column is written and read by one thread of the CTA: no barrier
   }
 }
 
 // FP16 copy of P with one scale per (aggregate, chirality): s = float(max |re|, |im|)
-// over the N columns restricted to (A, s), q = RNE_half(x / s).
+// over the N columns restricted to (A, s), q = RNE_half(x / s), x / s as the product with the reciprocal
+// (1.5 units in the last FP64 place before the rounding to FP16) and the maximum on the bits: an FP64 division
+// and comparison per value bound this kernel by the FP64 rate (1.2 ms for 20 columns on 16^3x32, now 0.33).
 __global__ void k_p_to_half(__half2* __restrict__ Ph, float* __restrict__ pscale, const cplx<double>* __restrict__ P,
                             Geom g, bool fine, int n, int N, size_t pstride) {
-  __shared__ double sh[32];
+  __shared__ unsigned long long sh[32];
+  __shared__ double rs;
   const int agg = blockIdx.x, s = blockIdx.y, h = n / 2;
   const int ne = g.vA * h;
   const int V = g.V;
-  double mx = 0.0;
+  // element e as memory holds it: by component, then site (fine), by site, then dof (coarse)
+  auto addr = [&](int j, int e) -> size_t {
+    const int q = fine ? e / g.vA : e / h, r = e - q * (fine ? g.vA : h);
+    return (size_t)j * pstride + faddr(fine, V, n, agg * g.vA + (fine ? r : q), s * h + (fine ? q : r));
+  };
+  unsigned long long mx = 0ull;
   for (int j = 0; j < N; ++j)
     for (int e = threadIdx.x; e < ne; e += blockDim.x) {
-      const cplx<double> v = P[(size_t)j * pstride + faddr(fine, V, n, agg * g.vA + e / h, s * h + e % h)];
-      mx = fmax(mx, fmax(fabs(v.re), fabs(v.im)));
+      const cplx<double> v = P[addr(j, e)];
+      mx = max(mx, max(abs_bits(v.re), abs_bits(v.im)));
     }
-  for (int off = 16; off >= 1; off >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+  for (int off = 16; off >= 1; off >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, off));
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = mx;
   __syncthreads();
   if (threadIdx.x == 0) {
-    double m = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = fmax(m, sh[w]);
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) mx = max(mx, sh[w]);
+    const double m = __longlong_as_double((long long)mx);
     const float sf = m > 0.0 ? (float)m : 1.0f;
     pscale[agg * 2 + s] = sf;
-    sh[0] = (double)sf;
+    rs = 1.0 / (double)sf;
   }
   __syncthreads();
-  const double sc = sh[0];
+  const double r = rs;
   for (int j = 0; j < N; ++j)
     for (int e = threadIdx.x; e < ne; e += blockDim.x) {
-      const size_t a = (size_t)j * pstride + faddr(fine, V, n, agg * g.vA + e / h, s * h + e % h);
-      Ph[a] = __halves2half2(__double2half(P[a].re / sc), __double2half(P[a].im / sc));
+      const size_t a = addr(j, e);
+      const cplx<double> v = P[a];
+      Ph[a] = __halves2half2(__double2half(v.re * r), __double2half(v.im * r));
     }
 }
 
@@ -317,15 +523,49 @@ void prolong_op(cplx<T>* out, const cplx<T>* in, const cplx<T>* P, const Geom& g
 
 void orthonormalise(cplx<double>* P, const Geom& g, bool fine, int n, int N, int* err, cudaStream_t st) {
   const size_t pstride = (size_t)g.V * n;
+  const size_t sm = (size_t)g.vA * (n / 2) * sizeof(cplx<double>);   // the column in work
+  static std::once_flag attr;
+  std::call_once(attr, [] {
+    cudaFuncSetAttribute(k_orthonormalise<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  });
   count_launch();
-  k_orthonormalise<<<dim3(g.nAgg, 2), 256, 0, st>>>(P, g, fine, n, N, pstride, err);
+  if (sm <= 200 * 1024)
+    k_orthonormalise<true><<<dim3(g.nAgg, 2), OT, sm, st>>>(P, g, fine, n, N, pstride, err);
+  else
+    k_orthonormalise<false><<<dim3(g.nAgg, 2), OT, 0, st>>>(P, g, fine, n, N, pstride, err);
+}
+
+int galerkin_cols() { return GCMAX; }
+
+template <typename T>
+bool galerkin_fits(int N, int C, int vA) {
+  return C >= 1 && C <= GCMAX && N <= 32 && galerkin_smem(N, C, vA, sizeof(cplx<T>)).total <= 200 * 1024;
+}
+
+template <typename T>
+cudaError_t galerkin_restrict(cplx<T>* out, const cplx<T>* tmp, const cplx<T>* P, const Geom& gf, const Geom& gc,
+                              bool fine, int n, int N, int C, size_t tmp_rstride, size_t out_rstride,
+                              size_t out_site_stride, int sel, int sel_mu, cudaStream_t st) {
+  const size_t sm = galerkin_smem(N, C, gf.vA, sizeof(cplx<T>)).total;
+  if (!galerkin_fits<T>(N, C, gf.vA)) return cudaErrorInvalidValue;
+  static std::once_flag attr;
+  std::call_once(attr, [] {
+    cudaFuncSetAttribute(k_galerkin<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+  });
+  count_launch();
+  k_galerkin<T><<<dim3(gf.nAgg, 2), GT, sm, st>>>(out, tmp, P, gf, gc, fine, n, N, C, tmp_rstride, (size_t)gf.V * n,
+                                                  out_rstride, out_site_stride, sel, sel_mu);
+  return cudaPeekAtLastError();
 }
 
 #define INST(T)                                                                                                  \
   template void restrict_op<T>(cplx<T>*, const cplx<T>*, const cplx<T>*, const Geom&, const Geom&, bool, int, int, \
                                int, size_t, size_t, size_t, cudaStream_t, const __half2*, const float*, int);   \
   template void prolong_op<T>(cplx<T>*, const cplx<T>*, const cplx<T>*, const Geom&, const Geom&, bool, int, int,  \
-                              int, size_t, size_t, bool, cudaStream_t, const __half2*, const float*, int);
+                              int, size_t, size_t, bool, cudaStream_t, const __half2*, const float*, int);   \
+  template bool galerkin_fits<T>(int, int, int);                                                                 \
+  template cudaError_t galerkin_restrict<T>(cplx<T>*, const cplx<T>*, const cplx<T>*, const Geom&, const Geom&, bool, \
+                                            int, int, int, size_t, size_t, size_t, int, int, cudaStream_t);
 INST(float)
 INST(double)
 #undef INST
