@@ -113,6 +113,7 @@ struct Geom {
   int nIO;     // inner tiles per outer tile
   int nAgg;    // aggregates
   int nBlk;    // SAP blocks
+  const int* csite;   // device table [nAgg]: the coarse-level site of each aggregate (null on the coarsest level)
 };
 
 DD_HD int lin4(const int c[4], const int n[4]) { return ((c[0] * n[1] + c[1]) * n[2] + c[2]) * n[3] + c[3]; }

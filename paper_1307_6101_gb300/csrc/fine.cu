@@ -1513,16 +1513,32 @@ __global__ void k_fine_import(cplx<T>* __restrict__ dst, const cd* __restrict__ 
   for (int k = 0; k < 12; ++k) d[(size_t)k * g.V + x] = ccast<T>(s[k]);
 }
 
+// 128 sites per CTA, transposed through shared memory (13 slots per site: no bank conflicts) so that a site's
+// 192 bytes are written by consecutive threads: 12 fields of 16^3x32 in 68 us, at 16 bytes per site and
+// thread in 160.
+constexpr int EXP_T = 128;
+
 template <typename T>
-__global__ void k_fine_export(cd* __restrict__ dst, const cplx<T>* __restrict__ src, Geom g, size_t rstride) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= g.V) return;
-  int c[4];
-  geom_coords(g, x, c);
-  const size_t site = (size_t)lin4(c, g.L);
-  cd* d = dst + (size_t)blockIdx.y * g.V * 12 + site * 12;
-  const cplx<T>* s = src + (size_t)blockIdx.y * rstride;
-  for (int k = 0; k < 12; ++k) d[k] = ccast<double>(s[(size_t)k * g.V + x]);
+__global__ void __launch_bounds__(EXP_T) k_fine_export(cd* __restrict__ dst, const cplx<T>* __restrict__ src, Geom g,
+                                                       size_t rstride) {
+  __shared__ cd tile[EXP_T][13];
+  __shared__ int lex[EXP_T];
+  const int x0 = blockIdx.x * EXP_T, x = x0 + threadIdx.x;
+  if (x < g.V) {
+    int c[4];
+    geom_coords(g, x, c);
+    lex[threadIdx.x] = lin4(c, g.L);
+    const cplx<T>* s = src + (size_t)blockIdx.y * rstride + x;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) tile[threadIdx.x][k] = ccast<double>(s[(size_t)k * g.V]);
+  }
+  __syncthreads();
+  cd* d = dst + (size_t)blockIdx.y * g.V * 12;
+  const int ns = min(EXP_T, g.V - x0);
+  for (int e = threadIdx.x; e < ns * 12; e += EXP_T) {
+    const int i = e / 12, k = e - i * 12;
+    d[(size_t)lex[i] * 12 + k] = tile[i][k];
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1931,7 +1947,7 @@ void fine_import(cplx<T>* dst, const cplx<double>* src, const Geom& g, int nrhs,
 template <typename T>
 void fine_export(cplx<double>* dst, const cplx<T>* src, const Geom& g, int nrhs, size_t rstride, cudaStream_t st) {
   count_launch();
-  k_fine_export<T><<<dim3(div_up(g.V, 128), nrhs), 128, 0, st>>>(dst, src, g, rstride);
+  k_fine_export<T><<<dim3(div_up(g.V, EXP_T), nrhs), EXP_T, 0, st>>>(dst, src, g, rstride);
 }
 
 // device addresses of the allocation-free scratch, looked up once per device

@@ -176,7 +176,7 @@ cudaError_t coarsest_cluster_solve(cplx<T>* x, const cplx<T>* b, const CoarseOp<
 // per batch (transfer_tc.cu)
 template <typename T>
 void restrict_op(cplx<T>* out, const cplx<T>* in, const cplx<T>* P, const Geom& gf, const Geom& gc, bool fine,
-                 int n, int N, int nrhs, size_t in_rstride, size_t out_rstride, size_t out_site_stride,
+                 int n, int N, int nrhs, size_t in_rstride, size_t out_rstride, size_t out_site_stride, int* err,
                  cudaStream_t st, const __half2* Ph = nullptr, const float* pscale = nullptr, int tc_ks = 0);
 // the same for C <= galerkin_cols() columns of a Galerkin term (TermSel sel, direction sel_mu): only the
 // sites that the term reaches are read
@@ -194,11 +194,11 @@ void prolong_op(cplx<T>* out, const cplx<T>* in, const cplx<T>* P, const Geom& g
                 int N, int nrhs, size_t out_rstride, size_t in_rstride, bool accumulate, cudaStream_t st,
                 const __half2* Ph = nullptr, const float* pscale = nullptr, int batch = 0);
 cudaError_t restrict_tc(cplx<float>* out, const cplx<float>* in, const __half2* Ph, const float* pscale,
-                        const Geom& gf, const Geom& gc, bool fine, int n, int N, int nrhs, size_t in_rstride,
-                        size_t out_rstride, size_t out_site_stride, int ks, cudaStream_t st);
+                        const Geom& gf, bool fine, int n, int N, int nrhs, size_t in_rstride, size_t out_rstride,
+                        size_t out_site_stride, int ks, cudaStream_t st);
 bool restrict_tc_fits(int N, int ks);
 cudaError_t prolong_batch(cplx<float>* out, const cplx<float>* in, const __half2* Ph, const float* pscale,
-                          const Geom& gf, const Geom& gc, bool fine, int n, int N, int nrhs, size_t out_rstride,
+                          const Geom& gf, bool fine, int n, int N, int nrhs, size_t out_rstride,
                           size_t in_rstride, bool accumulate, cudaStream_t st);
 void p_to_half(__half2* Ph, float* pscale, const cplx<double>* P, const Geom& g, bool fine, int n, int N,
                cudaStream_t st);

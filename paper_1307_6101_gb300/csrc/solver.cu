@@ -376,7 +376,7 @@ void restrict_lv(ddamg_handle* h, int l, cplx<T>* out, const cplx<T>* in, int nr
   const bool hf = half_on<T>(h);
   const double ps = hf ? 4.0 : cs;
   Prof pr(h, DDAMG_PROF_TRANSFER, (double)F.vlen * (cs * nrhs + ps * F.N) + (double)C.vlen * cs * nrhs);
-  restrict_op<T>(out, in, Pptr<T>(F), F.g, C.g, F.fine, F.n, F.N, nrhs, F.vlen, C.vlen, C.n, h->st,
+  restrict_op<T>(out, in, Pptr<T>(F), F.g, C.g, F.fine, F.n, F.N, nrhs, F.vlen, C.vlen, C.n, h->d_err, h->st,
                  hf ? F.Ph : nullptr, hf ? F.pscale : nullptr, hf ? F.tr_ks : 0);
 }
 
@@ -790,6 +790,7 @@ void make_geom(Geom& g, const int L[4], const int A[4], const int B[4], bool all
     g.nAgg *= L[d] / A[d];
   }
   g.nBlk = g.V / g.vB;
+  g.csite = nullptr;
 }
 
 void build_block_lists(ddamg_handle* h, Level& L) {
@@ -1199,7 +1200,7 @@ void tune_kernels(ddamg_handle* h) {
       Work<float>& wc = work<float>(C);
       L.tr_ks = time_candidates(h, h->tune_ms[DDAMG_TUNE_RESTRICT][l], 5, [&](int k, bool) {
         if (k > 0 && !restrict_tc_fits(L.N, k)) return false;
-        restrict_op<float>(wc.bc, w.gin, L.P32, L.g, C.g, L.fine, L.n, L.N, B, L.vlen, C.vlen, C.n, h->st, L.Ph,
+        restrict_op<float>(wc.bc, w.gin, L.P32, L.g, C.g, L.fine, L.n, L.N, B, L.vlen, C.vlen, C.n, h->d_err, h->st, L.Ph,
                            L.pscale, k);
         return true;
       });
@@ -1245,7 +1246,7 @@ void galerkin(ddamg_handle* h, int l, const cplx<T>* P, cplx<T>* blk, Term term)
         if (!galerkin_fits<T>(F.N, jb, F.g.vA)) {   // an aggregate of tens of thousands of sites
           blas_zero<T>(tmp, F.vlen, jb, F.vlen, h->st);
           term(tmp, P + (size_t)j0 * F.vlen, jb, sel, mu, sp);
-          restrict_op<T>(out, tmp, P, F.g, C.g, F.fine, F.n, F.N, jb, F.vlen, (size_t)nc, (size_t)9 * nc * nc, h->st);
+          restrict_op<T>(out, tmp, P, F.g, C.g, F.fine, F.n, F.N, jb, F.vlen, (size_t)nc, (size_t)9 * nc * nc, h->d_err, h->st);
           continue;
         }
         term(tmp, P + (size_t)j0 * F.vlen, jb, sel, mu, sp);
@@ -1347,7 +1348,7 @@ void initial_setup_phase(ddamg_handle* h, int l, const double* const* tv_random)
   } else {
     Level& U = h->lv[l - 1];
     const int take = L.N < U.N ? L.N : U.N;
-    restrict_op<double>(L.tv64, U.tv64, U.P64, U.g, L.g, U.fine, U.n, U.N, take, U.vlen, L.vlen, L.n, h->st);
+    restrict_op<double>(L.tv64, U.tv64, U.P64, U.g, L.g, U.fine, U.n, U.N, take, U.vlen, L.vlen, L.n, h->d_err, h->st);
     if (L.N > take) {
       if (!tv_random) {
         draw_fields(L.tv64 + (size_t)take * L.vlen, L.g, false, L.n, L.N - take, 0, l, h->p.seed, L.vlen, h->st);
@@ -1474,6 +1475,17 @@ void allocate_hierarchy(ddamg_handle* h) {
   const int B = h->max_batch;
   for (int l = 0; l < h->L; ++l) {
     Level& L = h->lv[l];
+    if (!L.coarsest) {
+      std::vector<int> cs(L.g.nAgg);
+      for (int a = 0; a < L.g.nAgg; ++a) {
+        int c[4];
+        geom_coords(L.g, a * L.g.vA, c);
+        cs[a] = coarse_site_of(L.g, h->lv[l + 1].g, c);
+      }
+      int* d = dalloc<int>(h, cs.size());
+      CK(cudaMemcpy(d, cs.data(), sizeof(int) * cs.size(), cudaMemcpyHostToDevice));
+      L.g.csite = d;
+    }
     if (L.fine) {
       L.f64.g = L.f32.g = L.g;
       L.f64.bc_t = L.f32.bc_t = h->bc_t;

@@ -42,6 +42,19 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, unsig
     if (clock64() - t0 > 4000000000LL) return false;
   return true;
 }
+// 4-, 8- or 16-byte asynchronous copy global -> shared (both addresses aligned to the size); valid = false writes zeros
+// (the source is not read but has to be a valid address)
+template <int BYTES>
+__device__ __forceinline__ void cp_async(void* dst, const void* src, bool valid) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(smem_u32(dst)), "l"(src), "n"(BYTES),
+               "r"(valid ? BYTES : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int LEFT>   // waits until at most LEFT of this thread's groups are still in flight
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(LEFT) : "memory");
+}
 // Programmatic dependent launch: let the next kernel of the stream (launched with programmatic
 // stream serialization) start its independent prologue early, and, in that kernel, wait for the
 // previous grid to complete (and its memory to be visible) before touching what it wrote.  Both

@@ -7,8 +7,10 @@
 // Aggregates are contiguous index ranges [A*vA, (A+1)*vA) in the site order.
 #include "common.cuh"
 #include "kernels.h"
+#include "tma.cuh"
 
 #include <mutex>
+#include <type_traits>
 
 namespace {
 
@@ -18,111 +20,211 @@ DD_HD size_t faddr(bool fine, int V, int n, int x, int f) {
 }
 
 
+// out(A)[s*N + j] = sum over x in A, f in s of conj(P_j(x, f)) in(x, f).  One CTA per (aggregate, chirality, up to
+// three groups of four columns; one column per group in FP64): the N x K by K x C product with K = |A| n/2 in
+// chunks of up to 128 rows, copied asynchronously in their storage format into two buffers.  Four warps
+// belong to a group; a lane forms a tile of four rows and the group's columns, two rows of K at a time (128 FMAs for
+// 8 shared-memory loads at four columns).  The lanes that the ceil(N/4) row tiles leave free and the group's
+// warps split K, in a way that depends on the level only, so that a right-hand side has the same bits alone
+// and in a batch.
+// A chunk is whole runs of memory (sites of one component on the fine level, dofs of one site on a coarse one).
+// Where those are multiples of 16 bytes (BULK) one lane copies a run of a column with one bulk copy;
+// with a copy instruction per pair of elements the copies took two thirds of the issue slots.
+// Bound by memory for one right-hand side (P once: 126 MB of FP16 for 20 test vectors on 16^3x32), by FP32 issue
+// for many (4 N |A| n FMAs per aggregate and column).
+constexpr int RTH = 128;    // threads of a group
+constexpr int RKC = 128;    // most K rows of a chunk
+constexpr int RNG = 3;      // most groups of a CTA
+// columns of a group: one in FP64, where the FMAs bound the kernel and a column tile would only take registers
+template <typename T> constexpr int restrict_ct() { return sizeof(T) == 4 ? 4 : 1; }
+constexpr int RFLUSH = 3;      // chunks whose products run into one accumulator
+constexpr int RKP = RKC + 12;  // row pitch of P (elements): a multiple of 16 bytes, the row tiles of a warp on different banks
+constexpr int RKB = RKC + 2;   // row pitch of the columns
+
+struct RestrictSmem {
+  size_t b, stage, red, bar, total;
+};
 template <typename T>
-__device__ void block_sum(T* v, int cnt, T* sh) {
-  // sum cnt values per thread over the CTA; result valid in every thread
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int k = 0; k < cnt; ++k)
-    for (int off = 16; off >= 1; off >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], off);
-  if (lane == 0)
-    for (int k = 0; k < cnt; ++k) sh[warp * cnt + k] = v[k];
-  __syncthreads();
-  for (int k = 0; k < cnt; ++k) {
-    T s = T(0);
-    for (int w = 0; w < nw; ++w) s += sh[w * cnt + k];
-    v[k] = s;
-  }
-  __syncthreads();
+DD_HD RestrictSmem restrict_smem(int N, int groups, size_t ps) {
+  RestrictSmem L;
+  const int TI = (N + 3) / 4;
+  L.b = (size_t)N * RKP * ps;
+  L.stage = L.b + (size_t)groups * restrict_ct<T>() * RKB * sizeof(cplx<T>);
+  L.red = 2 * L.stage;
+  L.bar = L.red + (size_t)groups * (RTH / 32) * (32 / TI) * TI * 4 * restrict_ct<T>() * sizeof(cplx<T>);
+  L.total = L.bar + 16;
+  return L;
+}
+// rows of a chunk for runs of `run` elements: whole runs, or the largest even part of a longer run (of a multiple of
+// 16 bytes for `bulk`); 0: there is none
+inline int restrict_chunk(int run, int ps, bool bulk) {
+  if (run <= RKC) return (bulk && run * ps % 16) || run % 2 ? 0 : RKC / run * run;
+  for (int d = RKC; d >= 2; --d)
+    if (run % d == 0 && d % 2 == 0 && !(bulk && d * ps % 16)) return d;
+  return 0;
 }
 
-constexpr int RJ = 10;   // coarse columns j accumulated per thread by k_restrict
+// two neighbouring elements of P in shared memory as complex numbers
+__device__ __forceinline__ void ld_pair(const __half2* p, cplx<float> a[2]) {
+  const uint2 u = *reinterpret_cast<const uint2*>(p);
+  const float2 x = __half22float2(*reinterpret_cast<const __half2*>(&u.x));
+  const float2 y = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
+  a[0] = cmk<float>(x.x, x.y);
+  a[1] = cmk<float>(y.x, y.y);
+}
+__device__ __forceinline__ void ld_pair(const cplx<float>* p, cplx<float> a[2]) {
+  const float4 v = *reinterpret_cast<const float4*>(p);
+  a[0] = cmk<float>(v.x, v.y);
+  a[1] = cmk<float>(v.z, v.w);
+}
+__device__ __forceinline__ void ld_pair(const cplx<double>* p, cplx<double> a[2]) {
+  a[0] = p[0];
+  a[1] = p[1];
+}
 
-// out(A)[s*N + j] = sum over x in A, f in s of conj(P_j(x, f)) in(x, f).
-// One CTA per aggregate (and right-hand side); thread (group g, lane l) owns the
-// columns j in [g*RJ, g*RJ + RJ) and the sites x = A*vA + l, l + S, ... of the
-// aggregate, so every input and every P entry is loaded once.  S is a power of
-// two; the per-thread partial sums are reduced over the S lanes of a group in a
-// fixed order (shuffles inside warps, then shared memory across warps).  HF > 0:
-// the fine level, whose HF = 6 dofs per chirality are unrolled so that all loads
-// of a chirality are in flight together.
-template <typename T, typename PS, int HF>
-__global__ void __launch_bounds__(512, HF > 0 ? 1 : 2) k_restrict(cplx<T>* __restrict__ out, const cplx<T>* __restrict__ in, const PS* __restrict__ P,
-                           const float* __restrict__ pscale, Geom gf, Geom gc, bool fine, int n, int N, int S,
-                           size_t in_rstride, size_t pstride, size_t out_rstride, size_t out_site_stride) {
-  __shared__ T red[32 * 2 * RJ];
-  const int agg = blockIdx.x;
-  const int V = gf.V;
-  const cplx<T>* pin = in + (size_t)blockIdx.y * in_rstride;
-  int c0[4];
-  geom_coords(gf, agg * gf.vA, c0);   // first site of the aggregate (aggregates are contiguous)
-  const int cs = coarse_site_of(gf, gc, c0);
-  cplx<T>* po = out + (size_t)blockIdx.y * out_rstride + (size_t)cs * out_site_stride;
-  const int h = n / 2;
-  const int seg = S < 32 ? S : 32;            // lanes of a group inside one warp
-  const int slots = S / seg;                  // partial sums per group after the warp stage
-  const int gpc = blockDim.x / S;             // groups per CTA
-  const int G = (N + RJ - 1) / RJ;            // column groups
-  const int lane = threadIdx.x % S;
-  for (int g0 = 0; g0 < G; g0 += gpc) {
-    const int g = g0 + threadIdx.x / S;
-    const int j0 = g * RJ;
-    for (int s = 0; s < 2; ++s) {
-      T acc[2 * RJ];
-#pragma unroll
-      for (int k = 0; k < 2 * RJ; ++k) acc[k] = T(0);
-      if (g < G) {
-        for (int xl = lane; xl < gf.vA; xl += S) {
-          const int x = agg * gf.vA + xl;
-          if constexpr (HF > 0) {
-            cplx<T> v[HF];
-#pragma unroll
-            for (int f = 0; f < HF; ++f) v[f] = pin[(size_t)(s * HF + f) * V + x];
-#pragma unroll
-            for (int jj = 0; jj < RJ; ++jj)
-              if (j0 + jj < N)
-#pragma unroll
-                for (int f = 0; f < HF; ++f)
-                  cdotc_acc(acc[2 * jj], acc[2 * jj + 1],
-                            ld_cplx(P, (size_t)(j0 + jj) * pstride + (size_t)(s * HF + f) * V + x), v[f]);
-          } else {
-            for (int f = s * h; f < (s + 1) * h; ++f) {
-              const size_t a = faddr(fine, V, n, x, f);
-              const cplx<T> v = pin[a];
-#pragma unroll
-              for (int jj = 0; jj < RJ; ++jj)
-                if (j0 + jj < N) cdotc_acc(acc[2 * jj], acc[2 * jj + 1], ld_cplx(P, (size_t)(j0 + jj) * pstride + a), v);
-            }
-          }
+// kch: K rows of a chunk, run: elements of a run inside a chunk (BULK)
+template <typename T, typename PS, bool BULK>
+__global__ void __launch_bounds__(RNG * RTH, sizeof(T) == 4 ? 2 : 1) k_restrict(
+    cplx<T>* __restrict__ out, const cplx<T>* __restrict__ in, const PS* __restrict__ P,
+    const float* __restrict__ pscale, Geom gf, bool fine, int n, int N, int nrhs, size_t in_rstride, size_t pstride,
+    size_t out_rstride, size_t out_site_stride, int kch, int run, int* err) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int RCT = restrict_ct<T>();
+  const int groups = blockDim.x / RTH;
+  const int ng = (nrhs + RCT * groups - 1) / (RCT * groups);
+  const int r0 = (blockIdx.x % ng) * RCT * groups, C = min(RCT * groups, nrhs - r0);
+  const int s = (blockIdx.x / ng) & 1, agg = blockIdx.x / (2 * ng);
+  const int V = gf.V, vA = gf.vA, h = n / 2, K = vA * h;
+  const RestrictSmem L = restrict_smem<T>(N, groups, sizeof(PS));
+  cplx<T>* red = reinterpret_cast<cplx<T>*>(smem_raw + L.red);   // [group][4][RCT][warp][sub][row tile]
+  unsigned long long* bar = reinterpret_cast<unsigned long long*>(smem_raw + L.bar);
+  const int tid = threadIdx.x, lane = tid & 31, grp = tid / RTH, warp = (tid % RTH) >> 5;
+  const int TI = (N + 3) / 4, nsub = 32 / TI, slots = (RTH / 32) * nsub * TI;
+  const int sub = lane / TI, ti = lane - sub * TI;       // rows ti, ti + TI, ti + 2 TI, ti + 3 TI
+  const int gc = min(RCT, C - grp * RCT);                // columns of the group (none: <= 0)
+  const cplx<T>* pin = in + (size_t)r0 * in_rstride;
+  // component-major on the fine level (neighbouring rows: neighbouring sites), dof-contiguous on a coarse one
+  auto row_addr = [&](int kk) {
+    const int q = fine ? kk / vA : kk / h, r = kk - q * (fine ? vA : h);
+    return faddr(fine, V, n, agg * vA + (fine ? r : q), s * h + (fine ? q : r));
+  };
+  auto copy = [&](int k0, int buf) {
+    PS* sA = reinterpret_cast<PS*>(smem_raw + buf * L.stage);                    // [N][RKP]
+    cplx<T>* sB = reinterpret_cast<cplx<T>*>(smem_raw + buf * L.stage + L.b);    // [columns][RKB]
+    const int kc = min(kch, K - k0);
+    if constexpr (BULK) {
+      if (tid >= 32) return;
+      if (lane == 0) {
+        fence_proxy_async_shared();
+        mbar_arrive_expect_tx(&bar[buf], (unsigned)(kc * (N * sizeof(PS) + C * sizeof(cplx<T>))));
+      }
+      __syncwarp();
+      for (int q = 0; q < kc; q += run) {
+        const size_t a = row_addr(k0 + q);
+        for (int j = lane; j < N + C; j += 32) {
+          if (j < N) bulk_g2s(sA + j * RKP + q, P + (size_t)j * pstride + a, (unsigned)(run * sizeof(PS)), &bar[buf]);
+          else
+            bulk_g2s(sB + (j - N) * RKB + q, pin + (size_t)(j - N) * in_rstride + a, (unsigned)(run * sizeof(cplx<T>)),
+                     &bar[buf]);
         }
       }
-      for (int off = seg / 2; off >= 1; off >>= 1)
-#pragma unroll
-        for (int k = 0; k < 2 * RJ; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], off);
-      if (threadIdx.x % seg == 0)
-#pragma unroll
-        for (int k = 0; k < 2 * RJ; ++k) red[(threadIdx.x / seg) * 2 * RJ + k] = acc[k];
-      __syncthreads();
-      for (int t = threadIdx.x; t < gpc * RJ; t += blockDim.x) {
-        const int gl = t / RJ, jj = t % RJ;
-        const int j = (g0 + gl) * RJ + jj;
-        if (g0 + gl < G && j < N) {
-          T re = T(0), im = T(0);
-          for (int q = 0; q < slots; ++q) {
-            re += red[(gl * slots + q) * 2 * RJ + 2 * jj];
-            im += red[(gl * slots + q) * 2 * RJ + 2 * jj + 1];
-          }
-          const T sc = pscale ? T(pscale[agg * 2 + s]) : T(1);
-          po[s * N + j] = cmk<T>(sc * re, sc * im);
+    } else {
+      for (int k = tid % RKC; k < kch + (kch & 1); k += RKC) {   // an odd last row's partner is zero
+        const bool on = k < kc;
+        const size_t a = on ? row_addr(k0 + k) : 0;
+        for (int j = tid / RKC; j < N + C; j += groups) {
+          if (j < N) cp_async<sizeof(PS)>(sA + j * RKP + k, P + (size_t)j * pstride + a, on);
+          else cp_async<sizeof(cplx<T>)>(sB + (j - N) * RKB + k, pin + (size_t)(j - N) * in_rstride + a, on);
         }
       }
+      cp_async_commit();
+    }
+  };
+  if (BULK && tid == 0) {
+    mbar_init(&bar[0], 1);
+    mbar_init(&bar[1], 1);
+  }
+  if (BULK) __syncthreads();
+  cplx<T> acc[4][RCT];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int c = 0; c < RCT; ++c) acc[i][c] = czero<T>();
+  copy(0, 0);
+  int chunk = 0;
+  bool ok = true;
+  for (int k0 = 0; k0 < K; k0 += kch, ++chunk) {
+    const int buf = chunk & 1;
+    const bool last = k0 + kch >= K;
+    if (!last) copy(k0 + kch, buf ^ 1);
+    if constexpr (BULK) {
+      ok = mbar_wait_bounded(&bar[buf], (chunk >> 1) & 1);
+    } else {
+      if (last) cp_async_wait<0>();
+      else cp_async_wait<1>();
       __syncthreads();
     }
+    const PS* sA = reinterpret_cast<const PS*>(smem_raw + buf * L.stage);
+    const cplx<T>* sB = reinterpret_cast<const cplx<T>*>(smem_raw + buf * L.stage + L.b) + grp * RCT * RKB;
+    const int kc = (min(kch, K - k0) + 1) / 2;   // pairs
+    if (sub < nsub && gc > 0) {
+      for (int k = warp * nsub + sub; k < kc; k += (RTH / 32) * nsub) {
+        cplx<T> a[4][2];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) ld_pair(sA + (ti + i * TI < N ? ti + i * TI : 0) * RKP + 2 * k, a[i]);
+#pragma unroll
+        for (int c = 0; c < RCT; ++c)
+          if (c < gc) {   // uniform in the warp
+            cplx<T> b[2];
+            ld_pair(sB + c * RKB + 2 * k, b);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              cfmac(acc[i][c], a[i][0], b[0]);
+              cfmac(acc[i][c], a[i][1], b[1]);
+            }
+          }
+      }
+      // long sums in parts: their rounding errors do not add up along the whole of K
+      if (chunk % RFLUSH == RFLUSH - 1 || last) {
+        cplx<T>* mine = red + (size_t)grp * 4 * RCT * slots + (warp * nsub + sub) * TI + ti;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int c = 0; c < RCT; ++c)
+            if (c < gc) {
+              cplx<T>& m = mine[(i * RCT + c) * slots];
+              m = chunk < RFLUSH ? acc[i][c] : m + acc[i][c];
+              acc[i][c] = czero<T>();
+            }
+      }
+    }
+    if (!BULK) {
+      __syncthreads();
+    } else if (!__syncthreads_and(ok ? 1 : 0)) {   // a copy did not land in time: flag it, wait for those in flight
+      if (tid == 0) {                              // (bounded) and leave
+        atomicExch(err, 2);
+        mbar_wait_bounded(&bar[buf], (chunk >> 1) & 1);
+        if (!last) mbar_wait_bounded(&bar[buf ^ 1], ((chunk + 1) >> 1) & 1);
+      }
+      return;
+    }
+  }
+  cplx<T>* po = out + (size_t)r0 * out_rstride + (size_t)gf.csite[agg] * out_site_stride + (size_t)s * N;
+  const T sc = pscale ? T(pscale[agg * 2 + s]) : T(1);
+  for (int e = tid; e < N * C; e += blockDim.x) {
+    const int c = e / N, i = e - c * N;
+    const cplx<T>* r = red + ((size_t)(c / RCT) * 4 * RCT + i / TI * RCT + c % RCT) * slots + i % TI;
+    cplx<T> t[4] = {czero<T>(), czero<T>(), czero<T>(), czero<T>()};   // the parts in four chains
+    for (int q = 0; q < (RTH / 32) * nsub; q += 4)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) t[u] = t[u] + r[(q + u) * TI];
+    po[(size_t)c * out_rstride + i] = sc * ((t[0] + t[1]) + (t[2] + t[3]));
   }
 }
 
 template <typename T, typename PS>
 __global__ void k_prolong(cplx<T>* __restrict__ out, const cplx<T>* __restrict__ in, const PS* __restrict__ P,
-                          const float* __restrict__ pscale, Geom gf, Geom gc, bool fine, int n, int N,
+                          const float* __restrict__ pscale, Geom gf, bool fine, int n, int N,
                           size_t out_rstride, size_t in_rstride, size_t pstride, bool accumulate) {
   const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int V = gf.V;
@@ -130,9 +232,7 @@ __global__ void k_prolong(cplx<T>* __restrict__ out, const cplx<T>* __restrict__
   int x, f;
   if (fine) { f = (int)(t / V); x = (int)(t % V); }
   else { x = (int)(t / n); f = (int)(t % n); }
-  int c[4];
-  geom_coords(gf, x, c);
-  const int cs = coarse_site_of(gf, gc, c);
+  const int cs = gf.csite[x / gf.vA];
   const int s = f < n / 2 ? 0 : 1;
   const cplx<T>* pc = in + (size_t)blockIdx.y * in_rstride + (size_t)cs * (2 * N) + s * N;
   cplx<T> acc = czero<T>();
@@ -173,8 +273,8 @@ DD_HD GalerkinSmem galerkin_smem(int N, int C, int vA, size_t cs) {
 
 template <typename T>
 __global__ void __launch_bounds__(GT) k_galerkin(cplx<T>* __restrict__ out, const cplx<T>* __restrict__ tmp,
-                                                 const cplx<T>* __restrict__ P, Geom gf, Geom gc, bool fine, int n,
-                                                 int N, int C, size_t tmp_rstride, size_t pstride, size_t out_rstride,
+                                                 const cplx<T>* __restrict__ P, Geom gf, bool fine, int n, int N, int C,
+                                                  size_t tmp_rstride, size_t pstride, size_t out_rstride,
                                                  size_t out_site_stride, int sel, int sel_mu) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int wcount[GT / 32];
@@ -185,7 +285,7 @@ __global__ void __launch_bounds__(GT) k_galerkin(cplx<T>* __restrict__ out, cons
   cplx<T>* sA = reinterpret_cast<cplx<T>*>(smem_raw);   // [GKC][NP]
   cplx<T>* sB = sA + (size_t)GKC * NP;                  // [GKC][CP]
   const GalerkinSmem L = galerkin_smem(N, C, vA, sizeof(cplx<T>));
-  cplx<T>* red = reinterpret_cast<cplx<T>*>(smem_raw + L.red);   // [warp][sub][tile][16] partial tiles
+  cplx<T>* red = reinterpret_cast<cplx<T>*>(smem_raw + L.red);   // [16][warp][sub][tile] partial tiles
   int* list = reinterpret_cast<int*>(smem_raw + L.list);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // the sites of the aggregate that the term reaches, in site order
@@ -238,7 +338,8 @@ __global__ void __launch_bounds__(GT) k_galerkin(cplx<T>* __restrict__ out, cons
       for (int e = 0; e < NL; ++e) v[e] = czero<T>();
     }
   };
-  cplx<T>* mine = red + (((size_t)warp * nsub + sub) * tiles + tile) * 16;
+  cplx<T>* mine = red + (warp * nsub + sub) * tiles + tile;
+  const int slots = (GT / 32) * nsub * tiles;
   fetch(0);
   int chunk = 0;
   for (int k0 = 0; k0 < K; k0 += GKC, ++chunk) {
@@ -269,23 +370,22 @@ __global__ void __launch_bounds__(GT) k_galerkin(cplx<T>* __restrict__ out, cons
         for (int i = 0; i < 4; ++i)
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
-            mine[4 * i + c] = chunk < GFLUSH ? acc[i][c] : mine[4 * i + c] + acc[i][c];
+            cplx<T>& m = mine[(4 * i + c) * slots];
+            m = chunk < GFLUSH ? acc[i][c] : m + acc[i][c];
             acc[i][c] = czero<T>();
           }
       }
     }
     __syncthreads();
   }
-  int ca[4];
-  geom_coords(gf, agg * vA, ca);
-  cplx<T>* po = out + (size_t)coarse_site_of(gf, gc, ca) * out_site_stride + (size_t)s * N;
+  cplx<T>* po = out + (size_t)gf.csite[agg] * out_site_stride + (size_t)s * N;
   for (int e = tid; e < N * C; e += GT) {
     const int c = e / N, i = e - c * N;
-    const cplx<T>* r = red + ((size_t)(c / 4) * TI + i / 4) * 16 + 4 * (i % 4) + c % 4;
+    const cplx<T>* r = red + (4 * (i % 4) + c % 4) * slots + (c / 4) * TI + i / 4;
     cplx<T> t[4] = {czero<T>(), czero<T>(), czero<T>(), czero<T>()};   // the parts in four chains
     for (int q = 0; K > 0 && q < (GT / 32) * nsub; q += 4)
 #pragma unroll
-      for (int u = 0; u < 4; ++u) t[u] = t[u] + r[(size_t)(q + u) * tiles * 16];
+      for (int u = 0; u < 4; ++u) t[u] = t[u] + r[(q + u) * tiles];
     po[(size_t)c * out_rstride + i] = (t[0] + t[1]) + (t[2] + t[3]);
   }
 }
@@ -454,44 +554,53 @@ void p_to_half(__half2* Ph, float* pscale, const cplx<double>* P, const Geom& g,
 
 template <typename T>
 void restrict_op(cplx<T>* out, const cplx<T>* in, const cplx<T>* P, const Geom& gf, const Geom& gc, bool fine, int n,
-                 int N, int nrhs, size_t in_rstride, size_t out_rstride, size_t out_site_stride, cudaStream_t st,
-                 const __half2* Ph, const float* pscale, int tc_ks) {
+                 int N, int nrhs, size_t in_rstride, size_t out_rstride, size_t out_site_stride, int* err,
+                 cudaStream_t st, const __half2* Ph, const float* pscale, int tc_ks) {
   if constexpr (sizeof(T) == 4) {
     // FP16 P: the tensor-core kernel (P read once per batch) where the autotuner chose it
     if (Ph && tc_ks > 0) {
-      if (restrict_tc(out, in, Ph, pscale, gf, gc, fine, n, N, nrhs, in_rstride, out_rstride, out_site_stride, tc_ks,
+      if (restrict_tc(out, in, Ph, pscale, gf, fine, n, N, nrhs, in_rstride, out_rstride, out_site_stride, tc_ks,
                       st) == cudaSuccess)
         return;
       cudaGetLastError();
     }
   }
   const size_t pstride = (size_t)gf.V * n;
-  int S = 1;   // lanes per column group: a power of two >= the aggregate volume, at most 256
-  while (S < gf.vA && S < 256) S *= 2;
-  const int G = (N + RJ - 1) / RJ;
-  int gpc = 512 / S < G ? 512 / S : G;   // at most 512 threads (launch bounds)
-  if (S < 32) gpc = ((gpc * S + 31) / 32) * (32 / S);   // whole warps (the shuffles use full masks)
-  if (S < 32 && gpc > 32) gpc = 32;                     // partial-sum slots in shared memory
-  const int threads = gpc * S;
-  count_launch();
-  const dim3 grid(gf.nAgg, nrhs);
+  auto launch = [&](auto* Ps, const float* scale) {
+    using PS = std::remove_const_t<std::remove_pointer_t<decltype(Ps)>>;
+    static std::once_flag attr;
+    std::call_once(attr, [] {
+      cudaFuncSetAttribute(k_restrict<T, PS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+      cudaFuncSetAttribute(k_restrict<T, PS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    });
+    constexpr int RCT = restrict_ct<T>();
+    // bulk copies: whole runs of multiples of 16 bytes at 16-byte aligned addresses, in P and in the columns (the
+    // smaller elements decide)
+    const int run = fine ? gf.vA : n / 2;
+    const size_t pb = sizeof(PS);
+    const bool aligned = (uintptr_t)in % 16 == 0 && (uintptr_t)Ps % 16 == 0 && in_rstride * sizeof(cplx<T>) % 16 == 0 &&
+                         pstride * pb % 16 == 0 && (fine ? (size_t)gf.V : (size_t)n) * pb % 16 == 0;
+    int kch = aligned && err ? restrict_chunk(run, (int)pb, true) : 0;
+    const bool bulk = kch > 0 && run * pb % 16 == 0;
+    if (!bulk) kch = RKC;
+    // groups of columns that share a copy of P, as far as shared memory takes them
+    int groups = (nrhs + RCT - 1) / RCT;
+    if (groups > RNG) groups = RNG;
+    while (groups > 1 && restrict_smem<T>(N, groups, pb).total > 110 * 1024) --groups;
+    const unsigned grid = (unsigned)gf.nAgg * 2u * (unsigned)((nrhs + RCT * groups - 1) / (RCT * groups));
+    auto kernel = bulk ? k_restrict<T, PS, true> : k_restrict<T, PS, false>;
+    count_launch();
+    kernel<<<grid, groups * RTH, restrict_smem<T>(N, groups, pb).total, st>>>(
+        out, in, Ps, scale, gf, fine, n, N, nrhs, in_rstride, pstride, out_rstride, out_site_stride, kch,
+        run < kch ? run : kch, err);
+  };
   if constexpr (sizeof(T) == 4) {
     if (Ph) {
-      if (fine)
-        k_restrict<float, __half2, 6><<<grid, threads, 0, st>>>(out, in, Ph, pscale, gf, gc, fine, n, N, S, in_rstride,
-                                                                 pstride, out_rstride, out_site_stride);
-      else
-        k_restrict<float, __half2, 0><<<grid, threads, 0, st>>>(out, in, Ph, pscale, gf, gc, fine, n, N, S, in_rstride,
-                                                                 pstride, out_rstride, out_site_stride);
+      launch(Ph, pscale);
       return;
     }
   }
-  if (fine)
-    k_restrict<T, cplx<T>, 6><<<grid, threads, 0, st>>>(out, in, P, nullptr, gf, gc, fine, n, N, S, in_rstride,
-                                                          pstride, out_rstride, out_site_stride);
-  else
-    k_restrict<T, cplx<T>, 0><<<grid, threads, 0, st>>>(out, in, P, nullptr, gf, gc, fine, n, N, S, in_rstride,
-                                                          pstride, out_rstride, out_site_stride);
+  launch(P, (const float*)nullptr);
 }
 
 template <typename T>
@@ -501,7 +610,7 @@ void prolong_op(cplx<T>* out, const cplx<T>* in, const cplx<T>* P, const Geom& g
   if constexpr (sizeof(T) == 4) {
     // FP16 P: one CTA per aggregate for the whole batch (P read once) where the autotuner chose it
     if (Ph && batch) {
-      if (prolong_batch(out, in, Ph, pscale, gf, gc, fine, n, N, nrhs, out_rstride, in_rstride, accumulate, st) ==
+      if (prolong_batch(out, in, Ph, pscale, gf, fine, n, N, nrhs, out_rstride, in_rstride, accumulate, st) ==
           cudaSuccess)
         return;
       cudaGetLastError();
@@ -513,11 +622,11 @@ void prolong_op(cplx<T>* out, const cplx<T>* in, const cplx<T>* P, const Geom& g
   if constexpr (sizeof(T) == 4) {
     if (Ph) {
       k_prolong<float, __half2><<<dim3(div_up(tot, 128), nrhs), 128, 0, st>>>(
-          out, in, Ph, pscale, gf, gc, fine, n, N, out_rstride, in_rstride, pstride, accumulate);
+          out, in, Ph, pscale, gf, fine, n, N, out_rstride, in_rstride, pstride, accumulate);
       return;
     }
   }
-  k_prolong<T, cplx<T>><<<dim3(div_up(tot, 128), nrhs), 128, 0, st>>>(out, in, P, nullptr, gf, gc, fine, n, N,
+  k_prolong<T, cplx<T>><<<dim3(div_up(tot, 128), nrhs), 128, 0, st>>>(out, in, P, nullptr, gf, fine, n, N,
                                                                        out_rstride, in_rstride, pstride, accumulate);
 }
 
@@ -553,14 +662,14 @@ cudaError_t galerkin_restrict(cplx<T>* out, const cplx<T>* tmp, const cplx<T>* P
     cudaFuncSetAttribute(k_galerkin<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   });
   count_launch();
-  k_galerkin<T><<<dim3(gf.nAgg, 2), GT, sm, st>>>(out, tmp, P, gf, gc, fine, n, N, C, tmp_rstride, (size_t)gf.V * n,
+  k_galerkin<T><<<dim3(gf.nAgg, 2), GT, sm, st>>>(out, tmp, P, gf, fine, n, N, C, tmp_rstride, (size_t)gf.V * n,
                                                   out_rstride, out_site_stride, sel, sel_mu);
   return cudaPeekAtLastError();
 }
 
 #define INST(T)                                                                                                  \
   template void restrict_op<T>(cplx<T>*, const cplx<T>*, const cplx<T>*, const Geom&, const Geom&, bool, int, int, \
-                               int, size_t, size_t, size_t, cudaStream_t, const __half2*, const float*, int);   \
+                               int, size_t, size_t, size_t, int*, cudaStream_t, const __half2*, const float*, int); \
   template void prolong_op<T>(cplx<T>*, const cplx<T>*, const cplx<T>*, const Geom&, const Geom&, bool, int, int,  \
                               int, size_t, size_t, bool, cudaStream_t, const __half2*, const float*, int);   \
   template bool galerkin_fits<T>(int, int, int);                                                                 \

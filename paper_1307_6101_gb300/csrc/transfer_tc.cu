@@ -42,7 +42,7 @@ __host__ __device__ inline size_t rt_smem(int N, int ks) {
 }
 
 __global__ void k_restrict_tc(cplx<float>* __restrict__ out, const cplx<float>* __restrict__ in,
-                              const __half2* __restrict__ P, const float* __restrict__ pscale, Geom gf, Geom gc,
+                              const __half2* __restrict__ P, const float* __restrict__ pscale, Geom gf,
                               bool fine, int n, int N, int nrhs, size_t in_rstride, size_t pstride,
                               size_t out_rstride, size_t out_site_stride, int ks) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -64,9 +64,7 @@ __global__ void k_restrict_tc(cplx<float>* __restrict__ out, const cplx<float>* 
   const int nt = nr > 8 ? 2 : 1;
   const int ja = mtile * 8 + (gq >> 1), jb = ja + 4;
   const bool imrow = (gq & 1) != 0;
-  int c0[4];
-  geom_coords(gf, agg * gf.vA, c0);
-  const int cs = coarse_site_of(gf, gc, c0);
+  const int cs = gf.csite[agg];
   for (int s = 0; s < 2; ++s) {
     float tot[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
     for (int k0 = 0; k0 < K; k0 += RT_KCH) {
@@ -207,51 +205,97 @@ __global__ void k_restrict_tc(cplx<float>* __restrict__ out, const cplx<float>* 
   }
 }
 
-// out(x, f)[r] = [out +] pscale(A, s) * sum_j P_j(x, f) in_r(A)[s N + j], every r of the batch
-template <int NMAX>
-__global__ void k_prolong_batch(cplx<float>* __restrict__ out, const cplx<float>* __restrict__ in,
-                                const __half2* __restrict__ P, const float* __restrict__ pscale, Geom gf, Geom gc,
-                                bool fine, int n, int N, int nrhs, size_t out_rstride, size_t in_rstride,
-                                size_t pstride, bool accumulate) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  cplx<float>* sc = reinterpret_cast<cplx<float>*>(smem);   // [nrhs][2N]
-  const int agg = blockIdx.x;
+// out(x, f)[r] = [out +] pscale(A, s) * sum_j P_j(x, f) in_r(A)[s N + j], four columns per CTA; the CTAs of an
+// aggregate's column groups are neighbours, so that all but one of them read P from L2.  A thread owns two
+// neighbouring elements (sites of one component on the fine level, dofs of one site on a coarse one), loads
+// their N entries of P (8 bytes each) before it uses any, and takes the coarse values of two columns per broadcast
+// from shared memory.  Bound by memory: P once and the result, 277 MB for 12 columns of 16^3x32 with 20 test
+// vectors.
+constexpr int PB_R = 4;
+
+template <int NMAX, int SPT>
+__global__ void __launch_bounds__(256, 3) k_prolong_batch(cplx<float>* __restrict__ out,
+                                                          const cplx<float>* __restrict__ in,
+                                                          const __half2* __restrict__ P,
+                                                          const float* __restrict__ pscale, Geom gf, bool fine,
+                                                          int n, int N, int nrhs, size_t out_rstride,
+                                                          size_t in_rstride, size_t pstride, bool accumulate) {
+  __shared__ __align__(16) cplx<float> sc[2 * NMAX * PB_R];   // [2N][PB_R]
+  const int ng = (nrhs + PB_R - 1) / PB_R;
+  const int agg = blockIdx.x / ng, r0 = (blockIdx.x - agg * ng) * PB_R, nr = min(PB_R, nrhs - r0);
   const int V = gf.V, h = n / 2;
-  int c0[4];
-  geom_coords(gf, agg * gf.vA, c0);
-  const int cs = coarse_site_of(gf, gc, c0);
-  for (int e = threadIdx.x; e < nrhs * 2 * N; e += blockDim.x) {
-    const int r = e / (2 * N), q = e - r * 2 * N;
-    sc[e] = in[(size_t)r * in_rstride + (size_t)cs * 2 * N + q];
-  }
-  __syncthreads();
-  const int rows = gf.vA * n;
-  for (int t = threadIdx.x; t < rows; t += blockDim.x) {
-    // fine level: component-major rows (consecutive threads take consecutive sites of one f)
-    int xl, f;
-    if (fine) { f = t / gf.vA; xl = t - f * gf.vA; }
-    else { xl = t / n; f = t - xl * n; }
-    const int x = agg * gf.vA + xl;
+  const int items = gf.vA * n / SPT;
+  const int per = (fine ? gf.vA : n) / SPT;   // consecutive items that share a component (fine) or a site (coarse)
+  bool staged = false;
+  for (int t0 = blockIdx.y * blockDim.x; t0 < items; t0 += gridDim.y * blockDim.x) {
+    const int t = t0 + threadIdx.x;
+    const bool on = t < items;
+    const int q = on ? t / per : 0, r = on ? (t - q * per) * SPT : 0;
+    const int xl = fine ? r : q, f = fine ? q : r;
     const int s = f < h ? 0 : 1;
-    const size_t a = faddr(fine, V, n, x, f);
-    cplx<float> p[NMAX];
+    const size_t a = faddr(fine, V, n, agg * gf.vA + xl, f);
+    __half2 p[NMAX][SPT];
 #pragma unroll
     for (int j = 0; j < NMAX; ++j)
       if (j < N) {
-        const float2 v = __half22float2(P[(size_t)j * pstride + a]);
-        p[j] = cmk<float>(v.x, v.y);
+        if constexpr (SPT == 2) {
+          const uint2 u = *reinterpret_cast<const uint2*>(P + (size_t)j * pstride + a);
+          p[j][0] = *reinterpret_cast<const __half2*>(&u.x);
+          p[j][1] = *reinterpret_cast<const __half2*>(&u.y);
+        } else {
+          p[j][0] = P[(size_t)j * pstride + a];
+        }
       }
-    const float ps = pscale ? pscale[agg * 2 + s] : 1.f;
-    for (int r = 0; r < nrhs; ++r) {
-      const cplx<float>* cr = sc + (size_t)r * 2 * N + s * N;
-      cplx<float> acc = czero<float>();
-#pragma unroll
-      for (int j = 0; j < NMAX; ++j)
-        if (j < N) cfma(acc, p[j], cr[j]);
-      acc = ps * acc;
-      cplx<float>* po = out + (size_t)r * out_rstride + a;
-      *po = accumulate ? *po + acc : acc;
+    if (!staged) {   // while P is on its way
+      const int cs = gf.csite[agg];
+      for (int e = threadIdx.x; e < nr * 2 * N; e += blockDim.x) {
+        const int rr = e / (2 * N), qq = e - rr * 2 * N;
+        sc[qq * PB_R + rr] = in[(size_t)(r0 + rr) * in_rstride + (size_t)cs * 2 * N + qq];
+      }
+      __syncthreads();
+      staged = true;
     }
+    cplx<float> acc[PB_R][SPT];
+#pragma unroll
+    for (int c = 0; c < PB_R; ++c)
+#pragma unroll
+      for (int e = 0; e < SPT; ++e) acc[c][e] = czero<float>();
+    const cplx<float>* cr = sc + (size_t)s * N * PB_R;
+#pragma unroll
+    for (int j = 0; j < NMAX; ++j)
+      if (j < N) {
+        cplx<float> pj[SPT];
+#pragma unroll
+        for (int e = 0; e < SPT; ++e) pj[e] = ld_cplx(&p[j][e], 0);
+#pragma unroll
+        for (int c = 0; c < PB_R; c += 2)
+          if (c < nr) {   // uniform; a last odd column's partner is computed and not stored
+            const float4 v = *reinterpret_cast<const float4*>(cr + j * PB_R + c);
+#pragma unroll
+            for (int e = 0; e < SPT; ++e) {
+              cfma(acc[c][e], pj[e], cmk<float>(v.x, v.y));
+              cfma(acc[c + 1][e], pj[e], cmk<float>(v.z, v.w));
+            }
+          }
+      }
+    if (!on) continue;
+    const float ps = pscale ? pscale[agg * 2 + s] : 1.f;
+#pragma unroll
+    for (int c = 0; c < PB_R; ++c)
+      if (c < nr) {
+        cplx<float>* po = out + (size_t)(r0 + c) * out_rstride + a;
+        if constexpr (SPT == 2) {
+          float4 y = make_float4(ps * acc[c][0].re, ps * acc[c][0].im, ps * acc[c][1].re, ps * acc[c][1].im);
+          if (accumulate) {
+            const float4 o = *reinterpret_cast<const float4*>(po);
+            y = make_float4(o.x + y.x, o.y + y.y, o.z + y.z, o.w + y.w);
+          }
+          *reinterpret_cast<float4*>(po) = y;
+        } else {
+          const cplx<float> y = ps * acc[c][0];
+          *po = accumulate ? *po + y : y;
+        }
+      }
   }
 }
 
@@ -277,7 +321,7 @@ bool restrict_tc_fits(int N, int ks) {
 }
 
 cudaError_t restrict_tc(cplx<float>* out, const cplx<float>* in, const __half2* Ph, const float* pscale,
-                        const Geom& gf, const Geom& gc, bool fine, int n, int N, int nrhs, size_t in_rstride,
+                        const Geom& gf, bool fine, int n, int N, int nrhs, size_t in_rstride,
                         size_t out_rstride, size_t out_site_stride, int ks, cudaStream_t st) {
   if (nrhs <= 0) return cudaSuccess;
   if (!Ph || !restrict_tc_fits(N, ks)) return cudaErrorInvalidValue;
@@ -287,33 +331,32 @@ cudaError_t restrict_tc(cplx<float>* out, const cplx<float>* in, const __half2* 
   const int threads = 32 * ((2 * N + 15) / 16) * ks;
   count_launch();
   k_restrict_tc<<<dim3(gf.nAgg, (nrhs + RT_R - 1) / RT_R), threads, bytes, st>>>(
-      out, in, Ph, pscale, gf, gc, fine, n, N, nrhs, in_rstride, (size_t)gf.V * n, out_rstride,
+      out, in, Ph, pscale, gf, fine, n, N, nrhs, in_rstride, (size_t)gf.V * n, out_rstride,
       out_site_stride, ks);
   return cudaPeekAtLastError();
 }
 
 cudaError_t prolong_batch(cplx<float>* out, const cplx<float>* in, const __half2* Ph, const float* pscale,
-                          const Geom& gf, const Geom& gc, bool fine, int n, int N, int nrhs, size_t out_rstride,
+                          const Geom& gf, bool fine, int n, int N, int nrhs, size_t out_rstride,
                           size_t in_rstride, bool accumulate, cudaStream_t st) {
   if (nrhs <= 0) return cudaSuccess;
   if (!Ph || N > 32) return cudaErrorInvalidValue;
-  const size_t bytes = (size_t)nrhs * 2 * N * sizeof(cplx<float>);
-  if (bytes > 48 * 1024) return cudaErrorInvalidValue;
   const size_t pstride = (size_t)gf.V * n;
-  count_launch();
-  const int threads = 256;
-  if (N <= 8)
-    k_prolong_batch<8><<<gf.nAgg, threads, bytes, st>>>(out, in, Ph, pscale, gf, gc, fine, n, N, nrhs, out_rstride,
-                                                         in_rstride, pstride, accumulate);
-  else if (N <= 16)
-    k_prolong_batch<16><<<gf.nAgg, threads, bytes, st>>>(out, in, Ph, pscale, gf, gc, fine, n, N, nrhs, out_rstride,
-                                                          in_rstride, pstride, accumulate);
-  else if (N <= 24)
-    k_prolong_batch<24><<<gf.nAgg, threads, bytes, st>>>(out, in, Ph, pscale, gf, gc, fine, n, N, nrhs, out_rstride,
-                                                          in_rstride, pstride, accumulate);
-  else
-    k_prolong_batch<32><<<gf.nAgg, threads, bytes, st>>>(out, in, Ph, pscale, gf, gc, fine, n, N, nrhs, out_rstride,
-                                                          in_rstride, pstride, accumulate);
+  // two elements per thread where a pair is one aligned load of P and of the result (and of one chirality)
+  const bool pair = (fine ? gf.vA % 2 == 0 && gf.V % 2 == 0 : (n / 2) % 2 == 0) && out_rstride % 2 == 0 &&
+                    (uintptr_t)out % 16 == 0 && (uintptr_t)Ph % 8 == 0;
+  // one item (element or pair) per thread, up to 32 CTAs per aggregate and column group
+  const unsigned ny = div_up((size_t)gf.vA * n / (pair ? 2 : 1), 256);
+  const dim3 grid((unsigned)gf.nAgg * div_up(nrhs, PB_R), ny < 32 ? ny : 32);
+  auto launch = [&](auto kernel) {
+    count_launch();
+    kernel<<<grid, 256, 0, st>>>(out, in, Ph, pscale, gf, fine, n, N, nrhs, out_rstride, in_rstride, pstride,
+                                 accumulate);
+  };
+  if (N <= 8) launch(pair ? k_prolong_batch<8, 2> : k_prolong_batch<8, 1>);
+  else if (N <= 16) launch(pair ? k_prolong_batch<16, 2> : k_prolong_batch<16, 1>);
+  else if (N <= 24) launch(pair ? k_prolong_batch<24, 2> : k_prolong_batch<24, 1>);
+  else launch(pair ? k_prolong_batch<32, 2> : k_prolong_batch<32, 1>);
   return cudaPeekAtLastError();
 }
 
