@@ -58,7 +58,7 @@ __global__ void k_coarse_apply(cplx<T>* __restrict__ out, const cplx<T>* __restr
     if (k > 0) {
       const int mu = (k - 1) % 4, dir = k <= 4 ? +1 : -1;
       nb = geom_neighbor(g, c, mu, dir);
-      const bool internal = hop_internal(g, c, mu, dir, g.A);
+      const bool internal = hop_internal(g, c, mu, dir, g.fA);
       if (sel == SEL_FULL) tk = true;
       else if (sel == SEL_AGG_SELF) tk = internal;
       else if (sel == SEL_AGG_FWD) tk = dir > 0 && mu == sel_mu && !internal;
@@ -216,8 +216,13 @@ __global__ void k_schur_even(cplx<T>* __restrict__ y, const cplx<T>* __restrict_
 // block-local order (bsite / bloc tables).  rho = (b - D z)_B, k MR steps on D_B
 // (hops leaving the block dropped), z_B += e_B; the operator is read from global
 // memory.
+// Largest CTA per rows-per-thread variant: what coarse_sap_sweep may launch, so that the compiler keeps the registers
+// within it (blocks of up to 3072 rows in FP64 and 3840 in FP32).
+template <typename T, int RPT> constexpr int coarse_sap_threads() {
+  return sizeof(T) == 8 ? (RPT == 1 ? 896 : RPT == 4 ? 576 : 384) : (RPT == 1 ? 1024 : RPT == 4 ? 800 : 480);
+}
 template <typename T, typename BS, int RPT>
-__global__ void k_coarse_sap(cplx<T>* __restrict__ z, const cplx<T>* __restrict__ bsrc,
+__global__ void __launch_bounds__(coarse_sap_threads<T, RPT>()) k_coarse_sap(cplx<T>* __restrict__ z, const cplx<T>* __restrict__ bsrc,
                              const BS* __restrict__ blk, const float* __restrict__ bscale, Geom g, int n,
                              size_t rstride, const int* __restrict__ blocks, int k_mr,
                              const int* __restrict__ bsite, const int* __restrict__ bloc) {
@@ -283,7 +288,7 @@ __global__ void k_coarse_sap(cplx<T>* __restrict__ z, const cplx<T>* __restrict_
         for (int mu = 0; mu < 4; ++mu)
           for (int sd = 0; sd < 2; ++sd) {
             const int dir = sd ? -1 : +1, k = sd ? 5 + mu : 1 + mu;
-            if (!hop_internal(g, c, mu, dir, g.B)) continue;
+            if (!hop_internal(g, c, mu, dir, g.fB)) continue;
             const cplx<T>* v = rs + (size_t)bloc[geom_neighbor(g, c, mu, dir)] * n;
 #pragma unroll 8
             for (int j = 0; j < n; ++j) cfma(acc, ld_cplx(blk, bidx(site, k, n, i, j)), v[j]);
@@ -391,7 +396,7 @@ __global__ void __launch_bounds__(768, 2) k_coarse_sap_cluster(cplx<T>* __restri
     sl9[0] = ns++;
     for (int sd = 0; sd < 2; ++sd)
       for (int mu = 0; mu < 4; ++mu)
-        sl9[(sd ? 5 : 1) + mu] = hop_internal(g, c, mu, sd ? -1 : +1, g.B) ? ns++ : -1;
+        sl9[(sd ? 5 : 1) + mu] = hop_internal(g, c, mu, sd ? -1 : +1, g.fB) ? ns++ : -1;
   }
   if (threadIdx.x == 0) mbar_init(bar, 1);
   __syncthreads();
@@ -653,7 +658,7 @@ __global__ void __launch_bounds__(768, 1) k_coarse_sap_persist(
       sl9[0] = ns++;
       for (int sd = 0; sd < 2; ++sd)
         for (int mu = 0; mu < 4; ++mu)
-          sl9[(sd ? 5 : 1) + mu] = hop_internal(g, co, mu, sd ? -1 : +1, g.B) ? ns++ : -1;
+          sl9[(sd ? 5 : 1) + mu] = hop_internal(g, co, mu, sd ? -1 : +1, g.fB) ? ns++ : -1;
     } else {
       for (int e = 0; e < 9; ++e) sl9[e] = -1;
     }
@@ -1044,7 +1049,7 @@ int coarse_sap_slots(const Geom& g) {
     int c[4];
     delin4(loc, g.B, c);   // the sites of the block at the origin
     int cnt = 1;
-    for (int k = 1; k < 9; ++k) cnt += hop_internal(g, c, (k - 1) % 4, k <= 4 ? +1 : -1, g.B) ? 1 : 0;
+    for (int k = 1; k < 9; ++k) cnt += hop_internal(g, c, (k - 1) % 4, k <= 4 ? +1 : -1, g.fB) ? 1 : 0;
     best = cnt > best ? cnt : best;
   }
   return best;

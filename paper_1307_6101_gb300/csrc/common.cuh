@@ -98,6 +98,25 @@ __device__ __forceinline__ unsigned long long abs_bits(double x) {
 // extents B, one of which tiles the other.  The larger is the outer tile O, the
 // smaller the inner tile I; index = (lin(c/O) * nIO + lin((c%O)/I)) * vI + lin(c%I),
 // so aggregates and SAP blocks are both contiguous index ranges.
+// Division by a fixed positive integer as a multiplication: with 2^(l-1) < d <= 2^l and m = ceil(2^(31+l) / d),
+// floor(x m / 2^(31+l)) = floor(x / d) for 0 <= x < 2^31 (m d exceeds 2^(31+l) by less than 2^l; Granlund and
+// Montgomery, "Division by invariant integers using multiplication", PLDI 1994).  An integer division takes about
+// twenty instructions, and a site's coordinates and neighbours some hundred divisions: in kernels that derive
+// them per thread they were the larger part of the time (k_prolong on 16^3x32: 55 us, 29 with a table).
+struct FDiv {
+  unsigned m;
+  int sh;
+};
+inline FDiv fdiv_make(int d) {
+  int l = 0;
+  while ((1ll << l) < d) ++l;
+  FDiv f;
+  f.m = (unsigned)(((1ull << (31 + l)) + (unsigned)d - 1) / (unsigned)d);
+  f.sh = 31 + l;
+  return f;
+}
+DD_HD int fdiv(int x, FDiv f) { return (int)(((unsigned long long)(unsigned)x * f.m) >> f.sh); }
+
 struct Geom {
   int L[4];
   int A[4];
@@ -113,6 +132,8 @@ struct Geom {
   int nIO;     // inner tiles per outer tile
   int nAgg;    // aggregates
   int nBlk;    // SAP blocks
+  FDiv fO[4], fI[4], fnO[4], fnI[4], fA[4], fB[4];   // divisions by the extents above
+  FDiv fvI, fnIO, fvA;
   const int* csite;   // device table [nAgg]: the coarse-level site of each aggregate (null on the coarsest level)
 };
 
@@ -128,23 +149,32 @@ DD_HD int geom_index(const Geom& g, const int c[4]) {
   int a[4], b[4], l[4];
 #pragma unroll
   for (int d = 0; d < 4; ++d) {
-    a[d] = c[d] / g.O[d];
-    int r = c[d] - a[d] * g.O[d];
-    b[d] = r / g.I[d];
+    a[d] = fdiv(c[d], g.fO[d]);
+    const int r = c[d] - a[d] * g.O[d];
+    b[d] = fdiv(r, g.fI[d]);
     l[d] = r - b[d] * g.I[d];
   }
   return (lin4(a, g.nO) * g.nIO + lin4(b, g.nI)) * g.vI + lin4(l, g.I);
 }
 
+// delin4 with the divisions by the extents n as f
+DD_HD void delin4(int l, const int n[4], const FDiv f[4], int c[4]) {
+#pragma unroll
+  for (int d = 3; d >= 1; --d) {
+    const int q = fdiv(l, f[d]);
+    c[d] = l - q * n[d];
+    l = q;
+  }
+  c[0] = l;
+}
+
 DD_HD void geom_coords(const Geom& g, int idx, int c[4]) {
   int l[4], b[4], a[4];
-  int loc = idx % g.vI;
-  int r = idx / g.vI;
-  int blk = r % g.nIO;
-  int agg = r / g.nIO;
-  delin4(loc, g.I, l);
-  delin4(blk, g.nI, b);
-  delin4(agg, g.nO, a);
+  const int r = fdiv(idx, g.fvI);
+  const int agg = fdiv(r, g.fnIO);
+  delin4(idx - r * g.vI, g.I, g.fI, l);
+  delin4(r - agg * g.nIO, g.nI, g.fnI, b);
+  delin4(agg, g.nO, g.fnO, a);
 #pragma unroll
   for (int d = 0; d < 4; ++d) c[d] = (a[d] * g.nI[d] + b[d]) * g.I[d] + l[d];
 }
@@ -158,17 +188,17 @@ DD_HD int geom_neighbor(const Geom& g, const int c[4], int mu, int dir) {
   return geom_index(g, n);
 }
 
-// does the hop from x in direction dir*mu stay in x's tile of extent t (with wrap)?
-DD_HD bool hop_internal(const Geom& g, const int c[4], int mu, int dir, const int* tile) {
+// does the hop from x in direction dir*mu stay in x's tile (with wrap)?  tile: g.fA or g.fB
+DD_HD bool hop_internal(const Geom& g, const int c[4], int mu, int dir, const FDiv* tile) {
   int n = c[mu] + dir;
   if (n < 0) n += g.L[mu];
   if (n >= g.L[mu]) n -= g.L[mu];
-  return (n / tile[mu]) == (c[mu] / tile[mu]);
+  return fdiv(n, tile[mu]) == fdiv(c[mu], tile[mu]);
 }
 
 // SAP block colour (sum of block coordinates mod 2)
 DD_HD int geom_block_colour(const Geom& g, const int c[4]) {
-  return (c[0] / g.B[0] + c[1] / g.B[1] + c[2] / g.B[2] + c[3] / g.B[3]) & 1;
+  return (fdiv(c[0], g.fB[0]) + fdiv(c[1], g.fB[1]) + fdiv(c[2], g.fB[2]) + fdiv(c[3], g.fB[3])) & 1;
 }
 
 DD_HD int geom_parity(const int c[4]) { return (c[0] + c[1] + c[2] + c[3]) & 1; }
@@ -177,7 +207,7 @@ DD_HD int geom_parity(const int c[4]) { return (c[0] + c[1] + c[2] + c[3]) & 1; 
 DD_HD int coarse_site_of(const Geom& fine, const Geom& coarse, const int c[4]) {
   int ca[4];
 #pragma unroll
-  for (int d = 0; d < 4; ++d) ca[d] = c[d] / fine.A[d];
+  for (int d = 0; d < 4; ++d) ca[d] = fdiv(c[d], fine.fA[d]);
   return geom_index(coarse, ca);
 }
 

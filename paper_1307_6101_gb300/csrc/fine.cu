@@ -197,16 +197,16 @@ __global__ void k_fine_dslash(cplx<T>* __restrict__ out, const cplx<T>* __restri
   int c[4];
   geom_coords(g, x, c);
   // the term of a hop that leaves the aggregate: sites without it are not written (nor read by the product with P^+)
-  if (sel == SEL_AGG_FWD && hop_internal(g, c, sel_mu, +1, g.A)) return;
-  if (sel == SEL_AGG_BWD && hop_internal(g, c, sel_mu, -1, g.A)) return;
+  if (sel == SEL_AGG_FWD && hop_internal(g, c, sel_mu, +1, g.fA)) return;
+  if (sel == SEL_AGG_BWD && hop_internal(g, c, sel_mu, -1, g.fA)) return;
   cplx<T> acc[12];
 #pragma unroll
   for (int k = 0; k < 12; ++k) acc[k] = czero<T>();
   cplx<T> nb[12], u[9];
 #pragma unroll 1
   for (int mu = 0; mu < 4; ++mu) {
-    const bool inf = hop_internal(g, c, mu, +1, g.A);
-    const bool inb = hop_internal(g, c, mu, -1, g.A);
+    const bool inf = hop_internal(g, c, mu, +1, g.fA);
+    const bool inb = hop_internal(g, c, mu, -1, g.fA);
     bool tf = true, tb = true;
     if (sel == SEL_AGG_SELF) { tf = inf; tb = inb; }
     else if (sel == SEL_AGG_FWD) { tf = (mu == sel_mu) && !inf; tb = false; }
@@ -414,7 +414,7 @@ __global__ void k_fine_sap(cplx<T>* __restrict__ z, const cplx<T>* __restrict__ 
 #pragma unroll 1
       for (int mu = 0; mu < 4; ++mu) {
         // a block that spans the whole time extent keeps the wrapping hop, with its boundary sign
-        if (hop_internal(g, c, mu, +1, g.B)) {
+        if (hop_internal(g, c, mu, +1, g.fB)) {
           const int n = geom_neighbor(g, c, mu, +1);
           const int sl = base + (n - blk * g.vB);
           const bool neg = mu == 0 && bc_t < 0 && c[0] == g.L[0] - 1;
@@ -426,7 +426,7 @@ __global__ void k_fine_sap(cplx<T>* __restrict__ z, const cplx<T>* __restrict__ 
           load_link(U, V, mu, x, u);
           hop_accumulate(mu, true, u, nb, acc);
         }
-        if (hop_internal(g, c, mu, -1, g.B)) {
+        if (hop_internal(g, c, mu, -1, g.fB)) {
           const int n = geom_neighbor(g, c, mu, -1);
           const int sl = base + (n - blk * g.vB);
           const bool neg = mu == 0 && bc_t < 0 && c[0] == 0;

@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_fine_sap_split(cplx<double>* _
     if (active && comp == 0)
 #pragma unroll 1
       for (int mu = 0; mu < 4; ++mu) {
-        const bool f = hop_internal(g, c, mu, +1, g.B), b = hop_internal(g, c, mu, -1, g.B);
+        const bool f = hop_internal(g, c, mu, +1, g.fB), b = hop_internal(g, c, mu, -1, g.fB);
         nin[2 * mu * S + l] =
             f || b ? (short)(2 * (geom_neighbor(g, c, mu, f ? +1 : -1) - blk * vB) + (f ? 1 : 0)) : (short)-1;
         nin[(2 * mu + 1) * S + l] = f && b ? (short)(2 * (geom_neighbor(g, c, mu, -1) - blk * vB)) : (short)-1;

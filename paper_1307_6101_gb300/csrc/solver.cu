@@ -790,6 +790,17 @@ void make_geom(Geom& g, const int L[4], const int A[4], const int B[4], bool all
     g.nAgg *= L[d] / A[d];
   }
   g.nBlk = g.V / g.vB;
+  for (int d = 0; d < 4; ++d) {
+    g.fO[d] = fdiv_make(g.O[d]);
+    g.fI[d] = fdiv_make(g.I[d]);
+    g.fnO[d] = fdiv_make(g.nO[d]);
+    g.fnI[d] = fdiv_make(g.nI[d]);
+    g.fA[d] = fdiv_make(g.A[d]);
+    g.fB[d] = fdiv_make(g.B[d]);
+  }
+  g.fvI = fdiv_make(g.vI);
+  g.fnIO = fdiv_make(g.nIO);
+  g.fvA = fdiv_make(g.vA);
   g.csite = nullptr;
 }
 

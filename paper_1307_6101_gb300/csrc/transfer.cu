@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(RNG * RTH, sizeof(T) == 4 ? 2 : 1) k_restrict(
   const cplx<T>* pin = in + (size_t)r0 * in_rstride;
   // component-major on the fine level (neighbouring rows: neighbouring sites), dof-contiguous on a coarse one
   auto row_addr = [&](int kk) {
-    const int q = fine ? kk / vA : kk / h, r = kk - q * (fine ? vA : h);
+    const int q = fine ? fdiv(kk, gf.fvA) : kk / h, r = kk - q * (fine ? vA : h);
     return faddr(fine, V, n, agg * vA + (fine ? r : q), s * h + (fine ? q : r));
   };
   auto copy = [&](int k0, int buf) {
@@ -226,13 +226,12 @@ template <typename T, typename PS>
 __global__ void k_prolong(cplx<T>* __restrict__ out, const cplx<T>* __restrict__ in, const PS* __restrict__ P,
                           const float* __restrict__ pscale, Geom gf, bool fine, int n, int N,
                           size_t out_rstride, size_t in_rstride, size_t pstride, bool accumulate) {
-  const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  // blockIdx.x: elements of a component (fine) or of all sites (coarse); blockIdx.z: component (fine)
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int V = gf.V;
-  if (t >= (size_t)V * n) return;
-  int x, f;
-  if (fine) { f = (int)(t / V); x = (int)(t % V); }
-  else { x = (int)(t / n); f = (int)(t % n); }
-  const int cs = gf.csite[x / gf.vA];
+  if (t >= (fine ? V : V * n)) return;
+  const int x = fine ? t : t / n, f = fine ? (int)blockIdx.z : t - x * n;
+  const int cs = gf.csite[fdiv(x, gf.fvA)];
   const int s = f < n / 2 ? 0 : 1;
   const cplx<T>* pc = in + (size_t)blockIdx.y * in_rstride + (size_t)cs * (2 * N) + s * N;
   cplx<T> acc = czero<T>();
@@ -295,7 +294,7 @@ __global__ void __launch_bounds__(GT) k_galerkin(cplx<T>* __restrict__ out, cons
     if (take && sel != SEL_AGG_SELF) {
       int c[4];
       geom_coords(gf, agg * vA + x0 + tid, c);
-      take = !hop_internal(gf, c, sel_mu, sel == SEL_AGG_FWD ? +1 : -1, gf.A);
+      take = !hop_internal(gf, c, sel_mu, sel == SEL_AGG_FWD ? +1 : -1, gf.fA);
     }
     const unsigned m = __ballot_sync(0xffffffffu, take);
     if (lane == 0) wcount[warp] = __popc(m);
@@ -428,7 +427,7 @@ __global__ void __launch_bounds__(OT) k_orthonormalise(cplx<double>* __restrict_
   // element e of the block: fine fields by component, then site; coarse fields by site, then dof
   auto addr = [&](int e) -> size_t {
     if (fine) {
-      const int f = e / g.vA;
+      const int f = fdiv(e, g.fvA);
       return (size_t)(s * h + f) * g.V + (size_t)agg * g.vA + (e - f * g.vA);
     }
     const int x = e / h;
@@ -513,7 +512,7 @@ __global__ void k_p_to_half(__half2* __restrict__ Ph, float* __restrict__ pscale
   const int V = g.V;
   // element e as memory holds it: by component, then site (fine), by site, then dof (coarse)
   auto addr = [&](int j, int e) -> size_t {
-    const int q = fine ? e / g.vA : e / h, r = e - q * (fine ? g.vA : h);
+    const int q = fine ? fdiv(e, g.fvA) : e / h, r = e - q * (fine ? g.vA : h);
     return (size_t)j * pstride + faddr(fine, V, n, agg * g.vA + (fine ? r : q), s * h + (fine ? q : r));
   };
   unsigned long long mx = 0ull;
@@ -617,16 +616,16 @@ void prolong_op(cplx<T>* out, const cplx<T>* in, const cplx<T>* P, const Geom& g
     }
   }
   const size_t pstride = (size_t)gf.V * n;
-  const size_t tot = (size_t)gf.V * n;
+  const dim3 grid(div_up(fine ? (size_t)gf.V : (size_t)gf.V * n, 128), nrhs, fine ? n : 1);
   count_launch();
   if constexpr (sizeof(T) == 4) {
     if (Ph) {
-      k_prolong<float, __half2><<<dim3(div_up(tot, 128), nrhs), 128, 0, st>>>(
+      k_prolong<float, __half2><<<grid, 128, 0, st>>>(
           out, in, Ph, pscale, gf, fine, n, N, out_rstride, in_rstride, pstride, accumulate);
       return;
     }
   }
-  k_prolong<T, cplx<T>><<<dim3(div_up(tot, 128), nrhs), 128, 0, st>>>(out, in, P, nullptr, gf, fine, n, N,
+  k_prolong<T, cplx<T>><<<grid, 128, 0, st>>>(out, in, P, nullptr, gf, fine, n, N,
                                                                        out_rstride, in_rstride, pstride, accumulate);
 }
 
