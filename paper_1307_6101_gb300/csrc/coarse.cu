@@ -5,6 +5,8 @@
 // 5..8 backward, so that the threads computing consecutive rows of one site
 // read consecutive words.
 #include <atomic>
+#include <mutex>
+
 #include <cooperative_groups.h>
 
 #include "common.cuh"
@@ -535,24 +537,460 @@ __global__ void __launch_bounds__(768, 2) k_coarse_sap_cluster(cplx<T>* __restri
 }
 
 // ---------------------------------------------------------------------------
-// Persistent coarse SAP: all `iters` SAP applications (a red then a black sweep each) of one
-// smoother call in one launch, for levels whose SAP blocks of both colours are resident at once.
-// Cluster c owns red block blocks0[c] and black block blocks1[c]; each CTA stages the blocks
-// inside both SAP blocks of its sites once, for the whole call.  A colour sweep is the sweep of
-// k_coarse_sap_cluster (same arithmetic, same order); sweeps are separated by a barrier over all
-// clusters, which the cooperative launch makes safe (all CTAs co-resident).  z is read through
-// L2 (ld.global.cg): values written by other SMs in the previous sweep are never taken from a
-// stale L1 line.
+// Coarse SAP on FP16 blocks (FP32 compute): one thread-block cluster per SAP block as above.  A warp forms RPL rows of a
+// site, its lanes each every 32nd column of the site's concatenated blocks, RB right-hand sides at a time (a block
+// entry is read and widened once for them, and they share the barriers).
+//
+// What bounds it is the chain of one MR step, about 2.5 us: matrix-vector product, exchange, sums, update.  So a column
+// of RPL rows is one load of the blocks and one of the vector for 4 RPL RB FMAs; the lanes share the sums out as they
+// fold them; a CTA keeps r on its own sites and their neighbours in the SAP block only, so p goes to the few CTAs that
+// own those, and the CTAs' partial dot products to all, by asynchronous stores that complete on the target's
+// mbarrier (a cluster barrier in their place waits for every store to be acknowledged: 25 against 31 us per
+// sweep).  The blocks inside the SAP block are staged before the launch waits for the previous sweep, first in
+// slot order, so that an MR step runs through one contiguous matrix; the others are read from L2 for rho.
+// ddamg_smooth on level 1 of 16^3x32 (4^3x8 sites, 40 dof, 2^4 blocks), 10 sweeps of 4 MR steps: 252 us for one
+// right-hand side and 1590 for twelve, where one thread per (row, block), partial rows through shared memory
+// and cluster barriers took 342 and 3103.
 
 // z in L2 only (values written by other CTAs of the launch)
 __device__ __forceinline__ cplx<float> ldz(const cplx<float>* p) {
   const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
   return cmk<float>(v.x, v.y);
 }
-__device__ __forceinline__ cplx<double> ldz(const cplx<double>* p) {
-  const double2 v = __ldcg(reinterpret_cast<const double2*>(p));
-  return cmk<double>(v.x, v.y);
+
+struct SapHSmem {
+  size_t zn, rf, pf, xa, zs, part, nbr, kof, nin, sc, voff, uoff, nu, pairs, np, flag, bar, total;
+};
+// nstage: staged blocks of the CTA; nblk: SAP blocks whose tables it keeps
+DD_HD SapHSmem saph_smem_layout(int vB, int n, int spc, int RB, int nstage, int nblk) {
+  SapHSmem L;
+  const size_t cs = sizeof(cplx<float>);
+  size_t o = al16((size_t)nstage * n * n * sizeof(__half2));
+  // the neighbours' z are read for rho only, which r takes the place of
+  L.zn = L.rf = o;
+  o = al16(o + (size_t)RB * n * cs * (9 * spc > vB ? 9 * spc : vB));
+  L.pf = o;
+  o = al16(o + (size_t)2 * RB * vB * n * cs);
+  L.xa = o;
+  o = al16(o + (size_t)RB * spc * n * cs);
+  L.zs = o;
+  o = al16(o + (size_t)RB * spc * n * cs);
+  L.part = o;  // [2][16][RB] dot products of the CTAs
+  o = al16(o + (size_t)2 * 16 * RB * sizeof(float4));
+  L.nbr = o;   // [nblk][spc][9] sites by slot
+  o = al16(o + (size_t)nblk * spc * 9 * sizeof(int));
+  L.kof = o;   // [nblk][spc][9] block index k of a slot
+  o = al16(o + (size_t)nblk * spc * 9 * sizeof(int));
+  L.nin = o;   // [nblk][spc] slots inside the SAP block
+  o = al16(o + (size_t)nblk * spc * sizeof(int));
+  L.sc = o;    // [nblk][spc] scales of the sites' blocks
+  o = al16(o + (size_t)nblk * spc * sizeof(float));
+  L.voff = o;  // [nblk][spc][9 n] position in r of a column inside the SAP block
+  o = al16(o + (size_t)nblk * spc * 9 * n * sizeof(short));
+  L.uoff = o;  // [nblk][9 spc] sites whose r the CTA keeps (positions in the SAP block): its own, then neighbours
+  o = al16(o + (size_t)nblk * 9 * spc * sizeof(short));
+  L.nu = o;    // [nblk] their number
+  o = al16(o + (size_t)nblk * sizeof(int));
+  L.pairs = o;   // [nblk][16 spc] (own site, other CTA that owns a neighbour of it)
+  o = al16(o + (size_t)nblk * spc * 16 * sizeof(short));
+  L.np = o;      // [nblk] their number
+  o = al16(o + (size_t)nblk * sizeof(int));
+  L.flag = o;
+  o = al16(o + 16);
+  L.bar = o;   // staged blocks; exchange buffers 0, 1
+  L.total = al16(o + 24);
+  return L;
 }
+constexpr int SAPH_W = 14;   // most warps
+// warps for `rows` rows of a CTA in groups of rpl: the fewest that share them out as evenly as SAPH_W
+DD_HD int saph_warps(int rows, int rpl) {
+  const int groups = rows / rpl, per = (groups + SAPH_W - 1) / SAPH_W;
+  return (groups + per - 1) / per;
+}
+// rows of a warp (n is even).  Eight rows: two lanes per column with four rows each, so that the eight lanes of a
+// 16-byte load hit all banks at an odd multiple of eight dofs (lanes of 32 different columns: half of them)
+DD_HD int saph_rpl(int n) { return n % 8 == 0 ? 8 : n % 4 == 0 ? 4 : 2; }
+
+// tables of SAP block q of the CTA (own: its spc sites there): slots in k order, those inside the SAP block first.  A
+// barrier follows.
+__device__ __forceinline__ void saph_tables(const Geom& g, int n, int RB, const int* own, int spc, const int* bloc,
+                                            const float* bscale, unsigned char* smem, const SapHSmem& L, int q) {
+  int* nbr = reinterpret_cast<int*>(smem + L.nbr) + q * spc * 9;
+  int* kof = reinterpret_cast<int*>(smem + L.kof) + q * spc * 9;
+  int* nin = reinterpret_cast<int*>(smem + L.nin) + q * spc;
+  short* voff = reinterpret_cast<short*>(smem + L.voff) + (size_t)q * spc * 9 * n;
+  // one lane per (site, k): whether its hop stays inside, then its slot by the ranks of the inside ones
+  for (int sl = threadIdx.x >> 5; sl < spc; sl += blockDim.x >> 5) {
+    const int k = threadIdx.x & 31;
+    int nb = own[sl], loc = -1;
+    if (k < 9) {
+      bool in = true;
+      if (k > 0) {
+        int c[4];
+        geom_coords(g, nb, c);
+        const int mu = (k - 1) & 3, dir = k <= 4 ? +1 : -1;
+        in = hop_internal(g, c, mu, dir, g.fB);
+        nb = geom_neighbor(g, c, mu, dir);
+      }
+      if (in) loc = bloc[nb];
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, k < 9 && loc >= 0);
+    const int ins = __popc(m), before = __popc(m & ((1u << k) - 1));
+    if (k == 0) {
+      nin[sl] = ins;
+      reinterpret_cast<float*>(smem + L.sc)[q * spc + sl] = bscale[own[sl]];
+    }
+    if (k < 9) {
+      const int slot = loc >= 0 ? before : ins + k - before;
+      nbr[sl * 9 + slot] = nb;
+      kof[sl * 9 + slot] = k;
+    }
+    for (int s = 0; s < ins; ++s) {   // the lane of slot s is the s-th that is inside
+      const int at = __shfl_sync(0xffffffffu, loc, __fns(m, 0, s + 1)) * n * RB;
+      for (int j = k; j < n; j += 32) voff[(sl * 9 + s) * n + j] = (short)(at + j);
+    }
+  }
+}
+
+// by one thread, a barrier after saph_tables and one before saph_block's exchanges: the sites whose r the CTA keeps (its
+// own, then every other site that one of them has inside the block, once) and the CTAs its sites go to
+__device__ __forceinline__ void saph_links(int n, int RB, int spc, int rank, unsigned char* smem, const SapHSmem& L, int q) {
+  const int* nin = reinterpret_cast<const int*>(smem + L.nin) + q * spc;
+  const short* voff = reinterpret_cast<const short*>(smem + L.voff) + (size_t)q * spc * 9 * n;
+  short* u = reinterpret_cast<short*>(smem + L.uoff) + q * 9 * spc;
+  short* pairs = reinterpret_cast<short*>(smem + L.pairs) + q * spc * 16;
+  int cnt = 0, np = 0;
+  for (int sl = 0; sl < spc; ++sl) u[cnt++] = (short)(rank * spc + sl);
+  for (int sl = 0; sl < spc; ++sl) {
+    unsigned to = 1u << rank;
+    for (int m = 1; m < nin[sl]; ++m) {
+      const int loc = voff[(sl * 9 + m) * n] / (n * RB);
+      bool seen = false;
+      for (int e = 0; e < cnt; ++e) seen = seen || u[e] == loc;
+      if (!seen) u[cnt++] = (short)loc;
+      const int t = loc / spc;
+      if (!(to >> t & 1u)) pairs[np++] = (short)(sl << 8 | t);
+      to |= 1u << t;
+    }
+  }
+  reinterpret_cast<int*>(smem + L.nu)[q] = cnt;
+  reinterpret_cast<int*>(smem + L.np)[q] = np;
+}
+
+// v[0 .. NV) summed over the lanes of the warp that are equal modulo M (1 or 2), which share the values out as they fold
+// them: lane l returns value (l / M) / (32 / M / NV)
+template <int NV, int M>
+__device__ __forceinline__ float warp_fold(float (&v)[NV], int lane) {
+  int off = 16;
+#pragma unroll
+  for (int w = NV / 2; w >= 1; w >>= 1, off >>= 1) {
+    const bool up = (lane & off) != 0;
+#pragma unroll
+    for (int k = 0; k < w; ++k) {
+      const float keep = up ? v[k + w] : v[k], send = up ? v[k] : v[k + w];
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+    }
+  }
+  for (; off >= M; off >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+  return v[0];
+}
+
+// RPL neighbouring rows of a column
+template <int RPL>
+struct HalfRows {
+  unsigned w[RPL];
+  __device__ __forceinline__ void load(const __half2* p) {
+    if constexpr (RPL == 2) {
+      *reinterpret_cast<uint2*>(w) = *reinterpret_cast<const uint2*>(p);
+    } else {
+#pragma unroll
+      for (int r = 0; r < RPL; r += 4) {
+        const uint4 v = *reinterpret_cast<const uint4*>(p + r);
+        w[r] = v.x;
+        w[r + 1] = v.y;
+        w[r + 2] = v.z;
+        w[r + 3] = v.w;
+      }
+    }
+  }
+};
+
+// One SAP block (table q of the CTA), right-hand sides rh0 .. rh0 + nb - 1 (nb <= RB): rho = (b - D z)_B, k MR steps,
+// z_B += e_B.  seq: exchanges of the CTA so far (their parity picks the buffer).  stage: [spc][nst slots][n][n] in
+// shared memory (every slot inside the SAP block is staged); ext(sl, slot): a block that is not; staged(): a barrier
+// that waits for the staged blocks; false: they did not arrive, z is not written.
+template <int RB, int RPL, bool L2Z, class Ext, class Staged>
+__device__ __forceinline__ void saph_block(cg::cluster_group& cluster, cplx<float>* z, const cplx<float>* bsrc,
+                                           int vB, int n, FDiv fn, size_t rstride, int rh0, int nb, int k_mr,
+                                           int spc, const int* own, unsigned char* smem, const SapHSmem& L, int q, unsigned& seq,
+                                           int* err, const __half2* stage, int nst, Ext ext, Staged staged) {
+  using C = cplx<float>;
+  constexpr int M = RPL == 8 ? 2 : 1, RL = RPL / M;   // lanes per column, rows of a lane
+  using HR = HalfRows<RL>;
+  constexpr int NV = 2 * RL * RB;                     // sums of a lane's rows: [right-hand side][row][re, im]
+  C* zn = reinterpret_cast<C*>(smem + L.zn);             // [RB][spc][9 n] z of the own sites and neighbours (rho)
+  // vectors on the SAP block, [vB][RB][n]; only the own sites and their neighbours in the block are kept up to date
+  C* rf = reinterpret_cast<C*>(smem + L.rf);             // residual
+  C* pf = reinterpret_cast<C*>(smem + L.pf);             // [2] exchanged vectors: r, then p
+  unsigned long long* xbar = reinterpret_cast<unsigned long long*>(smem + L.bar) + 1;   // [2]
+  C* xa = reinterpret_cast<C*>(smem + L.xa);             // [RB][rows] correction of the own rows
+  C* zs = reinterpret_cast<C*>(smem + L.zs);             // [RB][rows] z of the own rows
+  float4* part = reinterpret_cast<float4*>(smem + L.part);   // [2][16][RB]
+  const short* us = reinterpret_cast<const short*>(smem + L.uoff) + q * 9 * spc;
+  const int* nbr = reinterpret_cast<const int*>(smem + L.nbr) + q * spc * 9;
+  const int* nin = reinterpret_cast<const int*>(smem + L.nin) + q * spc;
+  const float* sc = reinterpret_cast<const float*>(smem + L.sc) + q * spc;
+  const short* voff = reinterpret_cast<const short*>(smem + L.voff) + (size_t)q * spc * 9 * n;
+  const int CLS = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nth >> 5;
+  const int rows = spc * n, N = vB * n, nn = n * n, zst = spc * 9 * n;
+  for (int e0 = tid; e0 < RB * zst; e0 += 4 * nth) {   // four loads in flight per thread
+    C v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = e0 + u * nth, t = fdiv(e, fn), rr = RB == 1 ? 0 : t / (9 * spc);
+      v[u] = czero<float>();
+      if (e < RB * zst && rr < nb) {
+        const C* pz = z + (size_t)(rh0 + rr) * rstride + (size_t)nbr[t - rr * 9 * spc] * n + (e - t * n);
+        v[u] = L2Z ? ldz(pz) : *pz;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (e0 + u * nth < RB * zst) zn[e0 + u * nth] = v[u];
+  }
+  bool ok = staged();
+  const int nu = reinterpret_cast<const int*>(smem + L.nu)[q];
+  const int npair = reinterpret_cast<const int*>(smem + L.np)[q];
+  const short* pairs = reinterpret_cast<const short*>(smem + L.pairs) + q * spc * 16;
+  // acc += column `h` of RPL rows times v
+  auto column = [&](float (&acc)[NV], const HR& h, const C (&v)[RB]) {
+#pragma unroll
+    for (int r = 0; r < RL; ++r) {
+      const float2 m = __half22float2(*reinterpret_cast<const __half2*>(&h.w[r]));
+#pragma unroll
+      for (int rr = 0; rr < RB; ++rr) {
+        float& re = acc[(rr * RL + r) * 2];
+        float& im = acc[(rr * RL + r) * 2 + 1];
+        re = fmaf(m.x, v[rr].re, re);
+        re = fmaf(-m.y, v[rr].im, re);
+        im = fmaf(m.x, v[rr].im, im);
+        im = fmaf(m.y, v[rr].re, im);
+      }
+    }
+  };
+  // lane -> (right-hand side, row of the group, re / im) of the value it holds after the fold
+  constexpr int LPV = 32 / M / NV;
+  const int vi = lane / M / LPV, v_rr = vi / (2 * RL), v_row = lane % M * RL + vi / 2 % RL, v_c = vi & 1;
+  const bool v_on = lane / M % LPV == 0;
+  const int c0 = lane / M, r0 = lane % M * RL;   // first column and row of the lane
+  // The own sites of d (an exchange buffer) to the CTAs that own their neighbours in the block, whose sites come back
+  // (adjacency is symmetric), a warp's asynchronous stores per site and CTA; and with dots the own rows' <d, r>, |d|^2 to every CTA.
+  // Everything completes on the target's barrier, so that nobody waits for more than the data.  A buffer is free again
+  // two exchanges later: a CTA sends the next vector but one only after every CTA's next dot products have come.
+  auto exchange = [&](C* d, bool dots) {
+    const unsigned buf = seq & 1, parity = (seq >> 1) & 1;
+    ++seq;
+    __syncthreads();
+    if (tid == 0)
+      mbar_arrive_expect_tx(&xbar[buf], (unsigned)((nu - spc) * RB * n * sizeof(C) + CLS * RB * sizeof(float4)));
+    for (int p = warp; p < npair; p += nw) {
+      const int sl = pairs[p] >> 8, t = pairs[p] & 255;
+      float4* o = reinterpret_cast<float4*>(d + (size_t)(rank * spc + sl) * RB * n);
+      for (int e = lane; e < RB * n / 2; e += 32) st_async_cluster(o + e, o[e], &xbar[buf], t);
+    }
+    for (int rr = nw > 1 ? warp - 1 : 0; rr >= 0 && rr < RB; rr += nw > 1 ? nw - 1 : 1) {   // a warp per right-hand side
+      float v[4] = {0.f, 0.f, 0.f, 0.f};
+      if (dots)
+        for (int e = lane; e < rows; e += 32) {
+          const int so = e / n, o = ((rank * spc + so) * RB + rr) * n + (e - so * n);
+          cdotc_acc(v[0], v[1], d[o], rf[o]);
+          cnorm2_acc(v[2], d[o]);
+        }
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+        for (int off = 16; off >= 1; off >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], off);
+      if (lane < CLS)
+        st_async_cluster(&part[(buf * 16 + rank) * RB + rr], make_float4(v[0], v[1], v[2], 0.f), &xbar[buf], lane);
+    }
+    if (!mbar_wait_bounded(&xbar[buf], parity)) {
+      ok = false;
+      atomicExch(err, 2);
+    }
+    return (const float4*)part + buf * 16 * RB;
+  };
+  auto buffer = [&] { return pf + (size_t)(seq & 1) * RB * N; };
+  C* px = buffer();
+  for (int g0 = warp; g0 < rows / RPL; g0 += nw) {
+    const int row0 = g0 * RPL, sl = row0 / n, i0 = row0 - sl * n;
+    float acc[NV];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) acc[k] = 0.f;
+    const C* vz = zn + sl * 9 * n;
+    const __half2* A = stage + sl * nst * nn + i0 + r0;
+    int c = c0;
+#pragma unroll 4
+    for (; c < nst * n; c += 32 / M) {
+      C v[RB];
+#pragma unroll
+      for (int rr = 0; rr < RB; ++rr) v[rr] = vz[rr * zst + c];
+      HR h;
+      h.load(A + c * n);
+      column(acc, h, v);
+    }
+#pragma unroll 5
+    for (; c < 9 * n; c += 32 / M) {
+      const int slot = c / n;
+      HR h;
+      h.load(ext(sl, slot) + (c - slot * n) * n + i0 + r0);
+      C v[RB];
+#pragma unroll
+      for (int rr = 0; rr < RB; ++rr) v[rr] = vz[rr * zst + c];
+      column(acc, h, v);
+    }
+    const float s = warp_fold<NV, M>(acc, lane);
+    if (v_on) {
+      const int i = i0 + v_row, row = row0 + v_row;
+      const float b = v_rr < nb ? reinterpret_cast<const float*>(bsrc + (size_t)(rh0 + v_rr) * rstride +
+                                                                 (size_t)own[sl] * n + i)[v_c] : 0.f;
+      reinterpret_cast<float*>(px + ((rank * spc + sl) * RB + v_rr) * n + i)[v_c] = b - sc[sl] * s;
+      reinterpret_cast<float*>(zs + v_rr * rows + row)[v_c] =
+          reinterpret_cast<const float*>(vz + v_rr * zst + i)[v_c];                       // slot 0 is the site itself
+    }
+  }
+  for (int e = tid; e < RB * rows; e += nth) xa[e] = czero<float>();
+  exchange(px, false);
+  for (int t = warp; t < nu * RB; t += nw) {   // r at the kept sites; every warp is past rho (the exchange's barrier)
+    const int at = (us[t / RB] * RB + t % RB) * n;
+    for (int j = lane; j < n; j += 32) rf[at + j] = px[at + j];
+  }
+  __syncthreads();
+  for (int it = 0; it < k_mr; ++it) {
+    C* pb = buffer();
+    for (int g0 = warp; g0 < rows / RPL; g0 += nw) {
+      const int row0 = g0 * RPL, sl = row0 / n, i0 = row0 - sl * n;
+      float acc[NV];
+#pragma unroll
+      for (int k = 0; k < NV; ++k) acc[k] = 0.f;
+      const short* vo = voff + sl * 9 * n;
+      const int nc = nin[sl] * n;
+      const __half2* A = stage + sl * nst * nn + i0 + r0;
+#pragma unroll 4
+      for (int c = c0; c < nc; c += 32 / M) {
+        const int o = vo[c];
+        C v[RB];
+#pragma unroll
+        for (int rr = 0; rr < RB; ++rr) v[rr] = rf[rr * n + o];
+        HR h;
+        h.load(A + c * n);
+        column(acc, h, v);
+      }
+      const float s = warp_fold<NV, M>(acc, lane);
+      if (v_on)
+        reinterpret_cast<float*>(pb + ((rank * spc + sl) * RB + v_rr) * n + i0 + v_row)[v_c] = sc[sl] * s;
+    }
+    const float4* dp = exchange(pb, true);
+    // alpha from the CTAs' partial sums in rank order (the same in every CTA), then r on the kept sites
+    C alpha[RB];
+#pragma unroll
+    for (int rr = 0; rr < RB; ++rr) {
+      float re = 0.f, im = 0.f, den = 0.f;
+#pragma unroll
+      for (int c = 0; c < 16; ++c)
+        if (c < CLS) {
+          const float4 t = dp[c * RB + rr];
+          re += t.x;
+          im += t.y;
+          den += t.z;
+        }
+      alpha[rr] = den > 0.f ? cmk<float>(re / den, im / den) : czero<float>();
+    }
+    for (int t = warp; t < nu * RB; t += nw) {
+      const int s = t / RB, rr = t - s * RB, at = (us[s] * RB + rr) * n;
+      C al = alpha[0];
+#pragma unroll
+      for (int k = 1; k < RB; ++k)
+        if (rr == k) al = alpha[k];
+      for (int j = lane; j < n; j += 32) {
+        const C r = rf[at + j];
+        if (s < spc) cfma(xa[rr * rows + s * n + j], al, r);
+        rf[at + j] = r - al * pb[at + j];
+      }
+    }
+    __syncthreads();
+  }
+  if (__syncthreads_and(ok ? 1 : 0))   // and before the next right-hand sides' z take the place of r
+    for (int e = tid; e < nb * rows; e += nth) {
+      const int rr = e / rows, o = e - rr * rows, so = o / n;
+      z[(size_t)(rh0 + rr) * rstride + (size_t)own[so] * n + (o - so * n)] = zs[e] + xa[e];
+    }
+  __syncthreads();   // zs and xa are free
+}
+
+// one colour sweep: cluster c of the launch owns SAP block blocks[c]
+template <int RB, int RPL>
+__global__ void __launch_bounds__(32 * SAPH_W, 2) k_coarse_sap_h(cplx<float>* __restrict__ z,
+                                                                 const cplx<float>* __restrict__ bsrc,
+                                                                 const __half2* __restrict__ blk,
+                                                                 const float* __restrict__ bscale, Geom g, int n,
+                                                                 FDiv fn, size_t rstride, int nrhs,
+                                                                 const int* __restrict__ blocks, int k_mr, int spc,
+                                                                 int nst, int* err, const int* __restrict__ bsite,
+                                                                 const int* __restrict__ bloc) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  // the next sweep (launched with programmatic stream serialization) may stage its blocks while
+  // this one runs; it waits for this grid before reading z or b
+  pdl_launch_dependents();
+  cg::cluster_group cluster = cg::this_cluster();
+  const int CLS = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const SapHSmem L = saph_smem_layout(g.vB, n, spc, RB, nst * spc, 1);
+  const __half2* stage = reinterpret_cast<const __half2*>(smem_raw);   // [spc][nst slots][n][n]
+  const int* kof = reinterpret_cast<const int*>(smem_raw + L.kof);
+  unsigned long long* bar = reinterpret_cast<unsigned long long*>(smem_raw + L.bar);
+  const int* own = bsite + (size_t)blocks[blockIdx.x / CLS] * g.vB + rank * spc;
+  const int nn = n * n;
+  if (threadIdx.x < 3) mbar_init(bar + threadIdx.x, 1);
+  saph_tables(g, n, RB, own, spc, bloc, bscale, smem_raw, L, 0);
+  cluster.sync();   // every CTA's exchange barriers are set up
+  if (threadIdx.x < 32) {
+    if (threadIdx.x == 0) mbar_arrive_expect_tx(bar, (unsigned)(spc * nst * nn * sizeof(__half2)));
+    __syncwarp();
+    for (int e = threadIdx.x; e < spc * nst; e += 32) {
+      const int sl = e / nst;
+      bulk_g2s(smem_raw + (size_t)e * nn * sizeof(__half2), blk + ((size_t)own[sl] * 9 + kof[sl * 9 + e - sl * nst]) * nn,
+               (unsigned)(nn * sizeof(__half2)), bar);
+    }
+  }
+  if (threadIdx.x == blockDim.x - 1) saph_links(n, RB, spc, rank, smem_raw, L, 0);
+  pdl_wait();   // the previous kernel's z and b are complete from here on
+  int ok = 1;
+  unsigned seq = 0;
+  for (int rh0 = 0; rh0 < nrhs; rh0 += RB)
+    saph_block<RB, RPL, false>(
+        cluster, z, bsrc, g.vB, n, fn, rstride, rh0, min(RB, nrhs - rh0), k_mr, spc, own, smem_raw, L, 0, seq, err,
+        stage, nst, [&](int sl, int slot) { return blk + ((size_t)own[sl] * 9 + kof[sl * 9 + slot]) * nn; },
+        [&] {
+          if (rh0 == 0) {
+            ok = __syncthreads_and(mbar_wait_bounded(bar, 0) ? 1 : 0);
+            if (!ok && threadIdx.x == 0) atomicExch(err, 2);
+          } else {
+            __syncthreads();
+          }
+          return ok != 0;
+        });
+  if (!ok && threadIdx.x == 0) mbar_wait_bounded(bar, 0);   // no copy may still be in flight at exit
+  cluster.sync();   // no CTA leaves while its last copies to others may still be read
+}
+
+// ---------------------------------------------------------------------------
+// Persistent coarse SAP: all `iters` SAP applications (a red then a black sweep each) of one
+// smoother call in one launch, for levels whose SAP blocks of both colours are resident at once.
+// Cluster c owns nbpc red and nbpc black blocks; each CTA stages the blocks inside those SAP blocks of its
+// sites once, for the whole call, and reads the others (hops leaving the block, for rho only) from L2.  A
+// block is done by saph_block (same arithmetic, same order as a launch per sweep); sweeps are separated
+// by a barrier over all clusters, which the cooperative launch makes safe (all CTAs co-resident).  z is
+// read through L2 (ld.global.cg): values written by other SMs in the previous sweep are never taken from
+// a stale L1 line.
 
 __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p) {
   unsigned v;
@@ -585,40 +1023,12 @@ __device__ bool persist_grid_sync(unsigned* cnt, unsigned target, cg::cluster_gr
   return *cluster.map_shared_rank(flag, 0) != 0;
 }
 
-struct PSapSmem {
-  size_t rfull, pbuf, part, red, sh, slot, flag, bar, total;
-};
-// nbpc SAP blocks of each colour per cluster; rows = nbpc * spc * n per CTA
-DD_HD PSapSmem psap_smem_layout(int vB, int n, int spc, int nsl, int nbpc, size_t bs, size_t ts) {
-  PSapSmem L;
-  size_t o = al16((size_t)2 * nbpc * spc * nsl * n * n * bs);
-  L.rfull = o;
-  o = al16(o + (size_t)nbpc * vB * n * 2 * ts);
-  L.pbuf = o;
-  o = al16(o + (size_t)2 * nbpc * vB * n * 2 * ts);
-  L.part = o;
-  o = al16(o + (size_t)9 * nbpc * spc * n * 2 * ts);
-  L.red = o;
-  o = al16(o + (size_t)2 * nbpc * 16 * 4 * ts);
-  L.sh = o;
-  o = al16(o + (size_t)(32 * 3 * nbpc + 4) * ts);
-  L.slot = o;
-  o = al16(o + (size_t)2 * nbpc * spc * 9 * sizeof(int));
-  L.flag = o;
-  o = al16(o + 16);
-  L.bar = o;
-  L.total = al16(o + 8);
-  return L;
-}
-
-// NB SAP blocks of each colour per cluster (1 or 2): CTA rank q owns sites q*spc .. q*spc+spc-1
-// of each of them; the rows of block j are rows j*spc*n .. (j+1)*spc*n-1 of the CTA, with their
-// own residual copy, MR direction and dot products.
-template <typename T, typename BS, int NB>
-__global__ void __launch_bounds__(768, 1) k_coarse_sap_persist(
-    cplx<T>* __restrict__ z, const cplx<T>* __restrict__ bsrc, const BS* __restrict__ blk,
-    const float* __restrict__ bscale, Geom g, int n, size_t rstride, int nrhs, const int* __restrict__ blocks0,
-    int nb0, const int* __restrict__ blocks1, int nb1, int k_mr, int spc, int nsl, int iters, int* err,
+template <int RPL>
+__global__ void __launch_bounds__(32 * SAPH_W, 1) k_coarse_sap_persist(
+    cplx<float>* __restrict__ z, const cplx<float>* __restrict__ bsrc, const __half2* __restrict__ blk,
+    const float* __restrict__ bscale, Geom g, int n, FDiv fn, size_t rstride, int nrhs,
+    const int* __restrict__ blocks0, int nb0, const int* __restrict__ blocks1, int nb1, int k_mr, int spc, int nsl,
+    int nbpc, int iters, int* err,
     const int* __restrict__ bsite, const int* __restrict__ bloc, unsigned* gcnt) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   cg::cluster_group cluster = cg::this_cluster();
@@ -626,217 +1036,56 @@ __global__ void __launch_bounds__(768, 1) k_coarse_sap_persist(
   const int rank = (int)cluster.block_rank();
   const int cid = blockIdx.x / CLS;
   const unsigned ncl = gridDim.x / CLS;
-  const int vB = g.vB;
-  const int rb = spc * n;          // rows of one block in this CTA
-  const int rows = NB * rb;
-  const size_t nn = (size_t)n * n;
-  const PSapSmem L = psap_smem_layout(vB, n, spc, nsl, NB, sizeof(BS), sizeof(T));
-  BS* stage = reinterpret_cast<BS*>(smem_raw);                                // [2][NB*spc][nsl][n][n]
-  cplx<T>* rfull = reinterpret_cast<cplx<T>*>(smem_raw + L.rfull);            // [NB][vB*n]
-  cplx<T>* pbuf = reinterpret_cast<cplx<T>*>(smem_raw + L.pbuf);              // [2][NB][vB*n]
-  cplx<T>* part = reinterpret_cast<cplx<T>*>(smem_raw + L.part);              // [9][rows]
-  T* red = reinterpret_cast<T*>(smem_raw + L.red);                            // [2][NB][16][4]
-  T* sh = reinterpret_cast<T*>(smem_raw + L.sh);                              // [32][3*NB] + 4
-  int* slot = reinterpret_cast<int*>(smem_raw + L.slot);                      // [2][NB*spc][9]
+  const int vB = g.vB, nn = n * n;
+  const SapHSmem L = saph_smem_layout(vB, n, spc, 1, 2 * nbpc * spc * nsl, 2 * nbpc);
+  __half2* stage = reinterpret_cast<__half2*>(smem_raw);   // [2][nbpc][spc][nsl slots][n][n]
+  const int* kof = reinterpret_cast<const int*>(smem_raw + L.kof);   // [2 nbpc][spc][9]
   int* flag = reinterpret_cast<int*>(smem_raw + L.flag);
   unsigned long long* bar = reinterpret_cast<unsigned long long*>(smem_raw + L.bar);
-  // block of colour c, slot j of this cluster (-1: none)
-  auto block_of = [&](int c, int j) -> int {
-    const int q = cid * NB + j;
-    return c ? (q < nb1 ? blocks1[q] : -1) : (q < nb0 ? blocks0[q] : -1);
+  // the own sites of block j of colour c (null: the cluster has none)
+  auto own_of = [&](int c, int j) -> const int* {
+    const int q = cid * nbpc + j;
+    if (q >= (c ? nb1 : nb0)) return nullptr;
+    return bsite + (size_t)(c ? blocks1 : blocks0)[q] * vB + rank * spc;
   };
-  // slots of the staged blocks (k order: self, forward mu, backward mu)
-  if (threadIdx.x < 2 * NB * spc) {
-    const int c = threadIdx.x / (NB * spc), js = threadIdx.x - c * NB * spc;
-    const int j = js / spc, s = js - j * spc;
-    int* sl9 = slot + (c * NB * spc + js) * 9;
-    const int bc = block_of(c, j);
-    if (bc >= 0) {
-      int co[4];
-      geom_coords(g, bsite[(size_t)bc * vB + rank * spc + s], co);
-      int ns = 0;
-      sl9[0] = ns++;
-      for (int sd = 0; sd < 2; ++sd)
-        for (int mu = 0; mu < 4; ++mu)
-          sl9[(sd ? 5 : 1) + mu] = hop_internal(g, co, mu, sd ? -1 : +1, g.fB) ? ns++ : -1;
-    } else {
-      for (int e = 0; e < 9; ++e) sl9[e] = -1;
-    }
-  }
-  if (threadIdx.x == 0) mbar_init(bar, 1);
-  __syncthreads();
-  if (threadIdx.x < 32) {
+  for (int cj = 0; cj < 2 * nbpc; ++cj)
+    if (const int* own = own_of(cj / nbpc, cj % nbpc)) saph_tables(g, n, 1, own, spc, bloc, bscale, smem_raw, L, cj);
+  if (threadIdx.x < 3) mbar_init(bar + threadIdx.x, 1);
+  cluster.sync();   // every CTA's exchange barriers are set up
+  if (threadIdx.x == blockDim.x - 1)
+    for (int cj = 0; cj < 2 * nbpc; ++cj)
+      if (own_of(cj / nbpc, cj % nbpc)) saph_links(n, 1, spc, rank, smem_raw, L, cj);
+  if (threadIdx.x == 0) {   // nsl slots of every site: those inside the SAP block, then others up to that number
     int cnt = 0;
-    for (int e = 0; e < 2 * NB * spc * 9; ++e) cnt += slot[e] >= 0 ? 1 : 0;
-    if (threadIdx.x == 0) mbar_arrive_expect_tx(bar, (unsigned)(cnt * nn * sizeof(BS)));
-    __syncwarp();
-    for (int e = threadIdx.x; e < 2 * NB * spc * 9; e += 32) {
-      const int cjs = e / 9, k = e % 9, q = slot[e];   // cjs = (c * NB + j) * spc + s
-      if (q >= 0) {
-        const int c = cjs / (NB * spc), js = cjs - c * NB * spc;
-        const int j = js / spc, s = js - j * spc;
-        const int site = bsite[(size_t)block_of(c, j) * vB + rank * spc + s];
-        bulk_g2s(stage + ((size_t)cjs * nsl + q) * nn, blk + ((size_t)site * 9 + k) * nn,
-                 (unsigned)(nn * sizeof(BS)), bar);
-      }
-    }
+    for (int cj = 0; cj < 2 * nbpc; ++cj) cnt += own_of(cj / nbpc, cj % nbpc) ? spc * nsl : 0;
+    mbar_arrive_expect_tx(bar, (unsigned)(cnt * nn * sizeof(__half2)));
+    for (int cj = 0; cj < 2 * nbpc; ++cj)
+      if (const int* own = own_of(cj / nbpc, cj % nbpc))
+        for (int sl = 0; sl < spc; ++sl)
+          for (int e = 0; e < nsl; ++e)
+            bulk_g2s(stage + ((size_t)(cj * spc + sl) * nsl + e) * nn,
+                     blk + ((size_t)own[sl] * 9 + kof[(cj * spc + sl) * 9 + e]) * nn, (unsigned)(nn * sizeof(__half2)),
+                     bar);
   }
   const int ok = __syncthreads_and(mbar_wait_bounded(bar, 0) ? 1 : 0);
   if (!ok && threadIdx.x == 0) atomicExch(err, 2);
-  const int k = threadIdx.x / rows;
-  const int rl = threadIdx.x - k * rows;
-  const int jb = rl / rb, rj = rl - jb * rb;      // block of the row, row inside that block's share
-  const int sl = rj / n, i = rj - (rj / n) * n;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-  // the rows this thread owns as a residual row (threadIdx.x < rows): block jr, local row rr
-  const int jr = threadIdx.x / rb, rr = threadIdx.x - (threadIdx.x / rb) * rb;
-  unsigned round = 0;
+  unsigned round = 0, seq = 0;
   bool alive = true;
   for (int it = 0; it < iters && alive; ++it)
     for (int c = 0; c < 2 && alive; ++c) {
-      const int bk = k < 9 ? block_of(c, jb) : -1;            // this thread's (row, k) block
-      const int bres = threadIdx.x < rows ? block_of(c, jr) : -1;   // this thread's residual row's block
-      const bool any = block_of(c, 0) >= 0;                    // uniform over the cluster
-      if (any) {
-        int site = 0, q = -1, nb = 0, nloc = 0;
-        T sc = T(1);
-        if (bk >= 0) {
-          site = bsite[(size_t)bk * vB + rank * spc + sl];
-          sc = bscale ? T(bscale[site]) : T(1);
-          nb = site;
-          q = slot[((c * NB + jb) * spc + sl) * 9 + k];
-          if (k > 0) {
-            int co[4];
-            geom_coords(g, site, co);
-            nb = geom_neighbor(g, co, (k - 1) % 4, k <= 4 ? +1 : -1);
-          }
-          nloc = q >= 0 ? bloc[nb] : 0;
-        }
-        const BS* Ms = stage + ((size_t)((c * NB + jb) * spc + sl) * nsl + (q >= 0 ? q : 0)) * nn + i;
-        const int* ownr = bres >= 0 ? bsite + (size_t)bres * vB + rank * spc : nullptr;
-        for (int rh = 0; rh < nrhs; ++rh) {
-          const size_t ro = (size_t)rh * rstride;
-          // rho = b - D z on the own rows (z through L2)
-          if (k < 9) {
-            cplx<T> acc = czero<T>();
-            if (bk >= 0) {
-              const cplx<T>* v = z + ro + (size_t)nb * n;
-              if (q < 0) {
-                const BS* M = blk + ((size_t)site * 9 + k) * nn + i;
-#pragma unroll 8
-                for (int j = 0; j < n; ++j) cfma(acc, ld_cplx(M, (size_t)j * n), ldz(v + j));
-              } else {
-#pragma unroll 8
-                for (int j = 0; j < n; ++j) cfma(acc, ld_cplx(Ms, (size_t)j * n), ldz(v + j));
-              }
-            }
-            part[k * rows + rl] = sc * acc;
-          }
-          __syncthreads();
-          cplx<T> r = czero<T>(), xs = czero<T>();
-          if (bres >= 0) {
-            cplx<T> d = czero<T>();
-#pragma unroll
-            for (int m = 0; m < 9; ++m) d = d + part[m * rows + threadIdx.x];
-            r = bsrc[ro + (size_t)ownr[rr / n] * n + rr % n] - d;
-            for (int cc = 0; cc < CLS; ++cc)
-              cluster.map_shared_rank(rfull + (size_t)jr * vB * n, cc)[(size_t)rank * rb + rr] = r;
-          }
-          cluster.sync();
-          for (int mr = 0; mr < k_mr; ++mr) {
-            const int buf = mr & 1;
-            cplx<T>* pb = pbuf + (size_t)buf * NB * vB * n;
-            T* rbf = red + buf * NB * 64;
-            // p = D_B r on the own rows, from the staged blocks and the local copy of r
-            if (k < 9) {
-              cplx<T> a = czero<T>();
-              if (bk >= 0 && q >= 0) {
-                const cplx<T>* v = rfull + (size_t)jb * vB * n + (size_t)nloc * n;
-#pragma unroll 8
-                for (int j = 0; j < n; ++j) cfma(a, ld_cplx(Ms, (size_t)j * n), v[j]);
-              }
-              part[k * rows + rl] = sc * a;
-            }
-            __syncthreads();
-            cplx<T> p = czero<T>();
-            T v3[3 * NB];
-#pragma unroll
-            for (int e = 0; e < 3 * NB; ++e) v3[e] = T(0);
-            if (bres >= 0) {
-#pragma unroll
-              for (int m = 0; m < 9; ++m) p = p + part[m * rows + threadIdx.x];
-              const cplx<T> t = cdotc(p, r);
-#pragma unroll
-              for (int jj = 0; jj < NB; ++jj)
-                if (jj == jr) {
-                  v3[3 * jj] = t.re;
-                  v3[3 * jj + 1] = t.im;
-                  v3[3 * jj + 2] = cnorm2(p);
-                }
-              for (int cc = 0; cc < CLS; ++cc)
-                cluster.map_shared_rank(pb + (size_t)jr * vB * n, cc)[(size_t)rank * rb + rr] = p;
-            }
-#pragma unroll
-            for (int e = 0; e < 3 * NB; ++e)
-              for (int off = 16; off >= 1; off >>= 1) v3[e] += __shfl_xor_sync(0xffffffffu, v3[e], off);
-            if (lane == 0)
-#pragma unroll
-              for (int e = 0; e < 3 * NB; ++e) sh[3 * NB * warp + e] = v3[e];
-            __syncthreads();
-            if (warp == 0) {   // warp partials summed by a shuffle tree (fixed order), sent to every CTA
-#pragma unroll
-              for (int e = 0; e < 3 * NB; ++e) {
-                T a = lane < nw ? sh[3 * NB * lane + e] : T(0);
-                for (int off = 16; off >= 1; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
-                v3[e] = a;
-              }
-              if (lane < CLS)
-#pragma unroll
-                for (int jj = 0; jj < NB; ++jj) {
-                  T* dst = cluster.map_shared_rank(rbf + jj * 64, lane) + rank * 4;
-                  dst[0] = v3[3 * jj];
-                  dst[1] = v3[3 * jj + 1];
-                  dst[2] = v3[3 * jj + 2];
-                }
-            }
-            cluster.sync();
-            cplx<T> alpha[NB];
-#pragma unroll
-            for (int jj = 0; jj < NB; ++jj) {
-              T a = T(0), bb = T(0), cc = T(0);
-              for (int q2 = 0; q2 < CLS; ++q2) {
-                a += rbf[jj * 64 + q2 * 4];
-                bb += rbf[jj * 64 + q2 * 4 + 1];
-                cc += rbf[jj * 64 + q2 * 4 + 2];
-              }
-              alpha[jj] = cc > T(0) ? cmk<T>(a / cc, bb / cc) : czero<T>();
-            }
-            if (bres >= 0) {
-              cplx<T> al = alpha[0];
-#pragma unroll
-              for (int jj = 1; jj < NB; ++jj)
-                if (jj == jr) al = alpha[jj];
-              cfma(xs, al, r);
-              r = r - al * p;
-            }
-            for (int e = threadIdx.x; e < NB * vB * n; e += blockDim.x) {
-              const int jj = e / (vB * n);
-              cplx<T> al = alpha[0];
-#pragma unroll
-              for (int j2 = 1; j2 < NB; ++j2)
-                if (j2 == jj) al = alpha[j2];
-              rfull[e] = rfull[e] - al * pb[e];
-            }
-            __syncthreads();
-          }
-          if (ok && bres >= 0) {
-            const size_t a = ro + (size_t)ownr[rr / n] * n + rr % n;
-            z[a] = ldz(z + a) + xs;
-          }
-          // every CTA is done with its copies of r, p and the partials before the next right-hand
-          // side writes into them
-          if (rh + 1 < nrhs) cluster.sync();
-        }
+      for (int j = 0; j < nbpc; ++j) {
+        const int cj = c * nbpc + j;
+        const int* own = own_of(c, j);
+        if (!own) continue;   // uniform over the cluster
+        for (int rh = 0; rh < nrhs; ++rh)
+          saph_block<1, RPL, true>(
+              cluster, z, bsrc, vB, n, fn, rstride, rh, 1, k_mr, spc, own, smem_raw, L, cj, seq, err,
+              (const __half2*)stage + (size_t)cj * spc * nsl * nn, nsl,
+              [&](int sl, int slot) { return blk + ((size_t)own[sl] * 9 + kof[(cj * spc + sl) * 9 + slot]) * nn; },
+              [&] {
+                __syncthreads();
+                return ok != 0;
+              });
       }
       if (it + 1 < iters || c == 0) {
         ++round;
@@ -1083,7 +1332,6 @@ int coarse_sap_cluster_plan(const Geom& g, int n, int* CLS_out, int* spc_out, in
     const size_t sm = sap_smem_layout(g.vB, n, spc, nsl, sizeof(cplx<T>), sizeof(T)).total;
     if (sm > 227 * 1024) continue;
     sap_cluster_attrs<T, cplx<T>>(sm, CLS);
-    if constexpr (sizeof(T) == 4) sap_cluster_attrs<float, __half2>(sm, CLS);
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1113,34 +1361,82 @@ int coarse_sap_cluster_plan(const Geom& g, int n, int* CLS_out, int* spc_out, in
 // SAP blocks of each colour per cluster, and whether all clusters (max(nb0, nb1) / nbpc of
 // op.sap_cls CTAs) can be resident at once on this device.
 size_t coarse_sap_persist_smem(const CoarseOp<float>& op, int nbpc) {
-  if (op.sap_cls <= 0) return 0;
-  const int spc = op.g.vB / op.sap_cls;
-  return psap_smem_layout(op.g.vB, op.n, spc, op.sap_nsl, nbpc, sizeof(__half2), sizeof(float)).total;
+  if (op.saph_cls <= 0) return 0;
+  const int spc = op.g.vB / op.saph_cls;
+  return saph_smem_layout(op.g.vB, op.n, spc, 1, 2 * nbpc * spc * op.sap_nsl, 2 * nbpc).total;
 }
 
 namespace {
-int persist_threads(const CoarseOp<float>& op, int nbpc) {
-  const int spc = op.g.vB / op.sap_cls;
-  return ((9 * nbpc * spc * op.n + 31) / 32) * 32;
+int saph_threads(int rows, int n) { return 32 * saph_warps(rows, saph_rpl(n)); }
+int saph_threads(const CoarseOp<float>& op) { return saph_threads(op.g.vB / op.saph_cls * op.n, op.n); }
+template <int RB>
+auto saph_kernel(int n) {
+  const int r = saph_rpl(n);
+  return r == 8 ? k_coarse_sap_h<RB, 8> : r == 4 ? k_coarse_sap_h<RB, 4> : k_coarse_sap_h<RB, 2>;
 }
-const void* persist_kernel(int nbpc) {
-  return nbpc == 2 ? (const void*)k_coarse_sap_persist<float, __half2, 2>
-                   : (const void*)k_coarse_sap_persist<float, __half2, 1>;
+auto saph_persist_kernel(const CoarseOp<float>& op) {
+  const int r = saph_rpl(op.n);
+  return r == 8 ? k_coarse_sap_persist<8> : r == 4 ? k_coarse_sap_persist<4> : k_coarse_sap_persist<2>;
+}
+void saph_attrs(const void* fn) {   // process-wide limits: the device maximum
+  cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cudaGetLastError();
 }
 }  // namespace
+
+// Cluster size and staged blocks per site (those inside the SAP block) of the kernel on FP16 blocks; 0 if none fits.
+// Sixteen CTAs per SAP block where all blocks of a colour are then resident at once, else eight: 16 blocks per colour
+// (16^3x32, 40 dof) 25.5 us per sweep with sixteen and 26.8 with eight, 34.0 and 37.4 for two right-hand sides;
+// 128 blocks (32^4) 112 and 115, 377 and 271 for four right-hand sides.  Staging all nine blocks of a site: 25.0
+// and 42, 148 and 204 for one right-hand side (fewer clusters fit).
+int coarse_saph_plan(const Geom& g, int n, int nblocks, int* CLS_out, int* nst_out, int prefer) {
+  *CLS_out = 0;
+  *nst_out = coarse_sap_slots(g);
+  for (int pass = 0; pass < 2; ++pass)   // the second without the residency condition
+    for (int CLS : {prefer, 16, 8, 4, 2}) {
+      if ((CLS != 2 && CLS != 4 && CLS != 8 && CLS != 16) || g.vB % CLS) continue;
+      const int spc = g.vB / CLS, rows = spc * n;
+      const size_t sm = saph_smem_layout(g.vB, n, spc, 1, *nst_out * spc, 1).total;
+      if (sm > 227 * 1024) continue;
+      const void* fn = (const void*)saph_kernel<1>(n);
+      saph_attrs(fn);
+      saph_attrs((const void*)saph_kernel<2>(n));
+      cudaLaunchConfig_t cfg = {};
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = CLS;
+      attr[0].val.clusterDim.y = 1;
+      attr[0].val.clusterDim.z = 1;
+      cfg.gridDim = dim3(CLS, 1, 1);
+      cfg.blockDim = dim3(saph_threads(rows, n), 1, 1);
+      cfg.dynamicSmemBytes = sm;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      int nclusters = 0;
+      if (cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) != cudaSuccess || nclusters < 1) {
+        cudaGetLastError();
+        continue;
+      }
+      if (pass == 0 && CLS == 16 && CLS != prefer && nclusters < nblocks) continue;
+      *CLS_out = CLS;
+      return 1;
+    }
+  return 0;
+}
 
 bool coarse_sap_persist_fits(const CoarseOp<float>& op, int nb0, int nb1, int* max_clusters, int* nbpc_out,
                              int min_nbpc) {
   if (max_clusters) *max_clusters = -1;
   if (nbpc_out) *nbpc_out = 0;
-  if (op.sap_cls <= 0 || !op.blkh || nb0 <= 0 || nb1 <= 0) return false;
-  const int CLS = op.sap_cls;
+  if (op.saph_cls <= 0 || !op.blkh || nb0 <= 0 || nb1 <= 0) return false;
+  const int CLS = op.saph_cls;
   const int nb = nb0 > nb1 ? nb0 : nb1;
   for (int nbpc = min_nbpc < 1 ? 1 : min_nbpc; nbpc <= 2; ++nbpc) {
-    const int threads = persist_threads(op, nbpc);
+    const int threads = saph_threads(op);
     const size_t sm = coarse_sap_persist_smem(op, nbpc);
-    if (threads > 768 || sm > 227 * 1024) continue;
-    const void* fn = persist_kernel(nbpc);
+    if (sm > 227 * 1024) continue;
+    const void* fn = (const void*)saph_persist_kernel(op);
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              227 * 1024) != cudaSuccess ||   // process-wide limit: the device maximum
         (CLS > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
@@ -1176,8 +1472,8 @@ cudaError_t coarse_sap_persist(cplx<float>* z, const cplx<float>* b, const Coars
                                int nb0, const int* blocks1, int nb1, int nrhs, size_t rstride, int k_mr, int iters,
                                int nbpc, unsigned* gcnt, cudaStream_t st) {
   if (nrhs <= 0 || iters <= 0) return cudaSuccess;
-  if (op.sap_cls <= 0 || !op.blkh || nb0 <= 0 || nb1 <= 0 || nbpc < 1 || nbpc > 2) return cudaErrorInvalidValue;
-  const int CLS = op.sap_cls, spc = op.g.vB / CLS;
+  if (op.saph_cls <= 0 || !op.blkh || nb0 <= 0 || nb1 <= 0 || nbpc < 1 || nbpc > 2) return cudaErrorInvalidValue;
+  const int CLS = op.saph_cls, spc = op.g.vB / CLS;
   const int nb = nb0 > nb1 ? nb0 : nb1;
   cudaError_t e = cudaMemsetAsync(gcnt, 0, sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
@@ -1190,62 +1486,61 @@ cudaError_t coarse_sap_persist(cplx<float>* z, const cplx<float>* b, const Coars
   attr[1].id = cudaLaunchAttributeCooperative;   // all clusters co-resident (they wait on one another)
   attr[1].val.cooperative = 1;
   cfg.gridDim = dim3(((nb + nbpc - 1) / nbpc) * CLS, 1, 1);
-  cfg.blockDim = dim3(persist_threads(op, nbpc), 1, 1);
+  cfg.blockDim = dim3(saph_threads(op), 1, 1);
   cfg.dynamicSmemBytes = coarse_sap_persist_smem(op, nbpc);
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   count_launch();
-  if (nbpc == 2)
-    return cudaLaunchKernelEx(&cfg, k_coarse_sap_persist<float, __half2, 2>, z, b, op.blkh, op.bscale, op.g, op.n,
-                              rstride, nrhs, blocks0, nb0, blocks1, nb1, k_mr, spc, op.sap_nsl, iters, op.err,
-                              op.bsite, op.bloc, gcnt);
-  return cudaLaunchKernelEx(&cfg, k_coarse_sap_persist<float, __half2, 1>, z, b, op.blkh, op.bscale, op.g, op.n,
-                            rstride, nrhs, blocks0, nb0, blocks1, nb1, k_mr, spc, op.sap_nsl, iters, op.err, op.bsite,
+  return cudaLaunchKernelEx(&cfg, saph_persist_kernel(op), z, b, op.blkh, op.bscale, op.g, op.n, fdiv_make(op.n), rstride, nrhs, blocks0, nb0,
+                            blocks1, nb1, k_mr, spc, op.sap_nsl, nbpc, iters, op.err, op.bsite,
                             op.bloc, gcnt);
 }
 
 template <typename T>
 cudaError_t coarse_sap_sweep(cplx<T>* z, const cplx<T>* b, const CoarseOp<T>& op, const int* blocks, int nblocks,
                              int nrhs, size_t rstride, int k_mr, cudaStream_t st) {
-  if (op.sap_cls > 0) {
-    const int spc = op.g.vB / op.sap_cls;
-    const int threads = ((9 * spc * op.n + 31) / 32) * 32;
-    const bool half = sizeof(T) == 4 && op.blkh;
+  const int cls = sizeof(T) == 4 && op.blkh ? op.saph_cls : op.sap_cls;
+  if (cls > 0) {
+    const int spc = op.g.vB / cls;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = op.sap_cls;
+    attr[0].val.clusterDim.x = cls;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     // consecutive colour sweeps: the next one stages its blocks while this one finishes
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3(nblocks * op.sap_cls, 1, 1);   // one cluster per SAP block loops over the batch
-    cfg.blockDim = dim3(threads, 1, 1);
-    cfg.dynamicSmemBytes =
-        sap_smem_layout(op.g.vB, op.n, spc, op.sap_nsl, half ? sizeof(__half2) : sizeof(cplx<T>), sizeof(T)).total;
+    cfg.gridDim = dim3(nblocks * cls, 1, 1);   // one cluster per SAP block loops over the batch
     cfg.stream = st;
     cfg.attrs = attr;
-    cfg.numAttrs = 2;
     count_launch();
     // with programmatic serialization first, then (if the attribute is refused) without it
     for (int na = 2; na >= 1; --na) {
       cfg.numAttrs = na;
       cudaError_t e;
       if constexpr (sizeof(T) == 4) {
-        if (half)
-          e = cudaLaunchKernelEx(&cfg, k_coarse_sap_cluster<float, __half2>, z, b, op.blkh, op.bscale, op.g, op.n,
-                                 rstride, nrhs, blocks, k_mr, spc, op.sap_nsl, op.err, op.bsite, op.bloc);
-        else
-          e = cudaLaunchKernelEx(&cfg, k_coarse_sap_cluster<T, cplx<T>>, z, b, (const cplx<T>*)op.blk,
-                                 (const float*)nullptr, op.g, op.n, rstride, nrhs, blocks, k_mr, spc, op.sap_nsl,
-                                 op.err, op.bsite, op.bloc);
-      } else {
-        e = cudaLaunchKernelEx(&cfg, k_coarse_sap_cluster<T, cplx<T>>, z, b, (const cplx<T>*)op.blk,
-                               (const float*)nullptr, op.g, op.n, rstride, nrhs, blocks, k_mr, spc, op.sap_nsl,
-                               op.err, op.bsite, op.bloc);
+        if (op.blkh) {
+          // two right-hand sides at a time unless that costs the second CTA per SM (a right-hand side's
+          // arithmetic does not depend on it)
+          auto smem = [&](int rb) { return saph_smem_layout(op.g.vB, op.n, spc, rb, op.saph_nst * spc, 1).total; };
+          const size_t two_per_sm = 113 * 1024;
+          const int rb = nrhs > 1 && smem(2) <= 227 * 1024 && (smem(2) <= two_per_sm || smem(1) > two_per_sm) ? 2 : 1;
+          cfg.blockDim = dim3(saph_threads(op), 1, 1);
+          cfg.dynamicSmemBytes = smem(rb);
+          e = cudaLaunchKernelEx(&cfg, rb == 2 ? saph_kernel<2>(op.n) : saph_kernel<1>(op.n), z, b,
+                                 op.blkh, op.bscale, op.g, op.n, fdiv_make(op.n), rstride, nrhs, blocks, k_mr, spc, op.saph_nst, op.err,
+                                 op.bsite, op.bloc);
+          if (e == cudaSuccess) return cudaSuccess;
+          cudaGetLastError();
+          continue;
+        }
       }
+      cfg.blockDim = dim3(((9 * spc * op.n + 31) / 32) * 32, 1, 1);
+      cfg.dynamicSmemBytes = sap_smem_layout(op.g.vB, op.n, spc, op.sap_nsl, sizeof(cplx<T>), sizeof(T)).total;
+      e = cudaLaunchKernelEx(&cfg, k_coarse_sap_cluster<T, cplx<T>>, z, b, (const cplx<T>*)op.blk, (const float*)nullptr,
+                             op.g, op.n, rstride, nrhs, blocks, k_mr, spc, op.sap_nsl, op.err, op.bsite, op.bloc);
       if (e == cudaSuccess) return cudaSuccess;
       cudaGetLastError();
     }

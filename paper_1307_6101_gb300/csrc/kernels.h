@@ -38,6 +38,8 @@ struct CoarseOp {
   int n_odd;
   int sap_cls;          // cluster size of the cluster SAP kernel (0: one CTA per SAP block)
   int sap_nsl = 0;      // blocks per site staged in shared memory by the cluster SAP kernel
+  int saph_cls = 0;     // the same two for the kernel on FP16 blocks
+  int saph_nst = 0;
   const int* bsite = nullptr;   // [nBlk][vB] sites of each SAP block (block-local order)
   const int* bloc = nullptr;    // [V] position of each site inside its SAP block
   int* err = nullptr;   // device error flag (bounded waits)
@@ -121,6 +123,8 @@ void coarse_selfinv_build(cplx<double>* inv, const cplx<double>* blk, int V, int
 template <typename T>
 // prefer: a cluster size (2, 4, 8, 16) to try first, anything else for the default order
 int coarse_sap_cluster_plan(const Geom& g, int n, int* CLS_out, int* spc_out, int* nsl_out, int prefer = 0);
+// the same for the kernel on FP16 blocks, for nblocks SAP blocks per colour: staged blocks per site in *nst
+int coarse_saph_plan(const Geom& g, int n, int nblocks, int* CLS_out, int* nst_out, int prefer = 0);
 // t(A odd) = S^{-1}(a b + c D_oe x)     (even entries of t untouched)
 template <typename T>
 void coarse_schur_odd(cplx<T>* t, const cplx<T>* x, const cplx<T>* b, const CoarseOp<T>& op, double a, double c,

@@ -348,7 +348,7 @@ template <typename T> bool half_on(const ddamg_handle* h) { return sizeof(T) == 
 template <typename T>
 void sap(ddamg_handle* h, Level& L, cplx<T>* z, const cplx<T>* b, int nrhs, int iterations) {
   if constexpr (sizeof(T) == 4) {
-    if (!L.fine && L.sap_persist && L.c32.sap_cls > 0 && half_on<T>(h) && iterations > 0) {
+    if (!L.fine && L.sap_persist && L.c32.saph_cls > 0 && half_on<T>(h) && iterations > 0) {
       // every sweep of the call in one launch (the tuner checked that it runs, eagerly and in a graph)
       Prof pr(h, DDAMG_PROF_COARSE_SAP,
               iterations * (sap_bytes<T>(L, 0, nrhs, true) + sap_bytes<T>(L, 1, nrhs, true)));
@@ -1565,6 +1565,7 @@ void allocate_hierarchy(ddamg_handle* h) {
       L.c32.sap_cls = coarse_sap_cluster_plan<float>(L.g, L.n, &cls, &spc, &L.c32.sap_nsl) ? cls : 0;
       L.c64.sap_cls = coarse_sap_cluster_plan<double>(L.g, L.n, &cls, &spc, &L.c64.sap_nsl) ? cls : 0;
       cudaGetLastError();
+      coarse_saph_plan(L.g, L.n, std::max(L.g.nBlk / 2, 1), &L.c32.saph_cls, &L.c32.saph_nst);
     }
     if (!L.coarsest) {
       L.tv64 = dalloc<cplx<double>>(h, L.vlen * L.N);
@@ -2399,6 +2400,8 @@ int ddamg_set_option(ddamg_handle* h, int option, int value) {
             (value && coarse_sap_cluster_plan<float>(L.g, L.n, &cls, &spc, &L.c32.sap_nsl, value)) ? cls : 0;
         L.c64.sap_cls =
             (value && coarse_sap_cluster_plan<double>(L.g, L.n, &cls, &spc, &L.c64.sap_nsl, value)) ? cls : 0;
+        L.c32.saph_cls = 0;
+        if (value) coarse_saph_plan(L.g, L.n, std::max(L.g.nBlk / 2, 1), &L.c32.saph_cls, &L.c32.saph_nst, value);
       }
       cudaGetLastError();
       if (h->half) {   // the persistent SAP launch follows the cluster plan
@@ -2457,7 +2460,7 @@ int ddamg_get_option(ddamg_handle* h, int option, int* value) {
     } else if (option == DDAMG_OPT_COARSEST_CLUSTER) {
       *value = (h->use_cluster && h->have_cplan32) ? h->cplan32.CL : 0;
     } else if (option == DDAMG_OPT_SAP_CLUSTER) {
-      *value = h->L > 2 ? h->lv[1].c32.sap_cls : 0;
+      *value = h->L > 2 ? (h->half ? h->lv[1].c32.saph_cls : h->lv[1].c32.sap_cls) : 0;
     } else if (option == DDAMG_OPT_HALF_STORAGE) {
       *value = h->half ? 1 : 0;
     } else if (option == DDAMG_OPT_COARSE_TC) {
