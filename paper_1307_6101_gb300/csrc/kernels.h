@@ -188,7 +188,7 @@ int galerkin_cols();
 template <typename T>
 bool galerkin_fits(int N, int C, int vA);
 template <typename T>
-cudaError_t galerkin_restrict(cplx<T>* out, const cplx<T>* tmp, const cplx<T>* P, const Geom& gf, const Geom& gc,
+cudaError_t galerkin_restrict(cplx<double>* out, const cplx<T>* tmp, const cplx<T>* P, const Geom& gf, const Geom& gc,
                               bool fine, int n, int N, int C, size_t tmp_rstride, size_t out_rstride,
                               size_t out_site_stride, int sel, int sel_mu, cudaStream_t st);
 // out(x, f) = [out +] sum_j P_j(x, f) in(A(x))[s(f)*N + j]

@@ -1238,13 +1238,15 @@ struct SetupTimer {
   }
 };
 
-// blk = the blocks of P_l^+ D_l P_l; term(t, p, jb, sel, mu, sp) = term (sel, mu) of D_l on the chirality-sp part
+// D_{l+1}'s FP64 blocks = those of P_l^+ D_l P_l (and the FP32 copy of them); term(t, p, jb, sel, mu, sp) = term (sel, mu) of D_l on the chirality-sp part
 // of jb fields p
 template <typename T, class Term>
-void galerkin(ddamg_handle* h, int l, const cplx<T>* P, cplx<T>* blk, Term term) {
+void galerkin(ddamg_handle* h, int l, const cplx<T>* P, Term term) {
   Level& F = h->lv[l];
   Level& C = h->lv[l + 1];
   const int nc = C.n;
+  const size_t nb = (size_t)C.g.V * 9 * nc * nc;
+  const bool fits = galerkin_fits<T>(F.N, galerkin_cols(), F.g.vA);
   const int jb_max = std::min(F.N, sizeof(T) == 4 ? galerkin_cols() : SETUP_CHUNK);
   cplx<T>* tmp = static_cast<cplx<T>*>(scratch(h, 4, sizeof(cplx<T>) * F.vlen * jb_max));
   for (int sp = 0; sp < 2; ++sp)
@@ -1253,19 +1255,22 @@ void galerkin(ddamg_handle* h, int l, const cplx<T>* P, cplx<T>* blk, Term term)
       const int mu = k == 0 ? 0 : (k - 1) % 4;
       for (int j0 = 0; j0 < F.N; j0 += jb_max) {
         const int jb = std::min(jb_max, F.N - j0);
-        cplx<T>* out = blk + (size_t)k * nc * nc + (size_t)(sp * F.N + j0) * nc;
-        if (!galerkin_fits<T>(F.N, jb, F.g.vA)) {   // an aggregate of tens of thousands of sites
+        const size_t at = (size_t)k * nc * nc + (size_t)(sp * F.N + j0) * nc;
+        if (!fits) {   // an aggregate of tens of thousands of sites
           blas_zero<T>(tmp, F.vlen, jb, F.vlen, h->st);
           term(tmp, P + (size_t)j0 * F.vlen, jb, sel, mu, sp);
-          restrict_op<T>(out, tmp, P, F.g, C.g, F.fine, F.n, F.N, jb, F.vlen, (size_t)nc, (size_t)9 * nc * nc, h->d_err, h->st);
+          restrict_op<T>(cop<T>(C).blk + at, tmp, P, F.g, C.g, F.fine, F.n, F.N, jb, F.vlen, (size_t)nc,
+                         (size_t)9 * nc * nc, h->d_err, h->st);
           continue;
         }
         term(tmp, P + (size_t)j0 * F.vlen, jb, sel, mu, sp);
-        if (galerkin_restrict<T>(out, tmp, P, F.g, C.g, F.fine, F.n, F.N, jb, F.vlen, (size_t)nc, (size_t)9 * nc * nc,
-                                 sel, mu, h->st) != cudaSuccess)
+        if (galerkin_restrict<T>(C.c64.blk + at, tmp, P, F.g, C.g, F.fine, F.n, F.N, jb, F.vlen, (size_t)nc,
+                                 (size_t)9 * nc * nc, sel, mu, h->st) != cudaSuccess)
           fail(DDAMG_ERR_CUDA, "launch of the Galerkin product failed");
       }
     }
+  if (!fits && sizeof(T) == 4) blas_convert<double, float>(C.c64.blk, C.c32.blk, nb, 1, 0, 0, h->st);
+  else blas_convert<float, double>(C.c32.blk, C.c64.blk, nb, 1, 0, 0, h->st);
 }
 
 void rebuild(ddamg_handle* h, int l) {
@@ -1282,7 +1287,6 @@ void rebuild(ddamg_handle* h, int l) {
   // in chunks of columns (bounded scratch: eight FP32 or four FP64 fields).  A handle with the FP32
   // preconditioner forms the product in FP32 from the FP32 copies of the operator and P (the preconditioner's
   // setup runs in single precision, Sec. 3); an FP64 handle in FP64.
-  const size_t nb = (size_t)C.g.V * 9 * C.n * C.n;
   if (h->p.precision != 0) {
     FineOp<float> fo = F.f32;   // FP32 storage, not the FP16 copies
     fo.Uh = nullptr;
@@ -1290,16 +1294,14 @@ void rebuild(ddamg_handle* h, int l) {
     CoarseOp<float> co = F.c32;
     co.blkh = nullptr;
     co.bscale = nullptr;
-    galerkin<float>(h, l, F.P32, C.c32.blk, [&](cplx<float>* t, const cplx<float>* p, int jb, int sel, int mu, int sp) {
+    galerkin<float>(h, l, F.P32, [&](cplx<float>* t, const cplx<float>* p, int jb, int sel, int mu, int sp) {
       if (F.fine) fine_dslash<float>(t, p, nullptr, fo, jb, F.vlen, sel, mu, sp, st);
       else coarse_apply<float>(t, p, nullptr, co, jb, F.vlen, sel, mu, sp, st);
     });
-    blas_convert<double, float>(C.c64.blk, C.c32.blk, nb, 1, 0, 0, st);
   } else {
-    galerkin<double>(h, l, F.P64, C.c64.blk, [&](cplx<double>* t, const cplx<double>* p, int jb, int sel, int mu, int sp) {
+    galerkin<double>(h, l, F.P64, [&](cplx<double>* t, const cplx<double>* p, int jb, int sel, int mu, int sp) {
       apply_D<double>(h, F, t, p, nullptr, jb, sel, mu, sp);
     });
-    blas_convert<float, double>(C.c32.blk, C.c64.blk, nb, 1, 0, 0, st);
   }
   if (C.coarsest && C.eo) {
     coarse_selfinv_build(C.c64.selfinv, C.c64.blk, C.g.V, C.n, h->d_err, st);

@@ -28,14 +28,6 @@ __device__ __forceinline__ unsigned map_rank_u32(const void* p, int rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
   return a;
 }
-// bulk copy of own shared memory (src) to the same kind of place (dst) in CTA `rank`, completing on its barrier bar
-__device__ __forceinline__ void bulk_s2cluster(void* dst, const void* src, unsigned bytes, unsigned long long* bar,
-                                               int rank) {
-  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   map_rank_u32(dst, rank)),
-               "r"(smem_u32(src)), "r"(bytes), "r"(map_rank_u32(bar, rank))
-               : "memory");
-}
 // 16-byte asynchronous store to the place that corresponds to dst in CTA `rank`, completing on its barrier bar
 __device__ __forceinline__ void st_async_cluster(float4* dst, float4 v, unsigned long long* bar, int rank) {
   asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(

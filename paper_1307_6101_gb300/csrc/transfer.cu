@@ -245,7 +245,9 @@ __global__ void k_prolong(cplx<T>* __restrict__ out, const cplx<T>* __restrict__
 // Galerkin products: columns of P^+ (term of D P), for C <= 8 columns of one launch.
 //   out[c][site of A][s*N + i] = sum over x in A, f in s of conj(P_i(x, f)) tmp_c(x, f)
 // A term of a hop that leaves the aggregate is nonzero on one face of it only, and only those sites are read
-// (tmp is not even written elsewhere): of 4^4 aggregates a quarter, for eight of the nine terms.
+// (tmp is not even written elsewhere): of 4^4 aggregates a quarter, for eight of the nine terms.  FP32 products are summed
+// in FP32 over two chunks and from there on with their rounding errors (pairs), so that a block entry is as exact
+// as its FP32 operands and the FP16 copy of it rounds as the FP64 product would.
 // One CTA per (aggregate, chirality): the N x K by K x C product with K staged in chunks, each lane a 4 x 4
 // tile of the result (64 FMAs for 8 shared-memory loads), the lanes that N x C does not need and the warps
 // splitting K (summed at the end in a fixed order).
@@ -256,7 +258,7 @@ constexpr int GT = 256;    // threads
 constexpr int GKC = 64;    // K rows per staged chunk
 constexpr int GCMAX = 8;   // columns per launch
 
-constexpr int GFLUSH = 4;  // chunks whose products run into one accumulator
+constexpr int GFLUSH = 2;  // chunks whose products run into one accumulator
 
 struct GalerkinSmem {
   size_t red, list, total;
@@ -265,13 +267,20 @@ DD_HD GalerkinSmem galerkin_smem(int N, int C, int vA, size_t cs) {
   GalerkinSmem L;
   const int tiles = ((N + 3) / 4) * ((C + 3) / 4);
   L.red = (((size_t)GKC * ((N | 1) + (C | 1)) * cs) + 15) & ~size_t(15);
-  L.list = L.red + (size_t)(GT / 32) * (32 / tiles) * tiles * 16 * cs;
+  L.list = L.red + (size_t)(cs == sizeof(cplx<float>) ? 2 : 1) * (GT / 32) * (32 / tiles) * tiles * 16 * cs;
   L.total = L.list + (size_t)vA * sizeof(int);
   return L;
 }
 
+// (hi, lo) += x without rounding error beyond lo's (Knuth's two-sum)
+__device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float x) {
+  const float s = __fadd_rn(hi, x), t = __fsub_rn(s, hi);
+  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(x, t)));
+  hi = s;
+}
+
 template <typename T>
-__global__ void __launch_bounds__(GT) k_galerkin(cplx<T>* __restrict__ out, const cplx<T>* __restrict__ tmp,
+__global__ void __launch_bounds__(GT) k_galerkin(cplx<double>* __restrict__ out, const cplx<T>* __restrict__ tmp,
                                                  const cplx<T>* __restrict__ P, Geom gf, bool fine, int n, int N, int C,
                                                   size_t tmp_rstride, size_t pstride, size_t out_rstride,
                                                  size_t out_site_stride, int sel, int sel_mu) {
@@ -361,7 +370,11 @@ __global__ void __launch_bounds__(GT) k_galerkin(cplx<T>* __restrict__ out, cons
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int c = 0; c < 4; ++c) cfmac(acc[i][c], a[i], b[c]);
+          for (int c = 0; c < 4; ++c) {
+            // FP64 FMAs bound the kernel: none for the part of a tile outside N x C
+            if (sizeof(T) == 8 && (i0 + i >= N || c0 + c >= C)) continue;
+            cfmac(acc[i][c], a[i], b[c]);
+          }
       }
       // long sums in parts: their rounding errors do not add up along the whole of K
       if (chunk % GFLUSH == GFLUSH - 1 || k0 + GKC >= K) {
@@ -370,22 +383,44 @@ __global__ void __launch_bounds__(GT) k_galerkin(cplx<T>* __restrict__ out, cons
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
             cplx<T>& m = mine[(4 * i + c) * slots];
-            m = chunk < GFLUSH ? acc[i][c] : m + acc[i][c];
+            if constexpr (sizeof(T) == 4) {
+              cplx<T>& e = mine[(16 + 4 * i + c) * slots];
+              cplx<T> hi = chunk < GFLUSH ? acc[i][c] : m, lo = chunk < GFLUSH ? czero<T>() : e;
+              if (chunk >= GFLUSH) {
+                two_sum_acc(hi.re, lo.re, acc[i][c].re);
+                two_sum_acc(hi.im, lo.im, acc[i][c].im);
+              }
+              m = hi;
+              e = lo;
+            } else {
+              m = chunk < GFLUSH ? acc[i][c] : m + acc[i][c];
+            }
             acc[i][c] = czero<T>();
           }
       }
     }
     __syncthreads();
   }
-  cplx<T>* po = out + (size_t)gf.csite[agg] * out_site_stride + (size_t)s * N;
+  cplx<double>* po = out + (size_t)gf.csite[agg] * out_site_stride + (size_t)s * N;
   for (int e = tid; e < N * C; e += GT) {
     const int c = e / N, i = e - c * N;
     const cplx<T>* r = red + (4 * (i % 4) + c % 4) * slots + (c / 4) * TI + i / 4;
+    if constexpr (sizeof(T) == 4) {
+      cplx<T> hi = czero<T>(), lo = czero<T>();
+      for (int q = 0; K > 0 && q < (GT / 32) * nsub; ++q) {
+        const cplx<T> h = r[q * tiles], l = r[16 * slots + q * tiles];
+        two_sum_acc(hi.re, lo.re, h.re);
+        two_sum_acc(hi.im, lo.im, h.im);
+        lo = lo + l;
+      }
+      po[(size_t)c * out_rstride + i] = cmk((double)hi.re + (double)lo.re, (double)hi.im + (double)lo.im);
+      continue;
+    }
     cplx<T> t[4] = {czero<T>(), czero<T>(), czero<T>(), czero<T>()};   // the parts in four chains
     for (int q = 0; K > 0 && q < (GT / 32) * nsub; q += 4)
 #pragma unroll
       for (int u = 0; u < 4; ++u) t[u] = t[u] + r[(q + u) * tiles];
-    po[(size_t)c * out_rstride + i] = (t[0] + t[1]) + (t[2] + t[3]);
+    po[(size_t)c * out_rstride + i] = ccast<double>((t[0] + t[1]) + (t[2] + t[3]));
   }
 }
 
@@ -651,7 +686,7 @@ bool galerkin_fits(int N, int C, int vA) {
 }
 
 template <typename T>
-cudaError_t galerkin_restrict(cplx<T>* out, const cplx<T>* tmp, const cplx<T>* P, const Geom& gf, const Geom& gc,
+cudaError_t galerkin_restrict(cplx<double>* out, const cplx<T>* tmp, const cplx<T>* P, const Geom& gf, const Geom& gc,
                               bool fine, int n, int N, int C, size_t tmp_rstride, size_t out_rstride,
                               size_t out_site_stride, int sel, int sel_mu, cudaStream_t st) {
   const size_t sm = galerkin_smem(N, C, gf.vA, sizeof(cplx<T>)).total;
@@ -672,7 +707,7 @@ cudaError_t galerkin_restrict(cplx<T>* out, const cplx<T>* tmp, const cplx<T>* P
   template void prolong_op<T>(cplx<T>*, const cplx<T>*, const cplx<T>*, const Geom&, const Geom&, bool, int, int,  \
                               int, size_t, size_t, bool, cudaStream_t, const __half2*, const float*, int);   \
   template bool galerkin_fits<T>(int, int, int);                                                                 \
-  template cudaError_t galerkin_restrict<T>(cplx<T>*, const cplx<T>*, const cplx<T>*, const Geom&, const Geom&, bool, \
+  template cudaError_t galerkin_restrict<T>(cplx<double>*, const cplx<T>*, const cplx<T>*, const Geom&, const Geom&, bool, \
                                             int, int, int, size_t, size_t, size_t, int, int, cudaStream_t);
 INST(float)
 INST(double)
