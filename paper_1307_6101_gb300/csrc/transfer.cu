@@ -246,8 +246,8 @@ __global__ void k_prolong(cplx<T>* __restrict__ out, const cplx<T>* __restrict__
 //   out[c][site of A][s*N + i] = sum over x in A, f in s of conj(P_i(x, f)) tmp_c(x, f)
 // A term of a hop that leaves the aggregate is nonzero on one face of it only, and only those sites are read
 // (tmp is not even written elsewhere): of 4^4 aggregates a quarter, for eight of the nine terms.  FP32 products are summed
-// in FP32 over two chunks and from there on with their rounding errors (pairs), so that a block entry is as exact
-// as its FP32 operands and the FP16 copy of it rounds as the FP64 product would.
+// in FP32 over two chunks and from there on with their rounding errors (pairs), and rounded to FP32 once: against
+// FP64 the blocks of 16^3x32 are off by 3.9e-8 (5.1e-8 with plain sums).
 // One CTA per (aggregate, chirality): the N x K by K x C product with K staged in chunks, each lane a 4 x 4
 // tile of the result (64 FMAs for 8 shared-memory loads), the lanes that N x C does not need and the warps
 // splitting K (summed at the end in a fixed order).
@@ -263,11 +263,16 @@ constexpr int GFLUSH = 2;  // chunks whose products run into one accumulator
 struct GalerkinSmem {
   size_t red, list, total;
 };
+// shares of a chunk's rows within a warp: as many as its lanes hold tiles, and no more than there are rows
+DD_HD int galerkin_nsub(int tiles) {
+  return 32 / tiles < GKC / (GT / 32) ? 32 / tiles : GKC / (GT / 32);
+}
 DD_HD GalerkinSmem galerkin_smem(int N, int C, int vA, size_t cs) {
   GalerkinSmem L;
   const int tiles = ((N + 3) / 4) * ((C + 3) / 4);
+  const int nsub = galerkin_nsub(tiles);
   L.red = (((size_t)GKC * ((N | 1) + (C | 1)) * cs) + 15) & ~size_t(15);
-  L.list = L.red + (size_t)(cs == sizeof(cplx<float>) ? 2 : 1) * (GT / 32) * (32 / tiles) * tiles * 16 * cs;
+  L.list = L.red + (size_t)(cs == sizeof(cplx<float>) ? 2 : 1) * (GT / 32) * nsub * tiles * 16 * cs;
   L.total = L.list + (size_t)vA * sizeof(int);
   return L;
 }
@@ -317,7 +322,7 @@ __global__ void __launch_bounds__(GT) k_galerkin(cplx<double>* __restrict__ out,
     __syncthreads();
   }
   const int nS = nsites, K = nS * h;
-  const int TI = (N + 3) / 4, TC = (C + 3) / 4, tiles = TI * TC, nsub = 32 / tiles;
+  const int TI = (N + 3) / 4, TC = (C + 3) / 4, tiles = TI * TC, nsub = galerkin_nsub(tiles);
   const int sub = lane / tiles, tile = lane - sub * tiles;
   const int i0 = 4 * (tile % TI), c0 = 4 * (tile / TI);
   cplx<T> acc[4][4];
@@ -371,13 +376,11 @@ __global__ void __launch_bounds__(GT) k_galerkin(cplx<double>* __restrict__ out,
         for (int i = 0; i < 4; ++i)
 #pragma unroll
           for (int c = 0; c < 4; ++c) {
-            // FP64 FMAs bound the kernel: none for the part of a tile outside N x C
-            if (sizeof(T) == 8 && (i0 + i >= N || c0 + c >= C)) continue;
             cfmac(acc[i][c], a[i], b[c]);
           }
       }
-      // long sums in parts: their rounding errors do not add up along the whole of K
-      if (chunk % GFLUSH == GFLUSH - 1 || k0 + GKC >= K) {
+      // long FP32 sums in parts: their rounding errors do not add up along the whole of K
+      if ((sizeof(T) == 4 && chunk % GFLUSH == GFLUSH - 1) || k0 + GKC >= K) {
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -393,7 +396,7 @@ __global__ void __launch_bounds__(GT) k_galerkin(cplx<double>* __restrict__ out,
               m = hi;
               e = lo;
             } else {
-              m = chunk < GFLUSH ? acc[i][c] : m + acc[i][c];
+              m = acc[i][c];
             }
             acc[i][c] = czero<T>();
           }
@@ -413,7 +416,7 @@ __global__ void __launch_bounds__(GT) k_galerkin(cplx<double>* __restrict__ out,
         two_sum_acc(hi.im, lo.im, h.im);
         lo = lo + l;
       }
-      po[(size_t)c * out_rstride + i] = cmk((double)hi.re + (double)lo.re, (double)hi.im + (double)lo.im);
+      po[(size_t)c * out_rstride + i] = cmk((double)(hi.re + lo.re), (double)(hi.im + lo.im));
       continue;
     }
     cplx<T> t[4] = {czero<T>(), czero<T>(), czero<T>(), czero<T>()};   // the parts in four chains
