@@ -8,6 +8,7 @@
 #include "kernels.h"
 
 #include <stdexcept>
+#include <type_traits>
 #include <unordered_map>
 
 #include <cstdio>
@@ -47,7 +48,7 @@ double* partials(size_t count, cudaStream_t st) {
 }
 
 int nchunks(size_t len) {
-  size_t c = (len + 4 * RT - 1) / (4 * RT);
+  size_t c = (len + 2 * RT - 1) / (2 * RT);
   if (c < 1) c = 1;
   if (c > MAXCHUNKS) c = MAXCHUNKS;
   return (int)c;
@@ -83,81 +84,103 @@ __device__ void chunk_range(size_t len, int nc, int c, size_t& lo, size_t& hi) {
   if (lo > len) lo = len;
 }
 
-// stage 1 of dot / norm: partial[(rhs * ndots + d) * nc + chunk] (re, im)
+// Sum 8 values per thread over the CTA (RT threads); thread k < 8 returns the sum of value k.  The lanes share the
+// values out as they fold (9 additions per lane), and eight threads add the warps' sums.  The order is that of
+// a butterfly over the lanes, then the warps by number.
+__device__ __forceinline__ double cta_fold8(double* v, double* sh) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int w = 4, off = 16; w >= 1; w >>= 1, off >>= 1) {
+    const bool up = (lane & off) != 0;
+#pragma unroll
+    for (int k = 0; k < w; ++k) {
+      const double keep = up ? v[k + w] : v[k], send = up ? v[k] : v[k + w];
+      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+    }
+  }
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+  if ((lane & 3) == 0) sh[warp * 8 + (lane >> 2)] = v[0];
+  __syncthreads();
+  double s = 0.0;
+  if (threadIdx.x < 8)
+#pragma unroll
+    for (int w = 0; w < RT / 32; ++w) s += sh[w * 8 + threadIdx.x];
+  return s;
+}
+
+// Stage 1 of dot: partial[(rhs * m + d) * nc + chunk] (re, im); blockIdx.z = group of four vectors d.
+// Bound by the FP64 rate, at FP32 by the launch: with the groups in one CTA one after another, 40 additions per lane
+// and group for the CTA sum and 48 CTAs for 8^4, 13 vectors of 8^4 took 51 us and six of 16^3x32 114 us.  Now 12
+// and 76 us (the FP64 rate: 72).
 template <typename T>
-__global__ void k_multidot1(double* __restrict__ part, const cplx<T>* __restrict__ V, size_t vstride, int m,
-                            const cplx<T>* __restrict__ w, size_t len, size_t rstride, int nc) {
-  __shared__ double sh[32 * 8];
-  const int chunk = blockIdx.x, rhs = blockIdx.y;
+__global__ void __launch_bounds__(RT) k_multidot1(double* __restrict__ part, const cplx<T>* __restrict__ V,
+                                                  size_t vstride, int m, const cplx<T>* __restrict__ w, size_t len,
+                                                  size_t rstride, int nc) {
+  __shared__ double sh[RT / 32 * 8];
+  const int chunk = blockIdx.x, rhs = blockIdx.y, d0 = 4 * blockIdx.z, nd = min(4, m - d0);
   size_t lo, hi;
   chunk_range(len, nc, chunk, lo, hi);
   const cplx<T>* pw = w + (size_t)rhs * rstride;
-  for (int d0 = 0; d0 < m; d0 += 4) {
-    // per-thread partials in the precision of the data (FP32 data: FP32 sums)
-    T at[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (size_t e = lo + threadIdx.x; e < hi; e += blockDim.x) {
+  const cplx<T>* pv = V + (size_t)d0 * vstride + (size_t)rhs * rstride;
+  // per-thread partials in the precision of the data (FP32 data: FP32 sums)
+  T at[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  auto products = [&](auto count) {   // a skipped FP64 FMA takes its time all the same: a loop for each count
+    for (size_t e = lo + threadIdx.x; e < hi; e += RT) {
       const cplx<T> we = pw[e];
 #pragma unroll
-      for (int dd = 0; dd < 4; ++dd) {
-        if (d0 + dd < m) {
-          const cplx<T> v = V[(size_t)(d0 + dd) * vstride + (size_t)rhs * rstride + e];
-          cdotc_acc(at[2 * dd], at[2 * dd + 1], v, we);
-        }
-      }
+      for (int dd = 0; dd < decltype(count)::value; ++dd)
+        cdotc_acc(at[2 * dd], at[2 * dd + 1], pv[(size_t)dd * vstride + e], we);
     }
-    double acc[8];
+  };
+  if (nd == 4) products(std::integral_constant<int, 4>());
+  else if (nd == 3) products(std::integral_constant<int, 3>());
+  else if (nd == 2) products(std::integral_constant<int, 2>());
+  else products(std::integral_constant<int, 1>());
+  double acc[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) acc[k] = (double)at[k];
-    cta_sum(acc, 8, sh);
-    if (threadIdx.x == 0)
-      for (int dd = 0; dd < 4 && d0 + dd < m; ++dd) {
-        double* p = part + (((size_t)rhs * m + d0 + dd) * nc + chunk) * 2;
-        p[0] = acc[2 * dd];
-        p[1] = acc[2 * dd + 1];
-      }
-  }
+  for (int k = 0; k < 8; ++k) acc[k] = (double)at[k];
+  const double t = cta_fold8(acc, sh);
+  if (threadIdx.x < 2 * nd)
+    part[(((size_t)rhs * m + d0 + (threadIdx.x >> 1)) * nc + chunk) * 2 + (threadIdx.x & 1)] = t;
 }
 
 // stage 1 of the multidot in double-FP32 arithmetic on FP64 vectors: the elements are split on
 // load, products and the per-thread sums are double-FP32, the CTA sum is FP64 (partials as above)
-__global__ void k_multidot1_df(double* __restrict__ part, const cplx<double>* __restrict__ V, size_t vstride,
-                               int m, const cplx<double>* __restrict__ w, size_t len, size_t rstride, int nc) {
-  __shared__ double sh[32 * 8];
-  const int chunk = blockIdx.x, rhs = blockIdx.y;
+__global__ void __launch_bounds__(RT) k_multidot1_df(double* __restrict__ part, const cplx<double>* __restrict__ V,
+                                                     size_t vstride, int m, const cplx<double>* __restrict__ w,
+                                                     size_t len, size_t rstride, int nc) {
+  __shared__ double sh[RT / 32 * 8];
+  const int chunk = blockIdx.x, rhs = blockIdx.y, d0 = 4 * blockIdx.z, nd = min(4, m - d0);
   size_t lo, hi;
   chunk_range(len, nc, chunk, lo, hi);
   const cplx<double>* pw = w + (size_t)rhs * rstride;
-  for (int d0 = 0; d0 < m; d0 += 4) {
-    dfl at[8];
+  const cplx<double>* pv = V + (size_t)d0 * vstride + (size_t)rhs * rstride;
+  dfl at[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) at[k] = dfl(0);
-    for (size_t e = lo + threadIdx.x; e < hi; e += blockDim.x) {
-      const cplx<double> wd = pw[e];
-      const dfl wr = df_from_double(wd.re), wi = df_from_double(wd.im);
+  for (int k = 0; k < 8; ++k) at[k] = dfl(0);
+  for (size_t e = lo + threadIdx.x; e < hi; e += RT) {
+    const cplx<double> wd = pw[e];
+    const dfl wr = df_from_double(wd.re), wi = df_from_double(wd.im);
 #pragma unroll
-      for (int dd = 0; dd < 4; ++dd) {
-        if (d0 + dd < m) {
-          const cplx<double> vd = V[(size_t)(d0 + dd) * vstride + (size_t)rhs * rstride + e];
-          const dfl vr = df_from_double(vd.re), vi = df_from_double(vd.im);
-          // conj(v) w
-          at[2 * dd] = fma(vr, wr, at[2 * dd]);
-          at[2 * dd] = fma(vi, wi, at[2 * dd]);
-          at[2 * dd + 1] = fma(vr, wi, at[2 * dd + 1]);
-          at[2 * dd + 1] = fma(-vi, wr, at[2 * dd + 1]);
-        }
+    for (int dd = 0; dd < 4; ++dd) {
+      if (dd < nd) {
+        const cplx<double> vd = pv[(size_t)dd * vstride + e];
+        const dfl vr = df_from_double(vd.re), vi = df_from_double(vd.im);
+        // conj(v) w
+        at[2 * dd] = fma(vr, wr, at[2 * dd]);
+        at[2 * dd] = fma(vi, wi, at[2 * dd]);
+        at[2 * dd + 1] = fma(vr, wi, at[2 * dd + 1]);
+        at[2 * dd + 1] = fma(-vi, wr, at[2 * dd + 1]);
       }
     }
-    double acc[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) acc[k] = df_to_double(at[k]);
-    cta_sum(acc, 8, sh);
-    if (threadIdx.x == 0)
-      for (int dd = 0; dd < 4 && d0 + dd < m; ++dd) {
-        double* p = part + (((size_t)rhs * m + d0 + dd) * nc + chunk) * 2;
-        p[0] = acc[2 * dd];
-        p[1] = acc[2 * dd + 1];
-      }
   }
+  double acc[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) acc[k] = df_to_double(at[k]);
+  const double t = cta_fold8(acc, sh);
+  if (threadIdx.x < 2 * nd)
+    part[(((size_t)rhs * m + d0 + (threadIdx.x >> 1)) * nc + chunk) * 2 + (threadIdx.x & 1)] = t;
 }
 
 // stage 2: res[rhs * m + d] = sum over chunks, fixed order
@@ -320,56 +343,95 @@ __global__ void k_gmres_begin(dd::GmresState s, int nrhs) {
   s.est[r] = b;
 }
 
-__global__ void k_gmres_step(dd::GmresState s, int j, int nrhs) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= nrhs) return;
-  if (s.done[r]) { s.inv[r] = 0.0; return; }   // finished rhs: next basis vector is exactly zero
+// One Arnoldi column per right-hand side: a warp each.  The j rotations of the earlier steps are a chain in the
+// running entry alone: lane 0 carries its real part and lane 1 its imaginary part (two FP64 FMAs and a shuffle per
+// rotation), what does not depend on it is formed by all lanes before and after.  8^4, steps 0 to 25:
+// 9.8 us on average (15.2 by one thread, whose FP64 operations take 31 ns each).
+__global__ void __launch_bounds__(32) k_gmres_step(dd::GmresState s, int j) {
+  __shared__ cplx<double> hh[65], cur[65], sh_sn[64];
+  __shared__ double sh_cs[64];
+  const int r = blockIdx.x, lane = threadIdx.x;
+  if (s.done[r]) {   // finished rhs: next basis vector is exactly zero
+    if (lane == 0) s.inv[r] = 0.0;
+    return;
+  }
   const int m = s.m;
   cplx<double>* H = s.H + (size_t)r * (m + 1) * m;
   cplx<double>* g = s.g + (size_t)r * (m + 1);
   double* cs = s.cs + (size_t)r * m;
   cplx<double>* sn = s.sn + (size_t)r * m;
-  cplx<double> h[64];
-  for (int i = 0; i <= j; ++i) h[i] = s.h1[(size_t)r * (m + 1) + i] + s.h2[(size_t)r * (m + 1) + i];
   const double hn = s.wnorm[r];
-  h[j + 1] = cmk(hn, 0.0);
-  for (int i = 0; i < j; ++i) {
-    const cplx<double> t = cs[i] * h[i] + sn[i] * h[i + 1];
-    h[i + 1] = cs[i] * h[i + 1] - cconj(sn[i]) * h[i];
-    h[i] = t;
+  for (int i = lane; i <= j; i += 32) {
+    hh[i] = s.h1[(size_t)r * (m + 1) + i] + s.h2[(size_t)r * (m + 1) + i];
+    if (i < j) {
+      sh_cs[i] = cs[i];
+      sh_sn[i] = sn[i];
+    }
   }
+  __syncwarp();
+  for (int i = lane; i < j; i += 32) cur[i + 1] = sh_cs[i] * hh[i + 1];
+  __syncwarp();
+  if (lane == 0) cur[0] = hh[0];
+  __syncwarp();
+  if (j > 0) {
+    const int p = lane & 1;   // every lane computes; lanes 0 and 1 store
+    double c = p ? cur[0].im : cur[0].re;
+    for (int i = 0; i < j; ++i) {
+      const cplx<double> si = sh_sn[i];
+      const double a = p ? cur[i + 1].im : cur[i + 1].re, im = p ? si.im : -si.im;
+      const double o = __shfl_xor_sync(0xffffffffu, c, 1);
+      c = fma(im, o, fma(-si.re, c, a));   // cs h_{i+1} - conj(sn) h_i
+      __syncwarp();
+      if (lane < 2) reinterpret_cast<double*>(&cur[i + 1])[p] = c;
+    }
+  }
+  __syncwarp();
+  for (int i = lane; i < j; i += 32) H[(size_t)i * m + j] = sh_cs[i] * cur[i] + sh_sn[i] * hh[i + 1];
+  if (lane) return;
+  const cplx<double> h0 = cur[j], h1 = cmk(hn, 0.0);
   double c;
   cplx<double> sg;
-  givens(h[j], h[j + 1], c, sg);
+  givens(h0, h1, c, sg);
   cs[j] = c;
   sn[j] = sg;
-  h[j] = c * h[j] + sg * h[j + 1];
-  h[j + 1] = czero<double>();
-  g[j + 1] = -1.0 * (cconj(sg) * g[j]);
-  g[j] = c * g[j];
-  for (int i = 0; i <= j + 1; ++i) H[(size_t)i * m + j] = h[i];
+  H[(size_t)j * m + j] = c * h0 + sg * h1;
+  H[(size_t)(j + 1) * m + j] = czero<double>();
+  const cplx<double> gj = g[j], g1 = -1.0 * (cconj(sg) * gj);
+  g[j + 1] = g1;
+  g[j] = c * gj;
   s.kr[r] = j + 1;
-  const double est = sqrt(cnorm2(g[j + 1]));
+  const double est = sqrt(cnorm2(g1));
   s.est[r] = est;
   s.inv[r] = hn > 0.0 ? 1.0 / hn : 0.0;
   if (est <= s.target[r] || hn == 0.0 || j + 1 == m) { s.done[r] = 1; s.inv[r] = 0.0; }
 }
 
-__global__ void k_gmres_solve_y(dd::GmresState s, int nrhs) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= nrhs) return;
+// y = R^{-1} g, a warp per right-hand side: R's upper triangle by columns in shared memory; with y_i known, all
+// lanes subtract its column from the rows above.
+__global__ void __launch_bounds__(32) k_gmres_solve_y(dd::GmresState s) {
+  __shared__ cplx<double> R[64 * 63 / 2];   // above the diagonal: column l from l (l - 1) / 2
+  __shared__ cplx<double> t[64], id[64];
+  const int r = blockIdx.x, lane = threadIdx.x;
   const int m = s.m;
   const int k = s.kr[r];
   const cplx<double>* H = s.H + (size_t)r * (m + 1) * m;
   const cplx<double>* g = s.g + (size_t)r * (m + 1);
   cplx<double>* y = s.y + (size_t)r * m;
-  for (int i = k; i < m; ++i) y[i] = czero<double>();
-  for (int i = k - 1; i >= 0; --i) {
-    cplx<double> t = g[i];
-    for (int l = i + 1; l < k; ++l) t = t - H[(size_t)i * m + l] * y[l];
+  for (int i = k + lane; i < m; i += 32) y[i] = czero<double>();
+  for (int i = 0; i < k; ++i)
+    for (int l = i + 1 + lane; l < k; l += 32) R[l * (l - 1) / 2 + i] = H[(size_t)i * m + l];
+  for (int i = lane; i < k; i += 32) {
     const cplx<double> d = H[(size_t)i * m + i];
     const double dn = cnorm2(d);
-    y[i] = dn > 0.0 ? (1.0 / dn) * (t * cconj(d)) : czero<double>();
+    id[i] = dn > 0.0 ? (1.0 / dn) * cconj(d) : czero<double>();
+    t[i] = g[i];
+  }
+  __syncwarp();
+  for (int i = k - 1; i >= 0; --i) {
+    const cplx<double> yi = t[i] * id[i];
+    for (int l = lane; l < i; l += 32) t[l] = t[l] - R[i * (i - 1) / 2 + l] * yi;
+    if (lane == 0) y[i] = yi;
+    __syncwarp();
   }
 }
 
@@ -388,7 +450,7 @@ void blas_multidot(cplx<double>* res, int res_stride, const cplx<T>* V, size_t v
   const int nc = nchunks(len);
   double* part = partials((size_t)nrhs * m * nc * 2, st);
   count_launch();
-  k_multidot1<T><<<dim3(nc, nrhs), RT, 0, st>>>(part, V, vstride, m, w, len, rstride, nc);
+  k_multidot1<T><<<dim3(nc, nrhs, div_up(m, 4)), RT, 0, st>>>(part, V, vstride, m, w, len, rstride, nc);
   count_launch();
   k_multidot2<<<dim3(m, nrhs), 128, 0, st>>>(res, part, m, nc, res_stride);
 }
@@ -399,7 +461,7 @@ void blas_multidot_df(cplx<double>* res, int res_stride, const cplx<double>* V, 
   const int nc = nchunks(len);
   double* part = partials((size_t)nrhs * m * nc * 2, st);
   count_launch();
-  k_multidot1_df<<<dim3(nc, nrhs), RT, 0, st>>>(part, V, vstride, m, w, len, rstride, nc);
+  k_multidot1_df<<<dim3(nc, nrhs, div_up(m, 4)), RT, 0, st>>>(part, V, vstride, m, w, len, rstride, nc);
   count_launch();
   k_multidot2<<<dim3(m, nrhs), 128, 0, st>>>(res, part, m, nc, res_stride);
 }
@@ -476,11 +538,11 @@ void blas_recip(double* a, int n, cudaStream_t st) { k_recip<<<div_up(n, 128), 1
 void gmres_begin(const GmresState& s, int nrhs, cudaStream_t st) { k_gmres_begin<<<div_up(nrhs, 32), 32, 0, st>>>(s, nrhs); }
 void gmres_step(const GmresState& s, int j, int nrhs, cudaStream_t st) {
   count_launch();
-  k_gmres_step<<<div_up(nrhs, 32), 32, 0, st>>>(s, j, nrhs);
+  k_gmres_step<<<nrhs, 32, 0, st>>>(s, j);
 }
 void gmres_solve_y(const GmresState& s, int nrhs, cudaStream_t st) {
   count_launch();
-  k_gmres_solve_y<<<div_up(nrhs, 32), 32, 0, st>>>(s, nrhs);
+  k_gmres_solve_y<<<nrhs, 32, 0, st>>>(s);
 }
 
 #define INST(T)                                                                                                 \
