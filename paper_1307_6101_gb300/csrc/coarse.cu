@@ -929,7 +929,7 @@ __device__ __forceinline__ void saph_block(cg::cluster_group& cluster, cplx<floa
 
 // one colour sweep: cluster c of the launch owns SAP block blocks[c]
 template <int RB, int RPL>
-__global__ void __launch_bounds__(32 * SAPH_W, 2) k_coarse_sap_h(cplx<float>* __restrict__ z,
+__global__ void __launch_bounds__(32 * SAPH_W, 2) k_csap_half(cplx<float>* __restrict__ z,
                                                                  const cplx<float>* __restrict__ bsrc,
                                                                  const __half2* __restrict__ blk,
                                                                  const float* __restrict__ bscale, Geom g, int n,
@@ -1024,7 +1024,7 @@ __device__ bool persist_grid_sync(unsigned* cnt, unsigned target, cg::cluster_gr
 }
 
 template <int RPL>
-__global__ void __launch_bounds__(32 * SAPH_W, 1) k_coarse_sap_persist(
+__global__ void __launch_bounds__(32 * SAPH_W, 1) k_csap_half_persist(
     cplx<float>* __restrict__ z, const cplx<float>* __restrict__ bsrc, const __half2* __restrict__ blk,
     const float* __restrict__ bscale, Geom g, int n, FDiv fn, size_t rstride, int nrhs,
     const int* __restrict__ blocks0, int nb0, const int* __restrict__ blocks1, int nb1, int k_mr, int spc, int nsl,
@@ -1372,11 +1372,11 @@ int saph_threads(const CoarseOp<float>& op) { return saph_threads(op.g.vB / op.s
 template <int RB>
 auto saph_kernel(int n) {
   const int r = saph_rpl(n);
-  return r == 8 ? k_coarse_sap_h<RB, 8> : r == 4 ? k_coarse_sap_h<RB, 4> : k_coarse_sap_h<RB, 2>;
+  return r == 8 ? k_csap_half<RB, 8> : r == 4 ? k_csap_half<RB, 4> : k_csap_half<RB, 2>;
 }
 auto saph_persist_kernel(const CoarseOp<float>& op) {
   const int r = saph_rpl(op.n);
-  return r == 8 ? k_coarse_sap_persist<8> : r == 4 ? k_coarse_sap_persist<4> : k_coarse_sap_persist<2>;
+  return r == 8 ? k_csap_half_persist<8> : r == 4 ? k_csap_half_persist<4> : k_csap_half_persist<2>;
 }
 void saph_attrs(const void* fn) {   // process-wide limits: the device maximum
   cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
