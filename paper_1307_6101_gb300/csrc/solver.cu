@@ -1256,7 +1256,7 @@ void galerkin(ddamg_handle* h, int l, const cplx<T>* P, Term term) {
       for (int j0 = 0; j0 < F.N; j0 += jb_max) {
         const int jb = std::min(jb_max, F.N - j0);
         const size_t at = (size_t)k * nc * nc + (size_t)(sp * F.N + j0) * nc;
-        if (!fits) {   // an aggregate of tens of thousands of sites
+        if (!fits) {   // one or two FP64 test vectors, or an aggregate of tens of thousands of sites
           blas_zero<T>(tmp, F.vlen, jb, F.vlen, h->st);
           term(tmp, P + (size_t)j0 * F.vlen, jb, sel, mu, sp);
           restrict_op<T>(cop<T>(C).blk + at, tmp, P, F.g, C.g, F.fine, F.n, F.N, jb, F.vlen, (size_t)nc,

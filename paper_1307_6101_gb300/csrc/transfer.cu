@@ -683,8 +683,12 @@ void orthonormalise(cplx<double>* P, const Geom& g, bool fine, int n, int N, int
 
 int galerkin_cols() { return GCMAX; }
 
+// FP64 with one or two test vectors: a 4 x 4 tile is mostly padding and a chunk of 64 rows too little in flight; the
+// rebuild of 24^3x48 with two takes 40.8 ms with these products and 24.6 with k_restrict, with four 53.9 and 68.5
+// (16^3x32: 8.4 and 5.6 ms with two, 11.0 and 14.2 with four, 73.6 and 128 with twenty).
 template <typename T>
 bool galerkin_fits(int N, int C, int vA) {
+  if (sizeof(T) == 8 && N <= 2) return false;
   return C >= 1 && C <= GCMAX && N <= 32 && galerkin_smem(N, C, vA, sizeof(cplx<T>)).total <= 200 * 1024;
 }
 
