@@ -1317,9 +1317,8 @@ void sap_cluster_attrs(size_t smem, int CLS) {
   if (CLS > 8) cudaFuncSetAttribute(k_coarse_sap_cluster<T, BS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
 }
 
-// cluster plan of the coarse SAP: cluster size CLS, sites per CTA and staged blocks per
-// site (0 if no plan fits).  Sized for operator storage in the compute precision, which
-// also covers the FP16 storage.
+// cluster plan of the coarse SAP on blocks in the compute precision: cluster size CLS, sites per CTA
+// and staged blocks per site (0, and nothing written, if no plan fits).
 template <typename T>
 int coarse_sap_cluster_plan(const Geom& g, int n, int* CLS_out, int* spc_out, int* nsl_out, int prefer) {
   const int nsl = coarse_sap_slots(g);
@@ -1359,11 +1358,13 @@ int coarse_sap_cluster_plan(const Geom& g, int n, int* CLS_out, int* spc_out, in
 
 // Persistent SAP on FP16 blocks (FP32 compute): the launch's shared memory and threads for nbpc
 // SAP blocks of each colour per cluster, and whether all clusters (max(nb0, nb1) / nbpc of
-// op.sap_cls CTAs) can be resident at once on this device.
+// op.saph_cls CTAs) can be resident at once on this device.  Cluster size and staged blocks per site
+// are those of the plan of the kernel on FP16 blocks (the other cluster kernel's plan refuses levels that
+// this one takes); 0 without a plan that stages every block inside the SAP block, which the MR steps read.
 size_t coarse_sap_persist_smem(const CoarseOp<float>& op, int nbpc) {
-  if (op.saph_cls <= 0) return 0;
+  if (op.saph_cls <= 0 || op.saph_nst < coarse_sap_slots(op.g)) return 0;
   const int spc = op.g.vB / op.saph_cls;
-  return saph_smem_layout(op.g.vB, op.n, spc, 1, 2 * nbpc * spc * op.sap_nsl, 2 * nbpc).total;
+  return saph_smem_layout(op.g.vB, op.n, spc, 1, 2 * nbpc * spc * op.saph_nst, 2 * nbpc).total;
 }
 
 namespace {
@@ -1391,13 +1392,13 @@ void saph_attrs(const void* fn) {   // process-wide limits: the device maximum
 // 128 blocks (32^4) 112 and 115, 377 and 271 for four right-hand sides.  Staging all nine blocks of a site: 25.0
 // and 42, 148 and 204 for one right-hand side (fewer clusters fit).
 int coarse_saph_plan(const Geom& g, int n, int nblocks, int* CLS_out, int* nst_out, int prefer) {
-  *CLS_out = 0;
-  *nst_out = coarse_sap_slots(g);
+  *CLS_out = *nst_out = 0;
+  const int nst = coarse_sap_slots(g);
   for (int pass = 0; pass < 2; ++pass)   // the second without the residency condition
     for (int CLS : {prefer, 16, 8, 4, 2}) {
       if ((CLS != 2 && CLS != 4 && CLS != 8 && CLS != 16) || g.vB % CLS) continue;
       const int spc = g.vB / CLS, rows = spc * n;
-      const size_t sm = saph_smem_layout(g.vB, n, spc, 1, *nst_out * spc, 1).total;
+      const size_t sm = saph_smem_layout(g.vB, n, spc, 1, nst * spc, 1).total;
       if (sm > 227 * 1024) continue;
       const void* fn = (const void*)saph_kernel<1>(n);
       saph_attrs(fn);
@@ -1420,6 +1421,7 @@ int coarse_saph_plan(const Geom& g, int n, int nblocks, int* CLS_out, int* nst_o
       }
       if (pass == 0 && CLS == 16 && CLS != prefer && nclusters < nblocks) continue;
       *CLS_out = CLS;
+      *nst_out = nst;
       return 1;
     }
   return 0;
@@ -1435,7 +1437,7 @@ bool coarse_sap_persist_fits(const CoarseOp<float>& op, int nb0, int nb1, int* m
   for (int nbpc = min_nbpc < 1 ? 1 : min_nbpc; nbpc <= 2; ++nbpc) {
     const int threads = saph_threads(op);
     const size_t sm = coarse_sap_persist_smem(op, nbpc);
-    if (sm > 227 * 1024) continue;
+    if (sm == 0 || sm > 227 * 1024) continue;
     const void* fn = (const void*)saph_persist_kernel(op);
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              227 * 1024) != cudaSuccess ||   // process-wide limit: the device maximum
@@ -1472,7 +1474,9 @@ cudaError_t coarse_sap_persist(cplx<float>* z, const cplx<float>* b, const Coars
                                int nb0, const int* blocks1, int nb1, int nrhs, size_t rstride, int k_mr, int iters,
                                int nbpc, unsigned* gcnt, cudaStream_t st) {
   if (nrhs <= 0 || iters <= 0) return cudaSuccess;
-  if (op.saph_cls <= 0 || !op.blkh || nb0 <= 0 || nb1 <= 0 || nbpc < 1 || nbpc > 2) return cudaErrorInvalidValue;
+  if (!op.blkh || nb0 <= 0 || nb1 <= 0 || nbpc < 1 || nbpc > 2) return cudaErrorInvalidValue;
+  const size_t sm = coarse_sap_persist_smem(op, nbpc);
+  if (sm == 0) return cudaErrorInvalidValue;
   const int CLS = op.saph_cls, spc = op.g.vB / CLS;
   const int nb = nb0 > nb1 ? nb0 : nb1;
   cudaError_t e = cudaMemsetAsync(gcnt, 0, sizeof(unsigned), st);
@@ -1487,13 +1491,13 @@ cudaError_t coarse_sap_persist(cplx<float>* z, const cplx<float>* b, const Coars
   attr[1].val.cooperative = 1;
   cfg.gridDim = dim3(((nb + nbpc - 1) / nbpc) * CLS, 1, 1);
   cfg.blockDim = dim3(saph_threads(op), 1, 1);
-  cfg.dynamicSmemBytes = coarse_sap_persist_smem(op, nbpc);
+  cfg.dynamicSmemBytes = sm;
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
   count_launch();
   return cudaLaunchKernelEx(&cfg, saph_persist_kernel(op), z, b, op.blkh, op.bscale, op.g, op.n, fdiv_make(op.n), rstride, nrhs, blocks0, nb0,
-                            blocks1, nb1, k_mr, spc, op.sap_nsl, nbpc, iters, op.err, op.bsite,
+                            blocks1, nb1, k_mr, spc, op.saph_nst, nbpc, iters, op.err, op.bsite,
                             op.bloc, gcnt);
 }
 

@@ -38,8 +38,8 @@ struct CoarseOp {
   int n_odd;
   int sap_cls;          // cluster size of the cluster SAP kernel (0: one CTA per SAP block)
   int sap_nsl = 0;      // blocks per site staged in shared memory by the cluster SAP kernel
-  int saph_cls = 0;     // the same two for the kernel on FP16 blocks
-  int saph_nst = 0;
+  int saph_cls = 0;     // the same two for the kernels on FP16 blocks (a launch per sweep, persistent), whose
+  int saph_nst = 0;     // plan is their own; 0 where it does not fit
   const int* bsite = nullptr;   // [nBlk][vB] sites of each SAP block (block-local order)
   const int* bloc = nullptr;    // [V] position of each site inside its SAP block
   int* err = nullptr;   // device error flag (bounded waits)
@@ -112,7 +112,8 @@ cudaError_t coarse_sap_sweep(cplx<T>* z, const cplx<T>* b, const CoarseOp<T>& op
 // stay resident (FP16 blocks, FP32 compute), nbpc (1 or 2) SAP blocks of each colour per cluster;
 // *gcnt: a device counter for the launch's barriers.  fits: the smallest nbpc for which all
 // clusters are resident at once (*max_clusters: clusters of that shape the device holds, -1: not
-// queried)
+// queried).  smem: 0 without a plan that stages every block inside a SAP block (nothing is launched then)
+int coarse_sap_slots(const Geom& g);
 size_t coarse_sap_persist_smem(const CoarseOp<float>& op, int nbpc);
 bool coarse_sap_persist_fits(const CoarseOp<float>& op, int nb0, int nb1, int* max_clusters = nullptr,
                              int* nbpc = nullptr, int min_nbpc = 1);

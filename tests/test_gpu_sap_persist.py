@@ -9,7 +9,7 @@ import numpy as np
 import pytest
 
 import synth
-from cases import Case, rel, THREE, BIG3
+from cases import Case, rel, THREE, BIG3, ODD3
 
 pytestmark = pytest.mark.gpu
 
@@ -55,6 +55,46 @@ def test_persistent_sap_matches_per_sweep_launches_and_oracle(dd, spec, form):
     sap = SAP(stencil_half(o.levels[1].op), c.sap[1], c.mr_steps)
     zref = np.stack([sap.smooth(b[i], z0[i], 3) for i in range(3)])
     assert rel(out[form], zref) <= TOL32, rel(out[form], zref)
+
+
+# widened level-1 SAP blocks (extents of 6 sites: 3-site blocks), which only the plan of the FP16 kernels takes
+WIDE = {
+    "24x24": dict(dims=(12, 8, 8, 8), levels=3, agg=((2, 2, 2, 2), (3, 2, 2, 2)), n_tv=(12, 12),
+                  sap=((2, 2, 2, 2), (2, 2, 2, 2))),
+    "24x32": dict(dims=(12, 8, 8, 8), levels=3, agg=((2, 2, 2, 2), (3, 2, 2, 2)), n_tv=(16, 16),
+                  sap=((2, 2, 2, 2), (2, 2, 2, 2))),
+    "24x40": dict(dims=(12, 8, 8, 8), levels=3, agg=((2, 2, 2, 2), (3, 2, 2, 2)), n_tv=(20, 20),
+                  sap=((2, 2, 2, 2), (2, 2, 2, 2))),
+    "36x16": dict(dims=(12, 12, 8, 8), levels=3, agg=((2, 2, 2, 2), (3, 3, 2, 2)), n_tv=(8, 8),
+                  sap=((2, 2, 2, 2), (2, 2, 2, 2))),
+    "54x8": ODD3,
+}
+
+
+@pytest.mark.parametrize("name", WIDE)
+def test_persistent_sap_on_widened_blocks(dd, name):
+    """Sites x dofs of a SAP block; 24 x 40 stages more than an SM's shared memory, so a launch per sweep runs there."""
+    from oracle.precision import stencil_half
+    from oracle.smoother import SAP
+    c = Case(**WIDE[name])
+    U = c.gauge()
+    tv = c.random_tv()
+    h, o = c.gpu(0, U, tv), c.oracle(U, tv)
+    dd.ddamg_set_option(h, dd.DDAMG_OPT_HALF_STORAGE, 1)
+    dims, n, _ = h.level_info(1)
+    assert dd.ddamg_get_option(h, dd.DDAMG_OPT_SAP_CLUSTER) > 0
+    b, z0 = _fields(3, dims, n, 61), _fields(3, dims, n, 62)
+    sap = SAP(stencil_half(o.levels[1].op), o.levels[1].sap.block, c.mr_steps)
+    zref = np.stack([sap.smooth(b[i], z0[i], 3) for i in range(3)])
+    out = []
+    for persist in (0, 1):
+        dd.ddamg_set_option(h, dd.DDAMG_OPT_SAP_PERSIST, persist)
+        assert dd.ddamg_get_option(h, dd.DDAMG_OPT_SAP_PERSIST) == (persist if name != "24x40" else 0)
+        z = z0.copy()
+        dd.ddamg_smooth(h, 1, 1, b, z, 3, 3)
+        assert rel(z, zref) <= TOL32, rel(z, zref)
+        out.append(z)
+    assert np.array_equal(out[0], out[1])
 
 
 def test_autotuner_records_the_sap_candidates(dd):

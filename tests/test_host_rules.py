@@ -1,0 +1,78 @@
+"""Host-side rules of the launchers that no GPU is needed for: a small program linked against the library calls
+them with no device visible.
+"""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+PKG = os.path.join(ROOT, "paper_1307_6101_gb300")
+
+PRELUDE = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "kernels.h"
+using namespace dd;
+#define CHECK(c) do { if (!(c)) { printf("line %d: %s\n", __LINE__, #c); return 1; } } while (0)
+// a lattice of two SAP blocks per direction
+static Geom geom(int b0, int b1, int b2, int b3) {
+  Geom g{};
+  const int B[4] = {b0, b1, b2, b3};
+  g.V = g.vB = 1;
+  for (int d = 0; d < 4; ++d) {
+    g.B[d] = B[d];
+    g.L[d] = 2 * B[d];
+    g.fB[d] = fdiv_make(B[d]);
+    g.vB *= B[d];
+    g.V *= g.L[d];
+  }
+  return g;
+}
+"""
+
+
+def run(tmp_path, body):
+    """Compile and run main() { PRELUDE; body } with no GPU visible."""
+    import __graft_entry__
+    __graft_entry__.build()
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not available")
+    src, exe = tmp_path / "t.cu", tmp_path / "t"
+    src.write_text(PRELUDE + "int main() {\n  int nd = 0;\n  if (cudaGetDeviceCount(&nd) == cudaSuccess && nd > 0) "
+                   "return 2;\n" + body + "\n  return 0;\n}\n")
+    cmd = [nvcc, "-gencode", "arch=compute_103a,code=sm_103a", "-std=c++17", "--expt-relaxed-constexpr", "-O0", "-I",
+           os.path.join(ROOT, "include"), "-I", os.path.join(PKG, "csrc"), str(src), os.path.join(PKG, "libddamg.so"),
+           "-Xlinker", "-rpath=" + PKG, "-o", str(exe)]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-2000:]
+    r = subprocess.run([str(exe)], capture_output=True, text=True, env={**os.environ, "CUDA_VISIBLE_DEVICES": ""})
+    assert r.returncode == 0, (r.returncode, r.stdout, r.stderr)
+
+
+def test_persistent_sap_stages_the_blocks_of_its_own_plan(tmp_path):
+    """Levels that only the plan of the FP16 kernels takes (sap_nsl stays 0 there): the persistent launch has room for
+    every block inside its SAP blocks, and refuses a plan that stages fewer."""
+    run(tmp_path, r"""
+  const int shapes[][5] = {{3, 2, 2, 2, 32}, {3, 3, 2, 2, 16}, {2, 3, 3, 3, 8}, {5, 2, 2, 2, 24}};
+  const int cls[] = {8, 4, 2, 8}, slots[] = {6, 7, 8, 6};
+  for (int t = 0; t < 4; ++t) {
+    CoarseOp<float> op{};
+    op.g = geom(shapes[t][0], shapes[t][1], shapes[t][2], shapes[t][3]);
+    op.n = shapes[t][4];
+    CHECK(coarse_sap_slots(op.g) == slots[t]);
+    op.saph_cls = cls[t];
+    op.saph_nst = slots[t];
+    const size_t nn = (size_t)op.n * op.n, spc = op.g.vB / cls[t];
+    for (int nbpc = 1; nbpc <= 2; ++nbpc)
+      CHECK(coarse_sap_persist_smem(op, nbpc) > 2 * nbpc * spc * slots[t] * nn * sizeof(__half2));
+    op.saph_nst = slots[t] - 1;
+    op.sap_nsl = slots[t];
+    CHECK(coarse_sap_persist_smem(op, 1) == 0);
+    op.saph_nst = 0;
+    CHECK(coarse_sap_persist_smem(op, 1) == 0);
+    CHECK(!coarse_sap_persist_fits(op, 4, 4));
+  }
+""")
