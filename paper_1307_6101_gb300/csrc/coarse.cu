@@ -561,6 +561,13 @@ __device__ __forceinline__ cplx<float> ldz(const cplx<float>* p) {
 struct SapHSmem {
   size_t zn, rf, pf, xa, zs, part, nbr, kof, nin, sc, voff, uoff, nu, pairs, np, flag, bar, total;
 };
+// A pair (own site of a CTA, CTA of the cluster) in 16 bits.  The exchanged vectors alone, 16 vB n bytes, keep a SAP
+// block below 7264 sites at n = 2, so a CTA of two or more has less than 4096 (and vB n below 2^15, as the positions
+// in r need, which are kept in shorts).
+constexpr int SAPH_SITES = 4096;   // most sites of a CTA
+DD_HD unsigned short saph_pair(int sl, int cta) { return (unsigned short)(sl << 4 | cta); }
+DD_HD int saph_pair_site(unsigned short p) { return p >> 4; }
+DD_HD int saph_pair_cta(unsigned short p) { return p & 15; }
 // nstage: staged blocks of the CTA; nblk: SAP blocks whose tables it keeps
 DD_HD SapHSmem saph_smem_layout(int vB, int n, int spc, int RB, int nstage, int nblk) {
   SapHSmem L;
@@ -658,7 +665,7 @@ __device__ __forceinline__ void saph_links(int n, int RB, int spc, int rank, uns
   const int* nin = reinterpret_cast<const int*>(smem + L.nin) + q * spc;
   const short* voff = reinterpret_cast<const short*>(smem + L.voff) + (size_t)q * spc * 9 * n;
   short* u = reinterpret_cast<short*>(smem + L.uoff) + q * 9 * spc;
-  short* pairs = reinterpret_cast<short*>(smem + L.pairs) + q * spc * 16;
+  unsigned short* pairs = reinterpret_cast<unsigned short*>(smem + L.pairs) + q * spc * 16;
   int cnt = 0, np = 0;
   for (int sl = 0; sl < spc; ++sl) u[cnt++] = (short)(rank * spc + sl);
   for (int sl = 0; sl < spc; ++sl) {
@@ -669,7 +676,7 @@ __device__ __forceinline__ void saph_links(int n, int RB, int spc, int rank, uns
       for (int e = 0; e < cnt; ++e) seen = seen || u[e] == loc;
       if (!seen) u[cnt++] = (short)loc;
       const int t = loc / spc;
-      if (!(to >> t & 1u)) pairs[np++] = (short)(sl << 8 | t);
+      if (!(to >> t & 1u)) pairs[np++] = saph_pair(sl, t);
       to |= 1u << t;
     }
   }
@@ -762,7 +769,7 @@ __device__ __forceinline__ void saph_block(cg::cluster_group& cluster, cplx<floa
   bool ok = staged();
   const int nu = reinterpret_cast<const int*>(smem + L.nu)[q];
   const int npair = reinterpret_cast<const int*>(smem + L.np)[q];
-  const short* pairs = reinterpret_cast<const short*>(smem + L.pairs) + q * spc * 16;
+  const unsigned short* pairs = reinterpret_cast<const unsigned short*>(smem + L.pairs) + q * spc * 16;
   // acc += column `h` of RPL rows times v
   auto column = [&](float (&acc)[NV], const HR& h, const C (&v)[RB]) {
 #pragma unroll
@@ -795,7 +802,7 @@ __device__ __forceinline__ void saph_block(cg::cluster_group& cluster, cplx<floa
     if (tid == 0)
       mbar_arrive_expect_tx(&xbar[buf], (unsigned)((nu - spc) * RB * n * sizeof(C) + CLS * RB * sizeof(float4)));
     for (int p = warp; p < npair; p += nw) {
-      const int sl = pairs[p] >> 8, t = pairs[p] & 255;
+      const int sl = saph_pair_site(pairs[p]), t = saph_pair_cta(pairs[p]);
       float4* o = reinterpret_cast<float4*>(d + (size_t)(rank * spc + sl) * RB * n);
       for (int e = lane; e < RB * n / 2; e += 32) st_async_cluster(o + e, o[e], &xbar[buf], t);
     }
@@ -1399,7 +1406,7 @@ int coarse_saph_plan(const Geom& g, int n, int nblocks, int* CLS_out, int* nst_o
       if ((CLS != 2 && CLS != 4 && CLS != 8 && CLS != 16) || g.vB % CLS) continue;
       const int spc = g.vB / CLS, rows = spc * n;
       const size_t sm = saph_smem_layout(g.vB, n, spc, 1, nst * spc, 1).total;
-      if (sm > 227 * 1024) continue;
+      if (sm > 227 * 1024 || spc > SAPH_SITES) continue;
       const void* fn = (const void*)saph_kernel<1>(n);
       saph_attrs(fn);
       saph_attrs((const void*)saph_kernel<2>(n));

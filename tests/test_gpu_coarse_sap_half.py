@@ -1,6 +1,7 @@
 """Coarse SAP on FP16 blocks (a cluster per SAP block): against the oracle on the same FP16 data for each cluster size, rows
 per warp of eight, four and two (dofs divisible by 8, 4 and 2), blocks that span a lattice direction (a neighbour in
-both directions), and one to three right-hand sides (pairs and a remainder).  FP32 bound: 2e-6 relative per sweep
+both directions), 192 sites to a CTA (384-site blocks on two CTAs), and one to three right-hand sides (pairs and a
+remainder).  FP32 bound: 2e-6 relative per sweep
 pair; a column has the same bits alone and in a batch.
 """
 import numpy as np
@@ -18,10 +19,12 @@ CASES = [
      (16, 8)),
     (dict(dims=(8, 4, 4, 4), levels=3, agg=((2, 2, 2, 2), (2, 1, 1, 1)), n_tv=(5, 6), sap=((2, 2, 2, 2), (2, 2, 2, 2))),
      (16, 4, 2)),
+    (dict(dims=(16, 8, 8, 12), levels=3, agg=((2, 2, 2, 2), (2, 2, 2, 2)), n_tv=(1, 1), sap=((2, 2, 2, 2), (4, 4, 4, 6))),
+     (2, 16)),
 ]
 
 
-@pytest.mark.parametrize("case,sizes", CASES, ids=["n24", "n20", "n10"])
+@pytest.mark.parametrize("case,sizes", CASES, ids=["n24", "n20", "n10", "n2"])
 def test_sweeps_against_oracle(case, sizes):
     import paper_1307_6101_gb300 as dd
     from oracle.precision import stencil_half
