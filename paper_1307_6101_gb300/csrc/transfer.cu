@@ -26,7 +26,10 @@ DD_HD size_t faddr(bool fine, int V, int n, int x, int f) {
 // belong to a group; a lane forms a tile of four rows and the group's columns, two rows of K at a time (128 FMAs for
 // 8 shared-memory loads at four columns).  The lanes that the ceil(N/4) row tiles leave free and the group's
 // warps split K, in a way that depends on the level only, so that a right-hand side has the same bits alone
-// and in a batch.
+// and in a batch.  A lane's products of a few chunks run in one chain and are then added to its part, so that neither
+// chain is long, and the parts are added with their rounding errors.  An FP16 column on 4^4 aggregates is off by
+// 0.9e-7 (8 test vectors) to 1.1e-7 (32) against 64 bits, 20 test vectors 1.0e-7; three chunks in one chain and plain sums of
+// the parts gave 1.33e-7 there, one lane per site and a butterfly over the lanes 1.11e-7 (6^4 aggregates 1.79e-7).
 // A chunk is whole runs of memory (sites of one component on the fine level, dofs of one site on a coarse one).
 // Where those are multiples of 16 bytes (BULK) one lane copies a run of a column with one bulk copy;
 // with a copy instruction per pair of elements the copies took two thirds of the issue slots.
@@ -37,7 +40,6 @@ constexpr int RKC = 128;    // most K rows of a chunk
 constexpr int RNG = 3;      // most groups of a CTA
 // columns of a group: one in FP64, where the FMAs bound the kernel and a column tile would only take registers
 template <typename T> constexpr int restrict_ct() { return sizeof(T) == 4 ? 4 : 1; }
-constexpr int RFLUSH = 3;      // chunks whose products run into one accumulator
 constexpr int RKP = RKC + 12;  // row pitch of P (elements): a multiple of 16 bytes, the row tiles of a warp on different banks
 constexpr int RKB = RKC + 2;   // row pitch of the columns
 
@@ -63,6 +65,15 @@ inline int restrict_chunk(int run, int ps, bool bulk) {
     if (run % d == 0 && d % 2 == 0 && !(bulk && d * ps % 16)) return d;
   return 0;
 }
+
+// (hi, lo) += x without rounding error beyond lo's (Knuth's two-sum)
+__device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float x) {
+  const float s = __fadd_rn(hi, x), t = __fsub_rn(s, hi);
+  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(x, t)));
+  hi = s;
+}
+// the sum that (hi, lo) hold; with an infinite hi, whose rounding error is not a number, hi
+__device__ __forceinline__ float two_sum(float hi, float lo) { return isfinite(hi) ? hi + lo : hi; }
 
 // two neighbouring elements of P in shared memory as complex numbers
 __device__ __forceinline__ void ld_pair(const __half2* p, cplx<float> a[2]) {
@@ -145,6 +156,10 @@ __global__ void __launch_bounds__(RNG * RTH, sizeof(T) == 4 ? 2 : 1) k_restrict(
     mbar_init(&bar[1], 1);
   }
   if (BULK) __syncthreads();
+  // chunks per chain: chains of `per` FMAs a chunk and nch / flush sums of them err least near flush^2 = nch / per
+  const int nch = (K + kch - 1) / kch, per = 4 * ((kch / 2 + (RTH / 32) * nsub - 1) / ((RTH / 32) * nsub));
+  int flush = 1;
+  while (flush * (flush + 1) * per < nch) ++flush;
   cplx<T> acc[4][RCT];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
@@ -184,8 +199,7 @@ __global__ void __launch_bounds__(RNG * RTH, sizeof(T) == 4 ? 2 : 1) k_restrict(
             }
           }
       }
-      // long sums in parts: their rounding errors do not add up along the whole of K
-      if (chunk % RFLUSH == RFLUSH - 1 || last) {
+      if (chunk % flush == flush - 1 || last) {
         cplx<T>* mine = red + (size_t)grp * 4 * RCT * slots + (warp * nsub + sub) * TI + ti;
 #pragma unroll
         for (int i = 0; i < 4; ++i)
@@ -193,7 +207,7 @@ __global__ void __launch_bounds__(RNG * RTH, sizeof(T) == 4 ? 2 : 1) k_restrict(
           for (int c = 0; c < RCT; ++c)
             if (c < gc) {
               cplx<T>& m = mine[(i * RCT + c) * slots];
-              m = chunk < RFLUSH ? acc[i][c] : m + acc[i][c];
+              m = chunk < flush ? acc[i][c] : m + acc[i][c];
               acc[i][c] = czero<T>();
             }
       }
@@ -214,11 +228,30 @@ __global__ void __launch_bounds__(RNG * RTH, sizeof(T) == 4 ? 2 : 1) k_restrict(
   for (int e = tid; e < N * C; e += blockDim.x) {
     const int c = e / N, i = e - c * N;
     const cplx<T>* r = red + ((size_t)(c / RCT) * 4 * RCT + i / TI * RCT + c % RCT) * slots + i % TI;
-    cplx<T> t[4] = {czero<T>(), czero<T>(), czero<T>(), czero<T>()};   // the parts in four chains
+    cplx<T> t[4] = {czero<T>(), czero<T>(), czero<T>(), czero<T>()};   // the parts in four chains, FP32 with their
+    cplx<T> lo[4] = {czero<T>(), czero<T>(), czero<T>(), czero<T>()};  // rounding errors
     for (int q = 0; q < (RTH / 32) * nsub; q += 4)
 #pragma unroll
-      for (int u = 0; u < 4; ++u) t[u] = t[u] + r[(q + u) * TI];
-    po[(size_t)c * out_rstride + i] = sc * ((t[0] + t[1]) + (t[2] + t[3]));
+      for (int u = 0; u < 4; ++u) {
+        const cplx<T> p = r[(q + u) * TI];
+        if constexpr (sizeof(T) == 4) {
+          two_sum_acc(t[u].re, lo[u].re, p.re);
+          two_sum_acc(t[u].im, lo[u].im, p.im);
+        } else {
+          t[u] = t[u] + p;
+        }
+      }
+    if constexpr (sizeof(T) == 4) {
+#pragma unroll
+      for (int u = 1; u < 4; ++u) {
+        two_sum_acc(t[0].re, lo[0].re, t[u].re);
+        two_sum_acc(t[0].im, lo[0].im, t[u].im);
+        lo[0] = lo[0] + lo[u];
+      }
+      po[(size_t)c * out_rstride + i] = sc * cmk(two_sum(t[0].re, lo[0].re), two_sum(t[0].im, lo[0].im));
+    } else {
+      po[(size_t)c * out_rstride + i] = sc * ((t[0] + t[1]) + (t[2] + t[3]));
+    }
   }
 }
 
@@ -275,13 +308,6 @@ DD_HD GalerkinSmem galerkin_smem(int N, int C, int vA, size_t cs) {
   L.list = L.red + (size_t)(cs == sizeof(cplx<float>) ? 2 : 1) * (GT / 32) * nsub * tiles * 16 * cs;
   L.total = L.list + (size_t)vA * sizeof(int);
   return L;
-}
-
-// (hi, lo) += x without rounding error beyond lo's (Knuth's two-sum)
-__device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float x) {
-  const float s = __fadd_rn(hi, x), t = __fsub_rn(s, hi);
-  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(x, t)));
-  hi = s;
 }
 
 template <typename T>
@@ -416,7 +442,7 @@ __global__ void __launch_bounds__(GT) k_galerkin(cplx<double>* __restrict__ out,
         two_sum_acc(hi.im, lo.im, h.im);
         lo = lo + l;
       }
-      po[(size_t)c * out_rstride + i] = cmk((double)(hi.re + lo.re), (double)(hi.im + lo.im));
+      po[(size_t)c * out_rstride + i] = cmk((double)two_sum(hi.re, lo.re), (double)two_sum(hi.im, lo.im));
       continue;
     }
     cplx<T> t[4] = {czero<T>(), czero<T>(), czero<T>(), czero<T>()};   // the parts in four chains
