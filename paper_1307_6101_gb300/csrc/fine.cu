@@ -1809,17 +1809,15 @@ void launch_sap_plain(cplx<T>* z, const cplx<T>* b, const LS* U, const CS* clov,
 }
 
 template <typename T>
-void fine_sap_sweep(cplx<T>* z, const cplx<T>* b, const FineOp<T>& op, const int* blocks, int nblocks, int nrhs,
-                    size_t rstride, int k_mr, cudaStream_t st) {
-  if (nrhs < 1 || nblocks < 1) return;   // the staged kernels issue their copies before the rhs loop
+cudaError_t fine_sap_sweep(cplx<T>* z, const cplx<T>* b, const FineOp<T>& op, const int* blocks, int nblocks, int nrhs,
+                           size_t rstride, int k_mr, cudaStream_t st) {
+  if (nrhs < 1 || nblocks < 1) return cudaSuccess;   // the staged kernels issue their copies before the rhs loop
   if constexpr (sizeof(T) == 8) {
     // Six threads per site, except where blocks of more than 64 sites (a cluster per block) are enough of
     // them to fill the chip with one thread per site: 4^4 blocks, 128 per colour: 670 us per sweep with
     // six threads and 540 with one, 16 per colour: 195 and 530.
-    if (op.g.vB <= 64 || nblocks < 96)
-      fine_sap_split(z, b, op, blocks, nblocks, nrhs, rstride, k_mr, st);   // a refused launch: the last error
-    else
-      launch_sap_plain<T, cplx<T>, T>(z, b, op.U, op.clov, op, blocks, nblocks, nrhs, rstride, k_mr, T(0), st);
+    if (op.g.vB <= 64 || nblocks < 96) return fine_sap_split(z, b, op, blocks, nblocks, nrhs, rstride, k_mr, st);
+    launch_sap_plain<T, cplx<T>, T>(z, b, op.U, op.clov, op, blocks, nblocks, nrhs, rstride, k_mr, T(0), st);
   } else {
     const bool tma = sap_tma_ok(op) && op.err;
     const bool b4 = op.err && sap_b4_ok(op, z, rstride);
@@ -1853,6 +1851,7 @@ void fine_sap_sweep(cplx<T>* z, const cplx<T>* b, const FineOp<T>& op, const int
       launch_sap_plain<T, cplx<T>, T>(z, b, op.U, op.clov, op, blocks, nblocks, nrhs, rstride, k_mr, T(0), st);
     }
   }
+  return cudaPeekAtLastError();
 }
 
 __global__ void k_links_to_half(__half2* __restrict__ dst, const cplx<double>* __restrict__ U, size_t n) {
@@ -2034,7 +2033,7 @@ int fine_residual_norm_noalloc(double* out, bool out_on_device, const cplx<doubl
 #define INST(T)                                                                                              \
   template void fine_dslash<T>(cplx<T>*, const cplx<T>*, const cplx<T>*, const FineOp<T>&, int, size_t, int, \
                                int, int, cudaStream_t);                                                      \
-  template void fine_sap_sweep<T>(cplx<T>*, const cplx<T>*, const FineOp<T>&, const int*, int, int, size_t, \
+  template cudaError_t fine_sap_sweep<T>(cplx<T>*, const cplx<T>*, const FineOp<T>&, const int*, int, int, size_t, \
                                   int, cudaStream_t);                                                        \
   template void links_import<T>(cplx<T>*, const cplx<double>*, const Geom&, cudaStream_t);                  \
   template void fine_import<T>(cplx<T>*, const cplx<double>*, const Geom&, int, size_t, cudaStream_t);      \

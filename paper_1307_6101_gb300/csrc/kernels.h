@@ -56,11 +56,12 @@ void set_gamma_products(const double* gg);
 template <typename T>
 void fine_dslash(cplx<T>* out, const cplx<T>* in, const cplx<T>* b, const FineOp<T>& op, int nrhs, size_t rstride,
                  int sel, int sel_mu, int in_chir, cudaStream_t st);
+// one SAP colour sweep; not cudaSuccess: nothing was launched
 template <typename T>
-void fine_sap_sweep(cplx<T>* z, const cplx<T>* b, const FineOp<T>& op, const int* blocks, int nblocks, int nrhs,
-                    size_t rstride, int k_mr, cudaStream_t st);
+cudaError_t fine_sap_sweep(cplx<T>* z, const cplx<T>* b, const FineOp<T>& op, const int* blocks, int nblocks, int nrhs,
+                           size_t rstride, int k_mr, cudaStream_t st);
 // FP64 with six threads per site (fine_split.cu): the full operator (b set: b - D in), and one SAP
-// colour sweep
+// colour sweep (cudaErrorInvalidConfiguration, nothing launched, above 1024 sites in a block)
 void fine_dslash_split(cplx<double>* out, const cplx<double>* in, const cplx<double>* b, const FineOp<double>& op,
                        int nrhs, size_t rstride, cudaStream_t st);
 cudaError_t fine_sap_split(cplx<double>* z, const cplx<double>* b, const FineOp<double>& op, const int* blocks,

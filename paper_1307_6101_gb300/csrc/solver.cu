@@ -362,7 +362,7 @@ void sap(ddamg_handle* h, Level& L, cplx<T>* z, const cplx<T>* b, int nrhs, int 
       if (L.nblocks[c] == 0) continue;
       Prof pr(h, L.fine ? DDAMG_PROF_FINE_SAP : DDAMG_PROF_COARSE_SAP, sap_bytes<T>(L, c, nrhs, half_on<T>(h)));
       if (L.fine)
-        fine_sap_sweep<T>(z, b, fop<T>(L), L.blocks[c], L.nblocks[c], nrhs, L.vlen, h->p.mr_steps, h->st);
+        CK(fine_sap_sweep<T>(z, b, fop<T>(L), L.blocks[c], L.nblocks[c], nrhs, L.vlen, h->p.mr_steps, h->st));
       else
         CK(coarse_sap_sweep<T>(z, b, cop<T>(L), L.blocks[c], L.nblocks[c], nrhs, L.vlen, h->p.mr_steps, h->st));
     }

@@ -76,3 +76,18 @@ def test_persistent_sap_stages_the_blocks_of_its_own_plan(tmp_path):
     CHECK(!coarse_sap_persist_fits(op, 4, 4));
   }
 """)
+
+
+def test_fine_sap_sweep_reports_a_refused_launch(tmp_path):
+    """A block that six threads per site cannot hold, and a launch that the runtime refuses: the caller learns of both."""
+    run(tmp_path, r"""
+  FineOp<double> op{};
+  op.g = geom(8, 8, 8, 4);
+  CHECK(fine_sap_sweep<double>(nullptr, nullptr, op, nullptr, 4, 1, 0, 3, nullptr) == cudaErrorInvalidConfiguration);
+  op.g = geom(2, 2, 2, 2);
+  CHECK(fine_sap_sweep<double>(nullptr, nullptr, op, nullptr, 4, 1, 0, 3, nullptr) != cudaSuccess);
+  CHECK(fine_sap_sweep<double>(nullptr, nullptr, op, nullptr, 0, 1, 0, 3, nullptr) == cudaSuccess);
+  FineOp<float> f{};
+  f.g = geom(2, 2, 2, 2);
+  CHECK(fine_sap_sweep<float>(nullptr, nullptr, f, nullptr, 4, 1, 0, 3, nullptr) != cudaSuccess);
+""")
