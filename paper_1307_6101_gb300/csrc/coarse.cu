@@ -5,7 +5,6 @@
 // 5..8 backward, so that the threads computing consecutive rows of one site
 // read consecutive words.
 #include <atomic>
-#include <mutex>
 
 #include <cooperative_groups.h>
 
@@ -1566,11 +1565,12 @@ cudaError_t coarse_sap_sweep(cplx<T>* z, const cplx<T>* b, const CoarseOp<T>& op
   // compiled kernel, the same on every device of this architecture); the entries are atomics
   // because serving workers launch from several host threads
   static std::atomic<int> maxthr[2][2][3];   // [FP64][FP16 blocks][rpt 1, 4, 8]; 0 = not queried
+  static DeviceOnce once[2][2][3];
   std::atomic<int>* mt = maxthr[sizeof(T) == 8][half ? 1 : 0];
   auto query = [&](const void* fn, int q) {
+    raise_smem_limit(once[sizeof(T) == 8][half ? 1 : 0][q], fn);
     int v = mt[q].load(std::memory_order_acquire);
     if (v == 0) {
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
       cudaFuncAttributes a;
       v = cudaFuncGetAttributes(&a, fn) == cudaSuccess ? a.maxThreadsPerBlock : -1;
       cudaGetLastError();
@@ -1664,11 +1664,8 @@ void coarse_schur_even(cplx<T>* y, const cplx<T>* x, const cplx<T>* t, const cpl
 
 void coarse_selfinv_build(cplx<double>* inv, const cplx<double>* blk, int V, int n, int* err, cudaStream_t st) {
   const size_t sm = ((size_t)n * 2 * n + n) * sizeof(cplx<double>);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_selfinv_build, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    attr = true;
-  }
+  static DeviceOnce once;
+  raise_smem_limit(once, (const void*)k_selfinv_build);
   count_launch();
   k_selfinv_build<<<V, 256, sm, st>>>(inv, blk, n, err);
 }

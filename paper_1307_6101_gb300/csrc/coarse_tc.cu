@@ -22,7 +22,6 @@
 #include "tma.cuh"
 
 #include <atomic>
-#include <mutex>
 
 namespace {
 
@@ -223,19 +222,10 @@ __global__ void k_coarse_apply_tc(cplx<float>* __restrict__ out, const cplx<floa
   }
 }
 
-// The dynamic shared-memory limit is a process-wide attribute of the kernel: it only ever grows
-// (under a lock, so that two threads preparing different sizes cannot leave it at the smaller)
 template <bool RESID>
-cudaError_t prepare_tc(size_t bytes) {
-  static std::atomic<size_t> set_to{0};
-  static std::mutex mu;
-  if (set_to.load(std::memory_order_acquire) >= bytes) return cudaSuccess;
-  std::lock_guard<std::mutex> lk(mu);
-  if (set_to.load(std::memory_order_relaxed) >= bytes) return cudaSuccess;
-  const cudaError_t e =
-      cudaFuncSetAttribute(k_coarse_apply_tc<RESID>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e == cudaSuccess) set_to.store(bytes, std::memory_order_release);
-  return e;
+cudaError_t prepare_tc() {
+  static dd::DeviceOnce once;
+  return dd::raise_smem_limit(once, (const void*)k_coarse_apply_tc<RESID>);
 }
 
 }  // namespace
@@ -277,12 +267,12 @@ cudaError_t coarse_apply_tc(cplx<float>* out, const cplx<float>* in, const cplx<
   const int threads = 32 * L.mt * ks;
   count_launch();
   if (b) {
-    const cudaError_t e = prepare_tc<true>(L.total);
+    const cudaError_t e = prepare_tc<true>();
     if (e != cudaSuccess) return e;
     k_coarse_apply_tc<true><<<grid, threads, L.total, st>>>(out, in, b, op.blkh, op.bscale, op.g, op.n, rstride,
                                                             nrhs, ks, op.err);
   } else {
-    const cudaError_t e = prepare_tc<false>(L.total);
+    const cudaError_t e = prepare_tc<false>();
     if (e != cudaSuccess) return e;
     k_coarse_apply_tc<false><<<grid, threads, L.total, st>>>(out, in, b, op.blkh, op.bscale, op.g, op.n, rstride,
                                                              nrhs, ks, op.err);

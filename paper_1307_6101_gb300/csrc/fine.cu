@@ -1691,11 +1691,8 @@ void launch_sap_tma(cplx<T>* z, const cplx<T>* b, const LS* U, const CS* clov, c
   const size_t seg_bytes =
       (size_t)op.g.vB * (36 * sizeof(LS) + 2 * ClovRows<CS>::per_chir * sizeof(CS) + 12 * sizeof(cplx<T>));
   const size_t sm = segs * seg_bytes + 16 + (threads / 32) * 3 * sizeof(T) + 16;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_fine_sap_tma<T, LS, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    attr = true;
-  }
+  static DeviceOnce once;
+  raise_smem_limit(once, (const void*)k_fine_sap_tma<T, LS, CS>);
   count_launch();
   k_fine_sap_tma<T, LS, CS><<<div_up(nblocks, segs), threads, sm, st>>>(z, b, U, clov, op.g, op.bc_t, rstride, nrhs,
                                                                        blocks, nblocks, seg, k_mr, op.err, shift);
@@ -1747,10 +1744,8 @@ void launch_sap_b4(cplx<float>* z, const cplx<float>* b, const LS* U, const CS* 
   constexpr int VB = 256;
   const size_t sm = (size_t)VB * (36 * sizeof(LS) + 2 * ClovRows<CS>::per_chir * sizeof(CS) + 12 * sizeof(cplx<float>)) +
                     16 + 2 * 24 * sizeof(float);
-  static std::once_flag attr;
-  std::call_once(attr, [&] {
-    cudaFuncSetAttribute(k_fine_sap_b4<LS, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  });
+  static DeviceOnce once;
+  raise_smem_limit(once, (const void*)k_fine_sap_b4<LS, CS>);
   count_launch();
   // programmatic stream serialization: consecutive colour sweeps overlap the next sweep's operator
   // staging with the end of the previous one (the kernel waits for the previous grid before it
@@ -1780,10 +1775,8 @@ void launch_sap_b4_eo(cplx<float>* z, const cplx<float>* b, const LS* U, const C
   constexpr int VB = 256;
   const size_t sm = (size_t)VB * (36 * sizeof(LS) + 2 * ClovRows<CS>::per_chir * sizeof(CS) + 12 * sizeof(cplx<float>)) +
                     (size_t)12 * 128 * sizeof(cplx<float>) + 16 + 2 * 12 * sizeof(float);
-  static std::once_flag attr;
-  std::call_once(attr, [&] {
-    cudaFuncSetAttribute(k_fine_sap_b4_eo<LS, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-  });
+  static DeviceOnce once;
+  raise_smem_limit(once, (const void*)k_fine_sap_b4_eo<LS, CS>);
   count_launch();
   k_fine_sap_b4_eo<LS, CS><<<nblocks, 128, sm, st>>>(z, b, U, mix, op.g, op.bc_t, rstride, nrhs, blocks, k_mr, op.err,
                                                      shift);
@@ -1797,11 +1790,8 @@ void launch_sap_plain(cplx<T>* z, const cplx<T>* b, const LS* U, const CS* clov,
   const int threads = seg >= 256 ? seg : 256;
   const int segs = threads / seg;
   const size_t sm = (size_t)threads * 12 * sizeof(cplx<T>) + (size_t)(threads / 32) * 3 * sizeof(T);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_fine_sap<T, LS, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    attr = true;
-  }
+  static DeviceOnce once;
+  raise_smem_limit(once, (const void*)k_fine_sap<T, LS, CS>);
   dim3 grid(div_up(nblocks, segs), nrhs);
   count_launch();
   k_fine_sap<T, LS, CS><<<grid, threads, sm, st>>>(z, b, U, clov, op.g, op.bc_t, rstride, blocks, nblocks, seg, k_mr,

@@ -16,8 +16,6 @@
 #include "common.cuh"
 #include "kernels.h"
 
-#include <mutex>
-
 namespace cg = cooperative_groups;
 
 namespace {
@@ -353,11 +351,9 @@ cudaError_t fine_sap_split(cplx<double>* z, const cplx<double>* b, const FineOp<
   const int threads = ((6 * S + 31) / 32) * 32;
   const size_t sm = (size_t)66 * S * sizeof(cplx<double>) + (72 + 6 * MAXCLS) * sizeof(double) + (size_t)8 * S * sizeof(short);
   if (threads > 768 || sm > 227 * 1024) return cudaErrorInvalidConfiguration;
-  static std::once_flag attr_once;
-  std::call_once(attr_once, [] {
-    cudaFuncSetAttribute(k_fine_sap_split<384>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    cudaFuncSetAttribute(k_fine_sap_split<768>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-  });
+  static DeviceOnce once384, once768;
+  if (threads <= 384) raise_smem_limit(once384, (const void*)k_fine_sap_split<384>);
+  else raise_smem_limit(once768, (const void*)k_fine_sap_split<768>);
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;

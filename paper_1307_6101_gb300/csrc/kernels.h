@@ -1,10 +1,42 @@
 // Internal launch API of the DD-alpha-AMG CUDA library (not part of the C ABI).
 #pragma once
 
+#include <atomic>
+
 #include "common.cuh"
 #include "dfloat.cuh"
 
 namespace dd {
+
+// Once per device of the process: kernel attributes belong to a device, and hierarchies may live on several.
+// Failures are tried again by the next call; two threads may both run f.
+class DeviceOnce {
+  std::atomic<unsigned long long> done_{0};
+
+ public:
+  template <class F>
+  cudaError_t run(int device, F f) {
+    const unsigned long long bit = device >= 0 && device < 64 ? 1ull << device : 0;   // others: every time
+    if (done_.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    const cudaError_t e = f();
+    if (e == cudaSuccess) done_.fetch_or(bit, std::memory_order_release);
+    return e;
+  }
+};
+
+// The dynamic shared memory that kernel fn may be launched with, raised to the current device's maximum (not to
+// one launch's size: a later, smaller launch must not lower it for an earlier, larger one)
+inline cudaError_t raise_smem_limit(DeviceOnce& once, const void* fn) {
+  int device = 0;
+  const cudaError_t e = cudaGetDevice(&device);
+  if (e != cudaSuccess) return e;
+  return once.run(device, [&] {
+    cudaFuncAttributes a;
+    const cudaError_t q = cudaFuncGetAttributes(&a, fn);
+    if (q != cudaSuccess) return q;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - (int)a.sharedSizeBytes);
+  });
+}
 
 // number of kernels this library has launched (all streams, all handles)
 void count_launch(int k = 1);

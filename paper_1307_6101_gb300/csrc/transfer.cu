@@ -9,7 +9,6 @@
 #include "kernels.h"
 #include "tma.cuh"
 
-#include <mutex>
 #include <type_traits>
 
 namespace {
@@ -631,11 +630,6 @@ void restrict_op(cplx<T>* out, const cplx<T>* in, const cplx<T>* P, const Geom& 
   const size_t pstride = (size_t)gf.V * n;
   auto launch = [&](auto* Ps, const float* scale) {
     using PS = std::remove_const_t<std::remove_pointer_t<decltype(Ps)>>;
-    static std::once_flag attr;
-    std::call_once(attr, [] {
-      cudaFuncSetAttribute(k_restrict<T, PS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-      cudaFuncSetAttribute(k_restrict<T, PS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    });
     constexpr int RCT = restrict_ct<T>();
     // bulk copies: whole runs of multiples of 16 bytes at 16-byte aligned addresses, in P and in the columns (the
     // smaller elements decide)
@@ -652,6 +646,8 @@ void restrict_op(cplx<T>* out, const cplx<T>* in, const cplx<T>* P, const Geom& 
     while (groups > 1 && restrict_smem<T>(N, groups, pb).total > 110 * 1024) --groups;
     const unsigned grid = (unsigned)gf.nAgg * 2u * (unsigned)((nrhs + RCT * groups - 1) / (RCT * groups));
     auto kernel = bulk ? k_restrict<T, PS, true> : k_restrict<T, PS, false>;
+    static DeviceOnce once[2];
+    raise_smem_limit(once[bulk], (const void*)kernel);
     count_launch();
     kernel<<<grid, groups * RTH, restrict_smem<T>(N, groups, pb).total, st>>>(
         out, in, Ps, scale, gf, fine, n, N, nrhs, in_rstride, pstride, out_rstride, out_site_stride, kch,
@@ -696,10 +692,8 @@ void prolong_op(cplx<T>* out, const cplx<T>* in, const cplx<T>* P, const Geom& g
 void orthonormalise(cplx<double>* P, const Geom& g, bool fine, int n, int N, int* err, cudaStream_t st) {
   const size_t pstride = (size_t)g.V * n;
   const size_t sm = (size_t)g.vA * (n / 2) * sizeof(cplx<double>);   // the column in work
-  static std::once_flag attr;
-  std::call_once(attr, [] {
-    cudaFuncSetAttribute(k_orthonormalise<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  });
+  static DeviceOnce once;
+  raise_smem_limit(once, (const void*)k_orthonormalise<true>);
   count_launch();
   if (sm <= 200 * 1024)
     k_orthonormalise<true><<<dim3(g.nAgg, 2), OT, sm, st>>>(P, g, fine, n, N, pstride, err);
@@ -724,10 +718,8 @@ cudaError_t galerkin_restrict(cplx<double>* out, const cplx<T>* tmp, const cplx<
                               size_t out_site_stride, int sel, int sel_mu, cudaStream_t st) {
   const size_t sm = galerkin_smem(N, C, gf.vA, sizeof(cplx<T>)).total;
   if (!galerkin_fits<T>(N, C, gf.vA)) return cudaErrorInvalidValue;
-  static std::once_flag attr;
-  std::call_once(attr, [] {
-    cudaFuncSetAttribute(k_galerkin<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  });
+  static DeviceOnce once;
+  raise_smem_limit(once, (const void*)k_galerkin<T>);
   count_launch();
   k_galerkin<T><<<dim3(gf.nAgg, 2), GT, sm, st>>>(out, tmp, P, gf, fine, n, N, C, tmp_rstride, (size_t)gf.V * n,
                                                   out_rstride, out_site_stride, sel, sel_mu);

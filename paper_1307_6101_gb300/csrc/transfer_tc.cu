@@ -16,9 +16,6 @@
 #include "common.cuh"
 #include "kernels.h"
 
-#include <atomic>
-#include <mutex>
-
 namespace {
 
 constexpr int RT_R = 16;     // right-hand sides per CTA of the restriction
@@ -299,18 +296,6 @@ __global__ void __launch_bounds__(256, 3) k_prolong_batch(cplx<float>* __restric
   }
 }
 
-// the kernel's dynamic shared-memory limit (process-wide) only ever grows, under a lock
-cudaError_t prepare_restrict_tc(size_t bytes) {
-  static std::atomic<size_t> set_to{0};
-  static std::mutex mu;
-  if (set_to.load(std::memory_order_acquire) >= bytes) return cudaSuccess;
-  std::lock_guard<std::mutex> lk(mu);
-  if (set_to.load(std::memory_order_relaxed) >= bytes) return cudaSuccess;
-  const cudaError_t e = cudaFuncSetAttribute(k_restrict_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e == cudaSuccess) set_to.store(bytes, std::memory_order_release);
-  return e;
-}
-
 }  // namespace
 
 namespace dd {
@@ -326,7 +311,8 @@ cudaError_t restrict_tc(cplx<float>* out, const cplx<float>* in, const __half2* 
   if (nrhs <= 0) return cudaSuccess;
   if (!Ph || !restrict_tc_fits(N, ks)) return cudaErrorInvalidValue;
   const size_t bytes = rt_smem(N, ks);
-  const cudaError_t e = prepare_restrict_tc(bytes);
+  static DeviceOnce once;
+  const cudaError_t e = raise_smem_limit(once, (const void*)k_restrict_tc);
   if (e != cudaSuccess) return e;
   const int threads = 32 * ((2 * N + 15) / 16) * ks;
   count_launch();

@@ -91,3 +91,21 @@ def test_fine_sap_sweep_reports_a_refused_launch(tmp_path):
   f.g = geom(2, 2, 2, 2);
   CHECK(fine_sap_sweep<float>(nullptr, nullptr, f, nullptr, 4, 1, 0, 3, nullptr) != cudaSuccess);
 """)
+
+
+def test_attributes_are_set_once_per_device(tmp_path):
+    """A kernel's shared-memory limit belongs to a device: each device of the process gets it once, a failure is tried
+    again, and without a device nothing is marked as done."""
+    run(tmp_path, r"""
+  DeviceOnce once;
+  int calls = 0;
+  auto count = [&] { ++calls; return cudaSuccess; };
+  for (int round = 0; round < 2; ++round)
+    for (int device : {0, 1, 63}) CHECK(once.run(device, count) == cudaSuccess);
+  CHECK(calls == 3);
+  CHECK(once.run(2, [&] { ++calls; return cudaErrorInvalidValue; }) == cudaErrorInvalidValue);
+  CHECK(once.run(2, count) == cudaSuccess && calls == 5);
+  CHECK(once.run(64, count) == cudaSuccess && once.run(64, count) == cudaSuccess && calls == 7);
+  DeviceOnce limit;
+  CHECK(raise_smem_limit(limit, nullptr) != cudaSuccess);
+""")
