@@ -158,7 +158,10 @@ struct ddamg_handle {
   cplx<double>* ox = nullptr;
   cplx<float>* pin32 = nullptr;
   cplx<float>* pout32 = nullptr;
-  int* d_err = nullptr;
+  // error flag of the kernels: 1 a singular block or dependent vectors, 2 a staging wait and 3 a barrier that ran out;
+  // in pinned host memory, so that every call can look at it after its synchronisation
+  int* h_err = nullptr;
+  int* d_err = nullptr;       // its device address
   int* h_done = nullptr;      // pinned
   double* h_scal = nullptr;   // pinned
   int* h_kr = nullptr;        // pinned
@@ -951,16 +954,18 @@ void gamma_products(double* out /* [6][4][4][2] */) {
         }
 }
 
+// Waits for the handle's stream and reports (once) what its kernels flagged; what: the meaning of flag 1 here
 void check_err_flag(ddamg_handle* h, const char* what) {
-  int e = 0;
-  CK(cudaMemcpyAsync(&e, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, h->st));
   sync(h);
-  if (e) {
-    CK(cudaMemsetAsync(h->d_err, 0, sizeof(int), h->st));
-    sync(h);
-    fail(DDAMG_ERR_SINGULAR, what);
-  }
+  const int e = *const_cast<volatile int*>(h->h_err);
+  if (!e) return;
+  *h->h_err = 0;
+  if (e == 2) fail(DDAMG_ERR_CUDA, "a shared-memory staging wait of a kernel timed out");
+  if (e == 3) fail(DDAMG_ERR_CUDA, "a barrier of the persistent SAP kernel timed out");
+  fail(DDAMG_ERR_SINGULAR, what);
 }
+// the same in calls whose kernels do not factorise anything
+void finish(ddamg_handle* h) { check_err_flag(h, "singular block or linearly dependent vectors"); }
 
 // FP16 storage copies: allocated on first use, filled from the FP64 data after
 // every change of it, and read by the FP32 kernels while h->half is set.
@@ -1115,13 +1120,12 @@ bool persist_works(ddamg_handle* h, Level& L) {
                                mr, 1, L.sap_nbpc, L.sap_gcnt, h->st) == cudaSuccess;
   cudaGetLastError();
   sync(h);
-  int e = 0;
-  CK(cudaMemcpy(&e, h->d_err, sizeof(int), cudaMemcpyDeviceToHost));
-  if (e) {
-    CK(cudaMemset(h->d_err, 0, sizeof(int)));
-    ok = false;
-  }
-  if (!ok) return false;
+  auto flagged = [&] {
+    const bool e = *const_cast<volatile int*>(h->h_err) != 0;
+    if (e) *h->h_err = 0;
+    return e;
+  };
+  if (flagged() || !ok) return false;
   cudaStream_t s = nullptr;
   cudaGraph_t g = nullptr;
   cudaGraphExec_t ge = nullptr;
@@ -1139,12 +1143,7 @@ bool persist_works(ddamg_handle* h, Level& L) {
   if (g) cudaGraphDestroy(g);
   cudaStreamDestroy(s);
   cudaGetLastError();
-  CK(cudaMemcpy(&e, h->d_err, sizeof(int), cudaMemcpyDeviceToHost));
-  if (e) {
-    CK(cudaMemset(h->d_err, 0, sizeof(int)));
-    ok = false;
-  }
-  return ok;
+  return !flagged() && ok;
 }
 
 void tune_kernels(ddamg_handle* h) {
@@ -1851,7 +1850,7 @@ void hook(ddamg_handle* h, int l, const double* in, double* out, int n, bool out
   f(to, ti);
   exp(O, dout, to);
   if (!out_dev) CK(cudaMemcpyAsync(out, dout, out_bytes, cudaMemcpyDeviceToHost, h->st));
-  sync(h);
+  finish(h);
 }
 
 }  // namespace
@@ -2003,13 +2002,7 @@ void server_worker(ddamg_server* S, SrvHier* H) {
       for (int q = 0; q < na; ++q) tols[q] = H->slots[q].rq->tol;
       KrylovResult res;
       outer_fgmres(h, na, 1.0, 1, &res, true, tols.data());
-      int e = 0;
-      CK(cudaMemcpyAsync(&e, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, h->st));
-      sync(h);
-      if (e == 2) {
-        CK(cudaMemsetAsync(h->d_err, 0, sizeof(int), h->st));
-        fail(DDAMG_ERR_CUDA, "a shared-memory staging wait of the SAP kernel timed out");
-      }
+      finish(h);
       cplx<double>* dx = static_cast<cplx<double>*>(scratch(h, 1, fb));
       for (int q = 0; q < na; ++q) {
         SrvSlot& sl = H->slots[q];
@@ -2190,8 +2183,9 @@ int ddamg_setup(const double* gauge, const int dims[4], int bc_t, double m0, dou
     CK(cudaMallocHost(&h->h_scal, sizeof(double) * 64));
     build_hierarchy(h);
     allocate_hierarchy(h);
-    h->d_err = dalloc<int>(h, 1);
-    CK(cudaMemsetAsync(h->d_err, 0, sizeof(int), h->st));
+    CK(cudaHostAlloc(&h->h_err, sizeof(int), cudaHostAllocMapped));
+    *h->h_err = 0;
+    CK(cudaHostGetDevicePointer(&h->d_err, h->h_err, 0));
     h->lv[0].f64.err = h->lv[0].f32.err = h->d_err;
     for (auto& L : h->lv) L.c64.err = L.c32.err = h->d_err;
     double gg[6 * 16 * 2];
@@ -2222,7 +2216,7 @@ int ddamg_setup(const double* gauge, const int dims[4], int bc_t, double m0, dou
       tune_kernels(h);
       free_graphs(h);
     }
-    sync(h);
+    finish(h);
   });
   if (rc != DDAMG_OK) {
     ddamg_free(h);
@@ -2241,6 +2235,7 @@ void ddamg_free(ddamg_handle* h) {
   for (void* p : h->allocs) cudaFree(p);
   for (auto& s : h->scr)
     if (s.p) cudaFree(s.p);
+  if (h->h_err) cudaFreeHost(h->h_err);
   if (h->h_done) cudaFreeHost(h->h_done);
   if (h->h_kr) cudaFreeHost(h->h_kr);
   if (h->h_scal) cudaFreeHost(h->h_scal);
@@ -2268,7 +2263,16 @@ int ddamg_update_gauge(ddamg_handle* h, const double* gauge, int n_inv) {
       if (h->p.precision != 0) iterative_setup_phase<float>(h, 0, i);
       else iterative_setup_phase<double>(h, 0, i);
     }
+    finish(h);
+  });
+}
+
+// Not part of the ABI: leaves what a kernel's timed-out wait leaves, for the tests of how it is reported
+int ddamg_test_raise_flag(ddamg_handle* h, int flag) {
+  if (!h) return DDAMG_ERR_ARG;
+  return guard([&] {
     sync(h);
+    *h->h_err = flag;
   });
 }
 
@@ -2301,15 +2305,7 @@ int ddamg_solve(ddamg_handle* h, const double* rhs, double* x, int n, double tol
       cplx<double>* dx = xdev ? reinterpret_cast<cplx<double>*>(x + (size_t)s0 * F.vlen * 2)
                               : static_cast<cplx<double>*>(scratch(h, 1, fbytes * nb));
       fine_export<double>(dx, h->ox, F.g, nb, F.vlen, h->st);
-      {
-        int e = 0;
-        CK(cudaMemcpyAsync(&e, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, h->st));
-        sync(h);
-        if (e == 2) {
-          CK(cudaMemsetAsync(h->d_err, 0, sizeof(int), h->st));
-          fail(DDAMG_ERR_CUDA, "a shared-memory staging wait of the SAP kernel timed out");
-        }
-      }
+      finish(h);
       if (!xdev) CK(cudaMemcpyAsync(x + (size_t)s0 * F.vlen * 2, dx, fbytes * nb, cudaMemcpyDeviceToHost, h->st));
       sync(h);
       for (int r = 0; r < nb; ++r) {
