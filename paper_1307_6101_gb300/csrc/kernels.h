@@ -211,11 +211,11 @@ cudaError_t coarsest_cluster_solve(cplx<T>* x, const cplx<T>* b, const CoarseOp<
 // out(A)[s*N + j] = sum_{x in A, f in s} conj(P_j(x, f)) in(x, f)
 // (Ph, pscale): optional FP16 copy of P with per-(aggregate, chirality) scales (FP32 compute only)
 // tc_ks >= 1 (FP32 compute on FP16 P only): the tensor-core kernel with that k-split, P read once
-// per batch (transfer_tc.cu)
+// per batch (transfer_tc.cu).  Returns the status of the launch
 template <typename T>
-void restrict_op(cplx<T>* out, const cplx<T>* in, const cplx<T>* P, const Geom& gf, const Geom& gc, bool fine,
-                 int n, int N, int nrhs, size_t in_rstride, size_t out_rstride, size_t out_site_stride, int* err,
-                 cudaStream_t st, const __half2* Ph = nullptr, const float* pscale = nullptr, int tc_ks = 0);
+cudaError_t restrict_op(cplx<T>* out, const cplx<T>* in, const cplx<T>* P, const Geom& gf, const Geom& gc, bool fine,
+                        int n, int N, int nrhs, size_t in_rstride, size_t out_rstride, size_t out_site_stride, int* err,
+                        cudaStream_t st, const __half2* Ph = nullptr, const float* pscale = nullptr, int tc_ks = 0);
 // the same for C <= galerkin_cols() columns of a Galerkin term (TermSel sel, direction sel_mu): only the
 // sites that the term reaches are read
 int galerkin_cols();
@@ -241,7 +241,7 @@ cudaError_t prolong_batch(cplx<float>* out, const cplx<float>* in, const __half2
 void p_to_half(__half2* Ph, float* pscale, const cplx<double>* P, const Geom& g, bool fine, int n, int N,
                cudaStream_t st);
 // in-place CGS2 per aggregate and chirality of N fields (FP64); err set on rank deficiency
-void orthonormalise(cplx<double>* P, const Geom& g, bool fine, int n, int N, int* err, cudaStream_t st);
+cudaError_t orthonormalise(cplx<double>* P, const Geom& g, bool fine, int n, int N, int* err, cudaStream_t st);
 
 // ---- random fields (setup) -----------------------------------------------------
 // nfields complex N(0,1) fields j0 .. j0+nfields-1 of `level` in that level's layout

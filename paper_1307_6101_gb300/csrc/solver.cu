@@ -379,8 +379,8 @@ void restrict_lv(ddamg_handle* h, int l, cplx<T>* out, const cplx<T>* in, int nr
   const bool hf = half_on<T>(h);
   const double ps = hf ? 4.0 : cs;
   Prof pr(h, DDAMG_PROF_TRANSFER, (double)F.vlen * (cs * nrhs + ps * F.N) + (double)C.vlen * cs * nrhs);
-  restrict_op<T>(out, in, Pptr<T>(F), F.g, C.g, F.fine, F.n, F.N, nrhs, F.vlen, C.vlen, C.n, h->d_err, h->st,
-                 hf ? F.Ph : nullptr, hf ? F.pscale : nullptr, hf ? F.tr_ks : 0);
+  CK(restrict_op<T>(out, in, Pptr<T>(F), F.g, C.g, F.fine, F.n, F.N, nrhs, F.vlen, C.vlen, C.n, h->d_err, h->st,
+                    hf ? F.Ph : nullptr, hf ? F.pscale : nullptr, hf ? F.tr_ks : 0));
 }
 
 template <typename T>
@@ -1210,8 +1210,8 @@ void tune_kernels(ddamg_handle* h) {
       Work<float>& wc = work<float>(C);
       L.tr_ks = time_candidates(h, h->tune_ms[DDAMG_TUNE_RESTRICT][l], 5, [&](int k, bool) {
         if (k > 0 && !restrict_tc_fits(L.N, k)) return false;
-        restrict_op<float>(wc.bc, w.gin, L.P32, L.g, C.g, L.fine, L.n, L.N, B, L.vlen, C.vlen, C.n, h->d_err, h->st, L.Ph,
-                           L.pscale, k);
+        CK(restrict_op<float>(wc.bc, w.gin, L.P32, L.g, C.g, L.fine, L.n, L.N, B, L.vlen, C.vlen, C.n, h->d_err, h->st,
+                              L.Ph, L.pscale, k));
         return true;
       });
       blas_zero<float>(wc.bc, C.vlen, B, C.vlen, h->st);
@@ -1258,8 +1258,8 @@ void galerkin(ddamg_handle* h, int l, const cplx<T>* P, Term term) {
         if (!fits) {   // one or two FP64 test vectors, or an aggregate of tens of thousands of sites
           blas_zero<T>(tmp, F.vlen, jb, F.vlen, h->st);
           term(tmp, P + (size_t)j0 * F.vlen, jb, sel, mu, sp);
-          restrict_op<T>(cop<T>(C).blk + at, tmp, P, F.g, C.g, F.fine, F.n, F.N, jb, F.vlen, (size_t)nc,
-                         (size_t)9 * nc * nc, h->d_err, h->st);
+          CK(restrict_op<T>(cop<T>(C).blk + at, tmp, P, F.g, C.g, F.fine, F.n, F.N, jb, F.vlen, (size_t)nc,
+                            (size_t)9 * nc * nc, h->d_err, h->st));
           continue;
         }
         term(tmp, P + (size_t)j0 * F.vlen, jb, sel, mu, sp);
@@ -1279,7 +1279,7 @@ void rebuild(ddamg_handle* h, int l) {
   cudaStream_t st = h->st;
   const size_t tot = F.vlen * (size_t)F.N;
   blas_convert<double, double>(F.P64, F.tv64, tot, 1, 0, 0, st);
-  orthonormalise(F.P64, F.g, F.fine, F.n, F.N, h->d_err, st);
+  CK(orthonormalise(F.P64, F.g, F.fine, F.n, F.N, h->d_err, st));
   check_err_flag(h, "test vectors are linearly dependent on an aggregate");
   blas_convert<float, double>(F.P32, F.P64, tot, 1, 0, 0, st);
   // Galerkin: column (s', j) of every block = P^+ (term of D applied to P_j restricted to chirality s'),
@@ -1360,7 +1360,8 @@ void initial_setup_phase(ddamg_handle* h, int l, const double* const* tv_random)
   } else {
     Level& U = h->lv[l - 1];
     const int take = L.N < U.N ? L.N : U.N;
-    restrict_op<double>(L.tv64, U.tv64, U.P64, U.g, L.g, U.fine, U.n, U.N, take, U.vlen, L.vlen, L.n, h->d_err, h->st);
+    CK(restrict_op<double>(L.tv64, U.tv64, U.P64, U.g, L.g, U.fine, U.n, U.N, take, U.vlen, L.vlen, L.n, h->d_err,
+                           h->st));
     if (L.N > take) {
       if (!tv_random) {
         draw_fields(L.tv64 + (size_t)take * L.vlen, L.g, false, L.n, L.N - take, 0, l, h->p.seed, L.vlen, h->st);

@@ -615,15 +615,15 @@ void p_to_half(__half2* Ph, float* pscale, const cplx<double>* P, const Geom& g,
 }
 
 template <typename T>
-void restrict_op(cplx<T>* out, const cplx<T>* in, const cplx<T>* P, const Geom& gf, const Geom& gc, bool fine, int n,
-                 int N, int nrhs, size_t in_rstride, size_t out_rstride, size_t out_site_stride, int* err,
-                 cudaStream_t st, const __half2* Ph, const float* pscale, int tc_ks) {
+cudaError_t restrict_op(cplx<T>* out, const cplx<T>* in, const cplx<T>* P, const Geom& gf, const Geom& gc, bool fine,
+                        int n, int N, int nrhs, size_t in_rstride, size_t out_rstride, size_t out_site_stride, int* err,
+                        cudaStream_t st, const __half2* Ph, const float* pscale, int tc_ks) {
   if constexpr (sizeof(T) == 4) {
     // FP16 P: the tensor-core kernel (P read once per batch) where the autotuner chose it
     if (Ph && tc_ks > 0) {
       if (restrict_tc(out, in, Ph, pscale, gf, fine, n, N, nrhs, in_rstride, out_rstride, out_site_stride, tc_ks,
                       st) == cudaSuccess)
-        return;
+        return cudaSuccess;
       cudaGetLastError();
     }
   }
@@ -652,14 +652,12 @@ void restrict_op(cplx<T>* out, const cplx<T>* in, const cplx<T>* P, const Geom& 
     kernel<<<grid, groups * RTH, restrict_smem<T>(N, groups, pb).total, st>>>(
         out, in, Ps, scale, gf, fine, n, N, nrhs, in_rstride, pstride, out_rstride, out_site_stride, kch,
         run < kch ? run : kch, err);
+    return cudaPeekAtLastError();
   };
   if constexpr (sizeof(T) == 4) {
-    if (Ph) {
-      launch(Ph, pscale);
-      return;
-    }
+    if (Ph) return launch(Ph, pscale);
   }
-  launch(P, (const float*)nullptr);
+  return launch(P, (const float*)nullptr);
 }
 
 template <typename T>
@@ -689,7 +687,7 @@ void prolong_op(cplx<T>* out, const cplx<T>* in, const cplx<T>* P, const Geom& g
                                                                        out_rstride, in_rstride, pstride, accumulate);
 }
 
-void orthonormalise(cplx<double>* P, const Geom& g, bool fine, int n, int N, int* err, cudaStream_t st) {
+cudaError_t orthonormalise(cplx<double>* P, const Geom& g, bool fine, int n, int N, int* err, cudaStream_t st) {
   const size_t pstride = (size_t)g.V * n;
   const size_t sm = (size_t)g.vA * (n / 2) * sizeof(cplx<double>);   // the column in work
   static DeviceOnce once;
@@ -699,6 +697,7 @@ void orthonormalise(cplx<double>* P, const Geom& g, bool fine, int n, int N, int
     k_orthonormalise<true><<<dim3(g.nAgg, 2), OT, sm, st>>>(P, g, fine, n, N, pstride, err);
   else
     k_orthonormalise<false><<<dim3(g.nAgg, 2), OT, 0, st>>>(P, g, fine, n, N, pstride, err);
+  return cudaPeekAtLastError();
 }
 
 int galerkin_cols() { return GCMAX; }
@@ -727,8 +726,9 @@ cudaError_t galerkin_restrict(cplx<double>* out, const cplx<T>* tmp, const cplx<
 }
 
 #define INST(T)                                                                                                  \
-  template void restrict_op<T>(cplx<T>*, const cplx<T>*, const cplx<T>*, const Geom&, const Geom&, bool, int, int, \
-                               int, size_t, size_t, size_t, int*, cudaStream_t, const __half2*, const float*, int); \
+  template cudaError_t restrict_op<T>(cplx<T>*, const cplx<T>*, const cplx<T>*, const Geom&, const Geom&, bool, int, \
+                                      int, int, size_t, size_t, size_t, int*, cudaStream_t, const __half2*,       \
+                                      const float*, int);                                                        \
   template void prolong_op<T>(cplx<T>*, const cplx<T>*, const cplx<T>*, const Geom&, const Geom&, bool, int, int,  \
                               int, size_t, size_t, bool, cudaStream_t, const __half2*, const float*, int);   \
   template bool galerkin_fits<T>(int, int, int);                                                                 \

@@ -109,3 +109,15 @@ def test_attributes_are_set_once_per_device(tmp_path):
   DeviceOnce limit;
   CHECK(raise_smem_limit(limit, nullptr) != cudaSuccess);
 """)
+
+
+def test_setup_kernels_report_a_refused_launch(tmp_path):
+    """Restriction and orthonormalisation return the status of their launch (refused here: there is no device)."""
+    run(tmp_path, r"""
+  Geom g = geom(2, 2, 2, 2);
+  g.vA = 16;
+  g.nAgg = g.V / 16;
+  CHECK(restrict_op<double>(nullptr, nullptr, nullptr, g, g, true, 12, 4, 1, 0, 0, 0, nullptr, nullptr) != cudaSuccess);
+  CHECK(restrict_op<float>(nullptr, nullptr, nullptr, g, g, true, 12, 4, 1, 0, 0, 0, nullptr, nullptr) != cudaSuccess);
+  CHECK(orthonormalise(nullptr, g, true, 12, 4, nullptr, nullptr) != cudaSuccess);
+""")
