@@ -327,9 +327,9 @@ struct SapSmem {
   size_t rfull, pbuf, part, red, sh, slot, bar, total;
 };
 DD_HD size_t al16(size_t x) { return (x + 15) & ~size_t(15); }
-DD_HD SapSmem sap_smem_layout(int vB, int n, int spc, int nsl, size_t bs, size_t ts) {
+DD_HD SapSmem sap_smem_layout(int vB, int n, int spc, int nsl, size_t ts) {
   SapSmem L;
-  size_t o = al16((size_t)spc * nsl * n * n * bs);
+  size_t o = al16((size_t)spc * nsl * n * n * 2 * ts);
   L.rfull = o;
   o = al16(o + (size_t)vB * n * 2 * ts);
   L.pbuf = o;
@@ -360,9 +360,9 @@ DD_HD SapSmem sap_smem_layout(int vB, int n, int spc, int nsl, size_t bs, size_t
 // dot products are summed in rank order, so every CTA computes the same alpha
 // and applies r <- r - alpha p to its whole copy.  Same arithmetic as
 // k_coarse_sap: rho = (b - D z)_B, k MR steps on D_B, z_B += e_B.
-template <typename T, typename BS>
+template <typename T>
 __global__ void __launch_bounds__(768, 2) k_coarse_sap_cluster(cplx<T>* __restrict__ z, const cplx<T>* __restrict__ bsrc,
-                                     const BS* __restrict__ blk, const float* __restrict__ bscale, Geom g, int n,
+                                     const cplx<T>* __restrict__ blk, Geom g, int n,
                                      size_t rstride, int nrhs, const int* __restrict__ blocks, int k_mr, int spc,
                                      int nsl, int* err, const int* __restrict__ bsite,
                                      const int* __restrict__ bloc) {
@@ -377,8 +377,8 @@ __global__ void __launch_bounds__(768, 2) k_coarse_sap_cluster(cplx<T>* __restri
   const int b = blocks[blockIdx.x / CLS];
   const int rows = spc * n;
   const size_t nn = (size_t)n * n;
-  const SapSmem L = sap_smem_layout(vB, n, spc, nsl, sizeof(BS), sizeof(T));
-  BS* stage = reinterpret_cast<BS*>(smem_raw);                                // [spc][nsl][n][n]
+  const SapSmem L = sap_smem_layout(vB, n, spc, nsl, sizeof(T));
+  cplx<T>* stage = reinterpret_cast<cplx<T>*>(smem_raw);                      // [spc][nsl][n][n]
   cplx<T>* rfull = reinterpret_cast<cplx<T>*>(smem_raw + L.rfull);            // [vB*n]
   cplx<T>* pbuf = reinterpret_cast<cplx<T>*>(smem_raw + L.pbuf);              // [2][vB*n]
   cplx<T>* part = reinterpret_cast<cplx<T>*>(smem_raw + L.part);              // [9][rows]
@@ -404,20 +404,19 @@ __global__ void __launch_bounds__(768, 2) k_coarse_sap_cluster(cplx<T>* __restri
   if (threadIdx.x < 32) {
     int cnt = 0;
     for (int e = 0; e < spc * 9; ++e) cnt += slot[e] >= 0 ? 1 : 0;
-    if (threadIdx.x == 0) mbar_arrive_expect_tx(bar, (unsigned)(cnt * nn * sizeof(BS)));
+    if (threadIdx.x == 0) mbar_arrive_expect_tx(bar, (unsigned)(cnt * nn * sizeof(cplx<T>)));
     __syncwarp();
     for (int e = threadIdx.x; e < spc * 9; e += 32) {
       const int sl = e / 9, k = e % 9, q = slot[e];
       if (q >= 0)
         bulk_g2s(stage + ((size_t)sl * nsl + q) * nn, blk + ((size_t)own[sl] * 9 + k) * nn,
-                 (unsigned)(nn * sizeof(BS)), bar);
+                 (unsigned)(nn * sizeof(cplx<T>)), bar);
     }
   }
   const int k = threadIdx.x / rows;
   const int rl = threadIdx.x - k * rows;
   const int sl = rl / n, i = rl - (rl / n) * n;
   const int site = own[sl];
-  const T sc = bscale ? T(bscale[site]) : T(1);
   int q = -1, nb = site, nloc = 0;
   if (k < 9) {
     q = slot[sl * 9 + k];
@@ -428,7 +427,7 @@ __global__ void __launch_bounds__(768, 2) k_coarse_sap_cluster(cplx<T>* __restri
     }
     nloc = q >= 0 ? bloc[nb] : 0;
   }
-  const BS* Ms = stage + ((size_t)sl * nsl + (q >= 0 ? q : 0)) * nn + i;   // staged row i (column-major)
+  const cplx<T>* Ms = stage + ((size_t)sl * nsl + (q >= 0 ? q : 0)) * nn + i;   // staged row i (column-major)
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
   int ok = 1;
   pdl_wait();   // the previous kernel's z and b are complete from here on
@@ -438,10 +437,10 @@ __global__ void __launch_bounds__(768, 2) k_coarse_sap_cluster(cplx<T>* __restri
     // rho = b - D z on the own rows: hops leaving the block from global memory ...
     cplx<T> acc = czero<T>();
     if (k < 9 && q < 0) {
-      const BS* M = blk + ((size_t)site * 9 + k) * nn + i;
+      const cplx<T>* M = blk + ((size_t)site * 9 + k) * nn + i;
       const cplx<T>* v = z + ro + (size_t)nb * n;
 #pragma unroll 8
-      for (int j = 0; j < n; ++j) cfma(acc, ld_cplx(M, (size_t)j * n), v[j]);
+      for (int j = 0; j < n; ++j) cfma(acc, M[(size_t)j * n], v[j]);
     }
     if (rh == 0) {
       ok = __syncthreads_and(mbar_wait_bounded(bar, 0) ? 1 : 0);
@@ -451,9 +450,9 @@ __global__ void __launch_bounds__(768, 2) k_coarse_sap_cluster(cplx<T>* __restri
     if (k < 9 && q >= 0) {
       const cplx<T>* v = z + ro + (size_t)nb * n;
 #pragma unroll 8
-      for (int j = 0; j < n; ++j) cfma(acc, ld_cplx(Ms, (size_t)j * n), v[j]);
+      for (int j = 0; j < n; ++j) cfma(acc, Ms[(size_t)j * n], v[j]);
     }
-    if (k < 9) part[k * rows + rl] = sc * acc;
+    if (k < 9) part[k * rows + rl] = acc;
     __syncthreads();
     cplx<T> r = czero<T>(), xs = czero<T>();
     if (threadIdx.x < rows) {
@@ -474,9 +473,9 @@ __global__ void __launch_bounds__(768, 2) k_coarse_sap_cluster(cplx<T>* __restri
         if (q >= 0) {
           const cplx<T>* v = rfull + (size_t)nloc * n;
 #pragma unroll 8
-          for (int j = 0; j < n; ++j) cfma(a, ld_cplx(Ms, (size_t)j * n), v[j]);
+          for (int j = 0; j < n; ++j) cfma(a, Ms[(size_t)j * n], v[j]);
         }
-        part[k * rows + rl] = sc * a;
+        part[k * rows + rl] = a;
       }
       __syncthreads();
       cplx<T> p = czero<T>();
@@ -1313,14 +1312,14 @@ int coarse_sap_slots(const Geom& g) {
 // The dynamic shared-memory limit of a kernel is a process-wide attribute: it is raised to the
 // device maximum (not to this plan's size), so that a hierarchy set up later with smaller blocks
 // cannot lower it below what an earlier hierarchy's launches use.
-template <typename T, typename BS>
+template <typename T>
 void sap_cluster_attrs(size_t smem, int CLS) {
-  if (cudaFuncSetAttribute(k_coarse_sap_cluster<T, BS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) !=
+  if (cudaFuncSetAttribute(k_coarse_sap_cluster<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) !=
       cudaSuccess) {
     cudaGetLastError();
-    cudaFuncSetAttribute(k_coarse_sap_cluster<T, BS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_coarse_sap_cluster<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   }
-  if (CLS > 8) cudaFuncSetAttribute(k_coarse_sap_cluster<T, BS>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (CLS > 8) cudaFuncSetAttribute(k_coarse_sap_cluster<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
 }
 
 // cluster plan of the coarse SAP on blocks in the compute precision: cluster size CLS, sites per CTA
@@ -1334,9 +1333,9 @@ int coarse_sap_cluster_plan(const Geom& g, int n, int* CLS_out, int* spc_out, in
     const int spc = g.vB / CLS;
     const int threads = ((9 * spc * n + 31) / 32) * 32;
     if (threads > 768) continue;   // launch bounds of k_coarse_sap_cluster
-    const size_t sm = sap_smem_layout(g.vB, n, spc, nsl, sizeof(cplx<T>), sizeof(T)).total;
+    const size_t sm = sap_smem_layout(g.vB, n, spc, nsl, sizeof(T)).total;
     if (sm > 227 * 1024) continue;
-    sap_cluster_attrs<T, cplx<T>>(sm, CLS);
+    sap_cluster_attrs<T>(sm, CLS);
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1349,7 +1348,7 @@ int coarse_sap_cluster_plan(const Geom& g, int n, int* CLS_out, int* spc_out, in
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int nclusters = 0;
-    if (cudaOccupancyMaxActiveClusters(&nclusters, k_coarse_sap_cluster<T, cplx<T>>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&nclusters, k_coarse_sap_cluster<T>, &cfg) != cudaSuccess) {
       cudaGetLastError();
       continue;
     }
@@ -1548,9 +1547,9 @@ cudaError_t coarse_sap_sweep(cplx<T>* z, const cplx<T>* b, const CoarseOp<T>& op
         }
       }
       cfg.blockDim = dim3(((9 * spc * op.n + 31) / 32) * 32, 1, 1);
-      cfg.dynamicSmemBytes = sap_smem_layout(op.g.vB, op.n, spc, op.sap_nsl, sizeof(cplx<T>), sizeof(T)).total;
-      e = cudaLaunchKernelEx(&cfg, k_coarse_sap_cluster<T, cplx<T>>, z, b, (const cplx<T>*)op.blk, (const float*)nullptr,
-                             op.g, op.n, rstride, nrhs, blocks, k_mr, spc, op.sap_nsl, op.err, op.bsite, op.bloc);
+      cfg.dynamicSmemBytes = sap_smem_layout(op.g.vB, op.n, spc, op.sap_nsl, sizeof(T)).total;
+      e = cudaLaunchKernelEx(&cfg, k_coarse_sap_cluster<T>, z, b, (const cplx<T>*)op.blk, op.g, op.n, rstride, nrhs,
+                             blocks, k_mr, spc, op.sap_nsl, op.err, op.bsite, op.bloc);
       if (e == cudaSuccess) return cudaSuccess;
       cudaGetLastError();
     }
