@@ -21,6 +21,7 @@
 
 #include <cstdint>
 #include <mutex>
+#include <stdexcept>
 
 namespace {
 
@@ -1642,6 +1643,7 @@ void fine_dslash(cplx<T>* out, const cplx<T>* in, const cplx<T>* b, const FineOp
       fine_dslash_split(out, in, b, op, nrhs, rstride, st);
       return;
     }
+    if (b) throw std::invalid_argument("fine_dslash: no FP64 residual of a single term");
   }
   dim3 grid(div_up(op.g.V, 128), nrhs);
   count_launch();

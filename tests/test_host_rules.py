@@ -13,6 +13,7 @@ PKG = os.path.join(ROOT, "paper_1307_6101_gb300")
 PRELUDE = r"""
 #include <cstdio>
 #include <cstdlib>
+#include <exception>
 #include "kernels.h"
 using namespace dd;
 #define CHECK(c) do { if (!(c)) { printf("line %d: %s\n", __LINE__, #c); return 1; } } while (0)
@@ -120,4 +121,22 @@ def test_setup_kernels_report_a_refused_launch(tmp_path):
   CHECK(restrict_op<double>(nullptr, nullptr, nullptr, g, g, true, 12, 4, 1, 0, 0, 0, nullptr, nullptr) != cudaSuccess);
   CHECK(restrict_op<float>(nullptr, nullptr, nullptr, g, g, true, 12, 4, 1, 0, 0, 0, nullptr, nullptr) != cudaSuccess);
   CHECK(orthonormalise(nullptr, g, true, 12, 4, nullptr, nullptr) != cudaSuccess);
+""")
+
+
+def test_residual_of_a_term_is_refused(tmp_path):
+    """b - (term of D) in FP64 has no kernel: it is refused, not computed without b."""
+    run(tmp_path, r"""
+  FineOp<double> op{};
+  op.g = geom(2, 2, 2, 2);
+  const cplx<double>* b = reinterpret_cast<const cplx<double>*>(&op);
+  for (int sel : {SEL_AGG_SELF, SEL_AGG_FWD, SEL_AGG_BWD, SEL_FULL}) {
+    bool refused = false;
+    try {
+      fine_dslash<double>(nullptr, nullptr, b, op, 1, 0, sel, 0, 0, nullptr);
+    } catch (const std::exception&) {
+      refused = true;
+    }
+    CHECK(refused);
+  }
 """)
