@@ -1805,10 +1805,8 @@ cudaError_t fine_sap_sweep(cplx<T>* z, const cplx<T>* b, const FineOp<T>& op, co
                            size_t rstride, int k_mr, cudaStream_t st) {
   if (nrhs < 1 || nblocks < 1) return cudaSuccess;   // the staged kernels issue their copies before the rhs loop
   if constexpr (sizeof(T) == 8) {
-    // Six threads per site, except where blocks of more than 64 sites (a cluster per block) are enough of
-    // them to fill the chip with one thread per site: 4^4 blocks, 128 per colour: 670 us per sweep with
-    // six threads and 540 with one, 16 per colour: 195 and 530.
-    if (op.g.vB <= 64 || nblocks < 96) return fine_sap_split(z, b, op, blocks, nblocks, nrhs, rstride, k_mr, st);
+    if (fine_sap_takes_split(op.g, nblocks, op.batch))
+      return fine_sap_split(z, b, op, blocks, nblocks, nrhs, rstride, k_mr, st);
     launch_sap_plain<T, cplx<T>, T>(z, b, op.U, op.clov, op, blocks, nblocks, nrhs, rstride, k_mr, T(0), st);
   } else {
     const bool tma = sap_tma_ok(op) && op.err;

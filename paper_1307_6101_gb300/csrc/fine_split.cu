@@ -162,6 +162,7 @@ __global__ void __launch_bounds__(6 * DS) k_fine_dslash_split(cplx<double>* __re
 // (three warps per SM at 2^4 blocks): 4 MR steps on 8^4 with 2^4 blocks 58 us per sweep (k_fine_sap, 8 CTAs:
 // 516), 16^3x32 800 (1050).
 constexpr int MAXCLS = 8;
+constexpr int SMS = 152;   // of a GB300
 
 template <int NT>   // most threads of a CTA
 __global__ void __launch_bounds__(NT, 768 / NT) k_fine_sap_split(cplx<double>* __restrict__ z,
@@ -323,6 +324,16 @@ __global__ void __launch_bounds__(NT, 768 / NT) k_fine_sap_split(cplx<double>* _
   }
 }
 
+// CTAs per block: at most 64 sites (384 threads, 64 KB of shared memory: two or three CTAs per SM) where a
+// cluster of eight reaches that, and more CTAs as long as there are fewer than SMs and a CTA keeps 16
+// sites.  The rule looks at the level only, not at the batch: the partial sums of a block must not
+// depend on it.
+int split_ctas(int vB, int nblocks) {
+  int CLS = 1;
+  while (CLS < MAXCLS && (vB > 64 * CLS || (nblocks * CLS < SMS && vB >= 32 * CLS))) CLS *= 2;
+  return CLS;
+}
+
 }  // namespace
 
 namespace dd {
@@ -337,16 +348,35 @@ void fine_dslash_split(cplx<double>* out, const cplx<double>* in, const cplx<dou
     k_fine_dslash_split<false><<<grid, 6 * DS, 0, st>>>(out, in, b, op.U, op.clov, op.g, op.bc_t, rstride);
 }
 
+// Six threads per site against one (k_fine_sap, CTAs of 256 threads).  With one, a wave of 152 CTAs takes 34 us and 47 for
+// each warp of a CTA that has sites, however few CTAs run.  Six take, for the sites of the SM with the most CTAs, 0.81 us
+// per site and 0.15 for each hop pass of an MR step (3 MR steps).  So six threads lose where the blocks of a
+// colour, for all right-hand sides, fill the waves of the other kernel.  us per sweep, six / one: 4^4 blocks, 32: 139 / 405,
+// 96: 378 / 403, 128: 490 / 404, 192: 690 / 800, 256: 916 / 800, 768: 2518 / 2380; 4^3 x 2, 256: 442 / 400, 384: 622 / 790;
+// 4^2 x 2^2, 512 in one field: 459 / 413, 128 in four: 377 / 405; 3^3 x 2, 2304: 1727 / 1638; 3^4, 128: 168 / 318,
+// 512: 561 / 630; 2^4, 2048: 325 / 410.
+// Above 256 sites one thread per site takes more registers than a CTA has.  The two sum in different orders and a column has
+// the same bits alone and in a batch, so the rule counts the batch that the handle was set up for, not the one at
+// hand: a handle for one right-hand side that smooths eight fields of 16 4^4 blocks takes 62 us per field and not 51.
+bool fine_sap_takes_split(const Geom& g, int nblocks, int batch) {
+  const int vB = g.vB, CLS = split_ctas(vB, nblocks), S = (vB + CLS - 1) / CLS;
+  if (vB > 256) return true;
+  int passes = 0, seg = 1;
+  for (int d = 0; d < 4; ++d) passes += g.B[d] == g.L[d] || g.B[d] > 2 ? 2 : g.B[d] - 1;
+  while (seg < vB) seg <<= 1;
+  const int per_cta = 256 / seg, warps = seg >= 32 ? per_cta * ((vB + 31) / 32) : 8;
+  const long long blocks = (long long)nblocks * batch;
+  auto waves = [](long long ctas) { return (double)((ctas + SMS - 1) / SMS); };
+  const double one = waves((blocks + per_cta - 1) / per_cta) * (34.0 + 47.0 * warps);
+  const double sites = (6 * S + 31) / 32 * 32 / 6.0;   // of a CTA, with the threads that have none
+  return waves(blocks * CLS) * sites * (0.81 + 0.15 * passes) < one;
+}
+
 cudaError_t fine_sap_split(cplx<double>* z, const cplx<double>* b, const FineOp<double>& op, const int* blocks,
                            int nblocks, int nrhs, size_t rstride, int k_mr, cudaStream_t st) {
   if (k_mr < 1) return cudaSuccess;   // e = 0
   const int vB = op.g.vB;
-  // CTAs per block: at most 64 sites (384 threads, 64 KB of shared memory: three CTAs per SM) where a
-  // cluster of eight reaches that, and more CTAs as long as there are fewer than SMs and a CTA keeps 16
-  // sites.  The rule looks at the level only, not at the batch: the partial sums of a block must not
-  // depend on it.
-  int CLS = 1;
-  while (CLS < MAXCLS && (vB > 64 * CLS || (nblocks * CLS < 152 && vB >= 32 * CLS))) CLS *= 2;
+  const int CLS = split_ctas(vB, nblocks);
   const int S = (vB + CLS - 1) / CLS;
   const int threads = ((6 * S + 31) / 32) * 32;
   const size_t sm = (size_t)66 * S * sizeof(cplx<double>) + (72 + 6 * MAXCLS) * sizeof(double) + (size_t)8 * S * sizeof(short);

@@ -49,6 +49,7 @@ struct FineOp {
   cplx<T>* U;    // [4][9][V]
   T* clov;       // [2][36][V]  (m0 + 4) + clover, packed Hermitian
   int* err;      // device error flag (bounded waits), may be null
+  int batch = 1; // right-hand sides that the handle was set up for
   // FP16 storage (FP32 compute only): when Uh is set the kernels read these instead
   const __half2* Uh = nullptr;   // [4][9][V] links
   const __half2* clovh = nullptr; // [2][18][V] clover term without the (m0 + 4) shift, pairs of packed reals
@@ -92,6 +93,8 @@ void fine_dslash(cplx<T>* out, const cplx<T>* in, const cplx<T>* b, const FineOp
 template <typename T>
 cudaError_t fine_sap_sweep(cplx<T>* z, const cplx<T>* b, const FineOp<T>& op, const int* blocks, int nblocks, int nrhs,
                            size_t rstride, int k_mr, cudaStream_t st);
+// whether FP64 SAP runs with six threads per site (nblocks per colour, handles set up for batch right-hand sides)
+bool fine_sap_takes_split(const Geom& g, int nblocks, int batch);
 // FP64 with six threads per site (fine_split.cu): the full operator (b set: b - D in), and one SAP
 // colour sweep (cudaErrorInvalidConfiguration, nothing launched, above 1024 sites in a block)
 void fine_dslash_split(cplx<double>* out, const cplx<double>* in, const cplx<double>* b, const FineOp<double>& op,

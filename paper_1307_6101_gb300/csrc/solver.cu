@@ -2188,6 +2188,7 @@ int ddamg_setup(const double* gauge, const int dims[4], int bc_t, double m0, dou
     *h->h_err = 0;
     CK(cudaHostGetDevicePointer(&h->d_err, h->h_err, 0));
     h->lv[0].f64.err = h->lv[0].f32.err = h->d_err;
+    h->lv[0].f64.batch = h->max_batch;
     for (auto& L : h->lv) L.c64.err = L.c32.err = h->d_err;
     double gg[6 * 16 * 2];
     gamma_products(gg);

@@ -42,3 +42,21 @@ def test_split_operator_and_sap_against_oracle(dims, block):
     for r in range(2):
         assert rel(out[r], o.levels[0].op.apply(f[r])) <= 1e-12
         assert rel(z1[r], o.levels[0].sap.smooth(f[r], z[r], 1)) <= 1e-12
+
+
+@pytest.mark.parametrize("max_rhs", [1, 8, 12])
+def test_sap_kernel_of_the_handles_batch(max_rhs):
+    """16 blocks of 4^4 sites per colour: six threads per site for batches of one and twelve, one thread per site for eight;
+    a column has the same bits alone and in a batch of any size."""
+    import paper_1307_6101_gb300 as dd
+    dims, block = (16, 8, 8, 8), (4, 4, 4, 4)
+    c = Case(dims=dims, levels=2, agg=(block,), n_tv=(1,), sap=(block,), max_rhs=max_rhs)
+    h, o = c.gpu(0), c.oracle()
+    f = np.ascontiguousarray(synth.random_spinors(9, dims, 5))
+    z = np.ascontiguousarray(synth.random_spinors(9, dims, 6))
+    z1, one = z.copy(), z[8:].copy()
+    dd.ddamg_smooth(h, 0, 0, f, z1, 9, 1)
+    dd.ddamg_smooth(h, 0, 0, f[8:].copy(), one, 1, 1)
+    assert np.array_equal(one[0], z1[8])
+    for r in (0, 8):
+        assert rel(z1[r], o.levels[0].sap.smooth(f[r], z[r], 1)) <= 1e-12

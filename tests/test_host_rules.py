@@ -140,3 +140,22 @@ def test_residual_of_a_term_is_refused(tmp_path):
     CHECK(refused);
   }
 """)
+
+
+def test_fp64_sap_kernel_per_batch(tmp_path):
+    """The FP64 SAP kernel by block, blocks per colour and batch: the faster of the two in each measured case."""
+    run(tmp_path, r"""
+  const Geom b4 = geom(4, 4, 4, 4), b442 = geom(4, 4, 2, 2), b43 = geom(4, 4, 4, 2), b3 = geom(3, 3, 3, 3);
+  for (int blocks : {8, 16, 32, 64, 96}) CHECK(fine_sap_takes_split(b4, blocks, 1));
+  CHECK(fine_sap_takes_split(b4, 8, 12) && fine_sap_takes_split(b4, 16, 12) && fine_sap_takes_split(b4, 16, 4));
+  CHECK(!fine_sap_takes_split(b4, 16, 8) && !fine_sap_takes_split(b4, 32, 4) && !fine_sap_takes_split(b4, 64, 2));
+  CHECK(!fine_sap_takes_split(b4, 64, 12) && !fine_sap_takes_split(b4, 128, 1) && !fine_sap_takes_split(b4, 512, 12));
+  CHECK(fine_sap_takes_split(b43, 64, 2) && fine_sap_takes_split(b43, 32, 12) && !fine_sap_takes_split(b43, 32, 8));
+  CHECK(fine_sap_takes_split(b442, 128, 4) && fine_sap_takes_split(b442, 512, 2) && !fine_sap_takes_split(b442, 512, 1));
+  CHECK(fine_sap_takes_split(b3, 32, 8) && fine_sap_takes_split(b3, 128, 1) && !fine_sap_takes_split(b3, 128, 2));
+  CHECK(fine_sap_takes_split(b3, 128, 4) && fine_sap_takes_split(b3, 128, 12) && !fine_sap_takes_split(b442, 512, 8));
+  CHECK(fine_sap_takes_split(geom(4, 4, 4, 3), 192, 1) && !fine_sap_takes_split(geom(4, 4, 4, 3), 192, 8));
+  CHECK(!fine_sap_takes_split(geom(3, 3, 3, 2), 192, 12) && fine_sap_takes_split(geom(3, 3, 3, 2), 192, 4));
+  for (int batch : {1, 2, 8, 12}) CHECK(fine_sap_takes_split(geom(2, 2, 2, 2), 2048, batch));
+  CHECK(fine_sap_takes_split(geom(8, 8, 4, 4), 512, 12));
+""")
