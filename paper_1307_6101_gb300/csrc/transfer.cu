@@ -27,7 +27,7 @@ DD_HD size_t faddr(bool fine, int V, int n, int x, int f) {
 // warps split K, in a way that depends on the level only, so that a right-hand side has the same bits alone
 // and in a batch.  A lane's products of a few chunks run in one chain and are then added to its part, so that neither
 // chain is long, and the parts are added with their rounding errors.  An FP16 column on 4^4 aggregates is off by
-// 0.9e-7 (8 test vectors) to 1.1e-7 (32) against 64 bits, 20 test vectors 1.0e-7; three chunks in one chain and plain sums of
+// 0.87e-7 (8 test vectors) to 1.09e-7 (32) against 64 bits, 20 test vectors 1.07e-7; three chunks in one chain and plain sums of
 // the parts gave 1.33e-7 there, one lane per site and a butterfly over the lanes 1.11e-7 (6^4 aggregates 1.79e-7).
 // A chunk is whole runs of memory (sites of one component on the fine level, dofs of one site on a coarse one).
 // Where those are multiples of 16 bytes (BULK) one lane copies a run of a column with one bulk copy;
@@ -65,6 +65,21 @@ inline int restrict_chunk(int run, int ps, bool bulk) {
   return 0;
 }
 
+// Chunks that run into one chain of a lane's FMAs: a chain of k roundings errs like sqrt(k / 2) of them, so what
+// counts is the FMAs of a chain plus the chains of a lane.  One chunk more than makes that least, since every end of a chain
+// costs time (16^3x32, 20 test vectors, restriction and interpolation of one column 146 us with one chunk and 142 with
+// two, of twelve 524 and 514), as long as it stays below a lane per site (up to 256 lanes), a butterfly over them and the
+// warps in a chain.
+inline int restrict_flush(int vA, int h, int N, int kch) {
+  const int nsub = 32 / ((N + 3) / 4), nch = (vA * h + kch - 1) / kch;
+  auto roundings = [&](int f) { return f * kch / (2.0 * nsub) + (double)nch / f; };
+  int lanes = 1, levels = 0, f = 1;
+  for (; lanes < vA && lanes < 256; lanes *= 2) levels += lanes < 32;
+  const double limit = 2.0 * h * ((vA + lanes - 1) / lanes) + 2 * levels + lanes / 32 - 2;
+  while (roundings(f + 1) < roundings(f)) ++f;
+  return f < nch && roundings(f + 1) <= limit ? f + 1 : f;
+}
+
 // (hi, lo) += x without rounding error beyond lo's (Knuth's two-sum)
 __device__ __forceinline__ void two_sum_acc(float& hi, float& lo, float x) {
   const float s = __fadd_rn(hi, x), t = __fsub_rn(s, hi);
@@ -92,12 +107,12 @@ __device__ __forceinline__ void ld_pair(const cplx<double>* p, cplx<double> a[2]
   a[1] = p[1];
 }
 
-// kch: K rows of a chunk, run: elements of a run inside a chunk (BULK)
+// kch: K rows of a chunk, run: elements of a run inside a chunk (BULK), flush: chunks that run into one chain of FMAs
 template <typename T, typename PS, bool BULK>
 __global__ void __launch_bounds__(RNG * RTH, sizeof(T) == 4 ? 2 : 1) k_restrict(
     cplx<T>* __restrict__ out, const cplx<T>* __restrict__ in, const PS* __restrict__ P,
     const float* __restrict__ pscale, Geom gf, bool fine, int n, int N, int nrhs, size_t in_rstride, size_t pstride,
-    size_t out_rstride, size_t out_site_stride, int kch, int run, int* err) {
+    size_t out_rstride, size_t out_site_stride, int kch, int run, int flush, int* err) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int RCT = restrict_ct<T>();
   const int groups = blockDim.x / RTH;
@@ -155,18 +170,14 @@ __global__ void __launch_bounds__(RNG * RTH, sizeof(T) == 4 ? 2 : 1) k_restrict(
     mbar_init(&bar[1], 1);
   }
   if (BULK) __syncthreads();
-  // chunks per chain: chains of `per` FMAs a chunk and nch / flush sums of them err least near flush^2 = nch / per
-  const int nch = (K + kch - 1) / kch, per = 4 * ((kch / 2 + (RTH / 32) * nsub - 1) / ((RTH / 32) * nsub));
-  int flush = 1;
-  while (flush * (flush + 1) * per < nch) ++flush;
   cplx<T> acc[4][RCT];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
     for (int c = 0; c < RCT; ++c) acc[i][c] = czero<T>();
   copy(0, 0);
-  int chunk = 0;
-  bool ok = true;
+  int chunk = 0, next = flush - 1;   // the chunk that ends the chain
+  bool ok = true, first = true;
   for (int k0 = 0; k0 < K; k0 += kch, ++chunk) {
     const int buf = chunk & 1;
     const bool last = k0 + kch >= K;
@@ -198,7 +209,7 @@ __global__ void __launch_bounds__(RNG * RTH, sizeof(T) == 4 ? 2 : 1) k_restrict(
             }
           }
       }
-      if (chunk % flush == flush - 1 || last) {
+      if (chunk == next || last) {
         cplx<T>* mine = red + (size_t)grp * 4 * RCT * slots + (warp * nsub + sub) * TI + ti;
 #pragma unroll
         for (int i = 0; i < 4; ++i)
@@ -206,9 +217,11 @@ __global__ void __launch_bounds__(RNG * RTH, sizeof(T) == 4 ? 2 : 1) k_restrict(
           for (int c = 0; c < RCT; ++c)
             if (c < gc) {
               cplx<T>& m = mine[(i * RCT + c) * slots];
-              m = chunk < flush ? acc[i][c] : m + acc[i][c];
+              m = first ? acc[i][c] : m + acc[i][c];
               acc[i][c] = czero<T>();
             }
+        first = false;
+        next += flush;
       }
     }
     if (!BULK) {
@@ -651,7 +664,7 @@ cudaError_t restrict_op(cplx<T>* out, const cplx<T>* in, const cplx<T>* P, const
     count_launch();
     kernel<<<grid, groups * RTH, restrict_smem<T>(N, groups, pb).total, st>>>(
         out, in, Ps, scale, gf, fine, n, N, nrhs, in_rstride, pstride, out_rstride, out_site_stride, kch,
-        run < kch ? run : kch, err);
+        run < kch ? run : kch, restrict_flush(gf.vA, n / 2, N, kch), err);
     return cudaPeekAtLastError();
   };
   if constexpr (sizeof(T) == 4) {
