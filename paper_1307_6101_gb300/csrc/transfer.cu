@@ -68,7 +68,7 @@ inline int restrict_chunk(int run, int ps, bool bulk) {
 // Chunks that run into one chain of a lane's FMAs: a chain of k roundings errs like sqrt(k / 2) of them, so what
 // counts is the FMAs of a chain plus the chains of a lane.  One chunk more than makes that least, since every end of a chain
 // costs time (16^3x32, 20 test vectors, restriction and interpolation of one column 146 us with one chunk and 142 with
-// two, of twelve 524 and 514), as long as it stays below a lane per site (up to 256 lanes), a butterfly over them and the
+// two, of twelve 524 and 513), as long as it stays below a lane per site (up to 256 lanes), a butterfly over them and the
 // warps in a chain.
 inline int restrict_flush(int vA, int h, int N, int kch) {
   const int nsub = 32 / ((N + 3) / 4), nch = (vA * h + kch - 1) / kch;
@@ -237,33 +237,55 @@ __global__ void __launch_bounds__(RNG * RTH, sizeof(T) == 4 ? 2 : 1) k_restrict(
   }
   cplx<T>* po = out + (size_t)r0 * out_rstride + (size_t)gf.csite[agg] * out_site_stride + (size_t)s * N;
   const T sc = pscale ? T(pscale[agg * 2 + s]) : T(1);
-  for (int e = tid; e < N * C; e += blockDim.x) {
-    const int c = e / N, i = e - c * N;
-    const cplx<T>* r = red + ((size_t)(c / RCT) * 4 * RCT + i / TI * RCT + c % RCT) * slots + i % TI;
-    cplx<T> t[4] = {czero<T>(), czero<T>(), czero<T>(), czero<T>()};   // the parts in four chains, FP32 with their
-    cplx<T> lo[4] = {czero<T>(), czero<T>(), czero<T>(), czero<T>()};  // rounding errors
-    for (int q = 0; q < (RTH / 32) * nsub; q += 4)
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const cplx<T> p = r[(q + u) * TI];
-        if constexpr (sizeof(T) == 4) {
-          two_sum_acc(t[u].re, lo[u].re, p.re);
-          two_sum_acc(t[u].im, lo[u].im, p.im);
-        } else {
-          t[u] = t[u] + p;
-        }
-      }
+  // The parts in four chains, FP32 with the rounding errors, then the chains in order: by one thread, or, where there
+  // are threads enough, by a lane per chain in the same order (the same bits).
+  auto add = [&](cplx<T>& hi, cplx<T>& lo, const cplx<T>& h) {
     if constexpr (sizeof(T) == 4) {
-#pragma unroll
-      for (int u = 1; u < 4; ++u) {
-        two_sum_acc(t[0].re, lo[0].re, t[u].re);
-        two_sum_acc(t[0].im, lo[0].im, t[u].im);
-        lo[0] = lo[0] + lo[u];
-      }
-      po[(size_t)c * out_rstride + i] = sc * cmk(two_sum(t[0].re, lo[0].re), two_sum(t[0].im, lo[0].im));
+      two_sum_acc(hi.re, lo.re, h.re);
+      two_sum_acc(hi.im, lo.im, h.im);
     } else {
-      po[(size_t)c * out_rstride + i] = sc * ((t[0] + t[1]) + (t[2] + t[3]));
+      hi = hi + h;
     }
+  };
+  auto part = [&](int e) {
+    const int c = e / N, i = e - c * N;
+    return red + ((size_t)(c / RCT) * 4 * RCT + i / TI * RCT + c % RCT) * slots + i % TI;
+  };
+  auto store = [&](int e, cplx<T> hi, const cplx<T>& lo) {
+    if constexpr (sizeof(T) == 4) hi = cmk(two_sum(hi.re, lo.re), two_sum(hi.im, lo.im));
+    po[(size_t)(e / N) * out_rstride + e % N] = sc * hi;
+  };
+  const int parts = (RTH / 32) * nsub;
+  if (4 * N * C <= (int)blockDim.x) {
+    if (tid >= ((4 * N * C + 31) & ~31)) return;   // whole warps
+    const int e = tid >> 2;
+    cplx<T> hi = czero<T>(), lo = czero<T>();
+    if (e < N * C)
+      for (int q = tid & 3; q < parts; q += 4) add(hi, lo, part(e)[q * TI]);
+    const cplx<T> h1 = hi, l1 = lo;
+#pragma unroll
+    for (int u = 1; u < 4; ++u) {
+      const int from = (lane & ~3) | u;
+      const cplx<T> h = cmk(__shfl_sync(0xffffffffu, h1.re, from), __shfl_sync(0xffffffffu, h1.im, from));
+      add(hi, lo, h);
+      if constexpr (sizeof(T) == 4)
+        lo = lo + cmk(__shfl_sync(0xffffffffu, l1.re, from), __shfl_sync(0xffffffffu, l1.im, from));
+    }
+    if (e < N * C && (tid & 3) == 0) store(e, hi, lo);
+    return;
+  }
+  for (int e = tid; e < N * C; e += blockDim.x) {
+    const cplx<T>* r = part(e);
+    cplx<T> hi[4] = {czero<T>(), czero<T>(), czero<T>(), czero<T>()}, lo[4] = {czero<T>(), czero<T>(), czero<T>(), czero<T>()};
+    for (int q = 0; q < parts; q += 4)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) add(hi[u], lo[u], r[(q + u) * TI]);
+#pragma unroll
+    for (int u = 1; u < 4; ++u) {
+      add(hi[0], lo[0], hi[u]);
+      lo[0] = lo[0] + lo[u];
+    }
+    store(e, hi[0], lo[0]);
   }
 }
 
