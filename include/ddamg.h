@@ -70,7 +70,8 @@ typedef struct ddamg_params {
   int precision;                       /* preconditioner: 0 FP64; 1 FP32; 2 FP32 arithmetic
                                           on FP16 storage (links, clover term, P, coarse
                                           blocks; per-site / per-aggregate scales)        */
-  int max_rhs;                         /* right-hand sides per batch                     */
+  int max_rhs;                         /* right-hand sides per batch; kernels are chosen for
+                                          this many, also where fewer are passed          */
   uint64_t seed;                       /* seed of the random start vectors of Alg. 3 when
                                           ddamg_setup draws them (tv_random = NULL)       */
   int sap_schur;                       /* 1: the FP32 preconditioner's fine-level SAP solves
