@@ -44,12 +44,13 @@ def test_split_operator_and_sap_against_oracle(dims, block):
         assert rel(z1[r], o.levels[0].sap.smooth(f[r], z[r], 1)) <= 1e-12
 
 
-@pytest.mark.parametrize("max_rhs", [1, 8, 12])
-def test_sap_kernel_of_the_handles_batch(max_rhs):
+@pytest.mark.parametrize("dims,block,max_rhs", [((16, 8, 8, 8), (4, 4, 4, 4), 1), ((16, 8, 8, 8), (4, 4, 4, 4), 8),
+                                                ((16, 8, 8, 8), (4, 4, 4, 4), 12), ((6, 6, 6, 4), (3, 3, 3, 2), 64)])
+def test_sap_kernel_of_the_handles_batch(dims, block, max_rhs):
     """16 blocks of 4^4 sites per colour: six threads per site for batches of one and twelve, one thread per site for eight;
-    a column has the same bits alone and in a batch of any size."""
+    8 blocks of 54 sites, four to a CTA: one thread per site for a batch of 64.  A column has the same bits alone and in a
+    batch of any size."""
     import paper_1307_6101_gb300 as dd
-    dims, block = (16, 8, 8, 8), (4, 4, 4, 4)
     c = Case(dims=dims, levels=2, agg=(block,), n_tv=(1,), sap=(block,), max_rhs=max_rhs)
     h, o = c.gpu(0), c.oracle()
     f = np.ascontiguousarray(synth.random_spinors(9, dims, 5))

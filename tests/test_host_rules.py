@@ -156,6 +156,7 @@ def test_fp64_sap_kernel_per_batch(tmp_path):
   CHECK(fine_sap_takes_split(b3, 128, 4) && fine_sap_takes_split(b3, 128, 12) && !fine_sap_takes_split(b442, 512, 8));
   CHECK(fine_sap_takes_split(geom(4, 4, 4, 3), 192, 1) && !fine_sap_takes_split(geom(4, 4, 4, 3), 192, 8));
   CHECK(!fine_sap_takes_split(geom(3, 3, 3, 2), 192, 12) && fine_sap_takes_split(geom(3, 3, 3, 2), 192, 4));
+  CHECK(fine_sap_takes_split(geom(3, 3, 3, 2), 8, 1) && !fine_sap_takes_split(geom(3, 3, 3, 2), 8, 64));
   for (int batch : {1, 2, 8, 12}) CHECK(fine_sap_takes_split(geom(2, 2, 2, 2), 2048, batch));
   CHECK(fine_sap_takes_split(geom(8, 8, 4, 4), 512, 12));
 """)
